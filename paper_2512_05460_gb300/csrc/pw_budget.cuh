@@ -105,18 +105,19 @@ __host__ __device__ __forceinline__ uint64_t q_slots(const QPlan& P) {
   return P.Bmax ? (uint64_t)P.G * P.Bmax : (uint64_t)P.K;
 }
 
-// ADAPTIVE stopping rule: from the first stage's G*B1 values of Q_R (q), the
+// ADAPTIVE stopping rule: from the first stage's G*B1 values of Q_R, the
 // smallest B with z standard errors of the median of means, sqrt(pi/2) sd(Q) /
 // sqrt(G B), inside eps theta, theta = max(mean Q, theta_0); clamped to
-// [B1, Bmax].  Sums in index order, operation by operation as the oracle.
-__host__ __device__ inline uint32_t adaptive_B(const double* q, uint32_t B1, uint32_t Bmax, uint32_t G, double eps,
-                                               double z, int32_t deg_s, int32_t deg_t) {
+// [B1, Bmax].  mean and ss (the squared deviations' sum) are accumulated by the
+// caller in index order; operation by operation as the oracle.
+__device__ __forceinline__ double adaptive_square(double q, double mean) {
+  const double d = __dsub_rn(q, mean);
+  return __dmul_rn(d, d);
+}
+
+__device__ inline uint32_t adaptive_B(double mean, double ss, uint32_t B1, uint32_t Bmax, uint32_t G, double eps,
+                                      double z, int32_t deg_s, int32_t deg_t) {
   const uint64_t K1 = (uint64_t)G * B1;
-  double sum = 0.0;
-  for (uint64_t k = 0; k < K1; ++k) sum = sum + q[k];
-  const double mean = sum / (double)K1;
-  double ss = 0.0;
-  for (uint64_t k = 0; k < K1; ++k) ss = ss + (q[k] - mean) * (q[k] - mean);
   const double s2 = K1 > 1 ? ss / (double)(K1 - 1) : 0.0;
   const double inv = 1.0 / (double)deg_s + 1.0 / (double)deg_t;
   const double theta0 = (1.0 / 8.0) * (1.0 - eps / 2.0) * inv * inv;

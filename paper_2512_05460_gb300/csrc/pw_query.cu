@@ -30,25 +30,34 @@ struct ProbeAcc {
 
 // ---------------------------------------------------------------------------
 // Budget of every query (Algorithm 1 line 1).  PILOT queries get their pilot
-// plan here and their R in pilot_budget_kernel.
+// plan here and their R in pilot_budget_scan_kernel.
 // ---------------------------------------------------------------------------
-__global__ void budget_init_kernel(int64_t nq, const int64_t* __restrict__ qs, const int64_t* __restrict__ qt,
-                                   const double* __restrict__ qeps, const int32_t* __restrict__ qL,
-                                   const uint64_t* __restrict__ qseed, BudgetArgs A, int64_t n,
-                                   const int4* __restrict__ node, QPlan* __restrict__ plans,
-                                   QPlan* __restrict__ pilot) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= nq) return;
-  const int64_t s = qs[q], t = qt[q];
-  const double eps = qeps[q];
-  const int32_t L = qL[q];
+struct QueryArrays {
+  const int64_t* s;
+  const int64_t* t;
+  const double* eps;
+  const int32_t* L;
+  const uint64_t* seed;
+};
+
+__device__ __forceinline__ void plan_one(int64_t q, const QueryArrays& Q, const BudgetArgs& A, int64_t n,
+                                         const int4* __restrict__ node, QPlan* plans, QPlan* pilot) {
+  const int64_t s = Q.s[q], t = Q.t[q];
+  const double eps = Q.eps[q];
+  const int32_t L = Q.L[q];
   const bool ok = !(s < 0 || s >= n || t < 0 || t >= n || !(eps > 0.0 && eps < 1.0) || L < 0);
-  const uint64_t seed = !ok ? 0 : (qseed ? qseed[q] : default_seed(A.global_seed, s, t, eps, L));
+  const uint64_t seed = !ok ? 0 : (Q.seed ? Q.seed[q] : default_seed(A.global_seed, s, t, eps, L));
   const int32_t ds = ok ? node[s].z : 1, dt = ok ? node[t].z : 1;
   QPlan P, PP;
   plan_query(s, t, eps, L, seed, n, ds, dt, A, &P, &PP);
   plans[q] = P;
   if (pilot) pilot[q] = PP;
+}
+
+__global__ void budget_init_kernel(int64_t nq, QueryArrays Q, BudgetArgs A, int64_t n, const int4* __restrict__ node,
+                                   QPlan* __restrict__ plans, QPlan* __restrict__ pilot) {
+  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (q < nq) plan_one(q, Q, A, n, node, plans, pilot);
 }
 
 // Q slots of the batch: the sum of K, or of G Bmax for ADAPTIVE queries
@@ -66,23 +75,6 @@ __global__ void sum_k_kernel(const QPlan* __restrict__ plans, int64_t nq, unsign
   if (threadIdx.x == 0) *out = sh[0];
 }
 
-// PILOT: R >= 4 sigma^2 / theta (Lemma 3.7) from the pilot probes' (S1, S2),
-// summed over probes in the oracle's order.
-__global__ void pilot_budget_kernel(int64_t nq, QPlan* __restrict__ plans, const QPlan* __restrict__ pilot,
-                                    const double* __restrict__ pilot_s, BudgetArgs A, const int4* __restrict__ node) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= nq) return;
-  const QPlan PP = pilot[q];
-  if (PP.K == 0) return;
-  QPlan& P = plans[q];
-  double sum_var = 0.0, sum_q = 0.0;
-  for (uint32_t k = 0; k < PP.K; ++k) {
-    const double* sk = pilot_s + 2 * (PP.probe_begin + k);
-    pilot_accumulate(sum_var, sum_q, sk[0], sk[1], PP.R);
-  }
-  pilot_finish(P, sum_var, sum_q, PP.K, node[P.s].z, node[P.t].z, A);
-}
-
 // Walk kernel of each query and the offsets of its work.  A query's probes run
 // in the probe-table kernel when building z^(k) once is cheaper than
 // evaluating it at each of the probe's 2 R (L + 1) visits, by the graph's cost
@@ -96,72 +88,102 @@ struct ModeArgs {
   double visit_gain;  // saving per visit when entries come from the table
 };
 
-// keep_q (the second stage of ADAPTIVE queries): the Q slots stay where the
-// first stage put them.
-__global__ void scan_kernel(QPlan* __restrict__ plans, int64_t nq, unsigned long long* __restrict__ prefix,
-                            Totals* __restrict__ totals, ModeArgs M, int keep_q) {
-  __shared__ unsigned long long sh[4][1024];
-  __shared__ unsigned long long sh_steps[1024], sh_visits[1024], sh_work[1024];
-  const int tid = threadIdx.x, nt = blockDim.x;
+struct ScanArgs {
+  QPlan* plans;
+  unsigned long long* prefix;
+  Totals* totals;
+  ModeArgs M;
+  int32_t keep_q;      // the second stage of ADAPTIVE queries: the Q slots stay where the first stage put them
+  int32_t g0, g1;      // g1 > 0: a sharded query keeps only median-of-means blocks [g0, g1)
+};
+
+// Walk mode and offsets of every query, by one block of at most 1024 threads.
+// A thread owns a contiguous range of queries; its partial sums are scanned by
+// warp shuffles, then over the warps.  (One thread adding 1024 partials from
+// shared memory took 37 us, whatever the batch; this takes 4 to 6.)
+__device__ void scan_plans(const ScanArgs& S, int64_t nq) {
+  constexpr int kScan = 4, kSums = 3, kAll = kScan + kSums;
+  __shared__ unsigned long long sh[kAll][32];
+  QPlan* plans = S.plans;
+  unsigned long long* prefix = S.prefix;
+  const ModeArgs& M = S.M;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
   const int64_t per = (nq + nt - 1) / nt;
   const int64_t b0 = per * tid, b = b0 < nq ? b0 : nq, e = b + per < nq ? b + per : nq;
-  unsigned long long a[4] = {0, 0, 0, 0}, steps = 0, visits = 0, work = 0;
+  // scanned: per-visit tiles, per-visit probes (accumulators), table probes, Q
+  // slots; summed: steps, visits, probes
+  unsigned long long a[kAll] = {0, 0, 0, 0, 0, 0, 0};
   for (int64_t q = b; q < e; ++q) {
     QPlan& P = plans[q];
+    // a sharded query (a batch of one): probe indices keep their global values
+    // (k_begin), so the walks are those of the whole query
+    if (S.g1 > 0 && P.status == PW_OK && P.K != 0) {
+      P.k_begin = (uint32_t)S.g0 * P.B;
+      P.K = (uint32_t)(S.g1 - S.g0) * P.B;
+      P.G = (uint32_t)(S.g1 - S.g0);
+    }
     const double v = 2.0 * (double)P.R * (double)(P.L + 1);
     uint32_t mode = M.forced != 0 ? (uint32_t)M.forced
                                   : (M.probe_cost < v * M.visit_gain ? 2u : 1u);
     if (!M.table_ok) mode = 1u;
     P.mode = mode;
     const unsigned long long K = P.K;
-    a[0] += mode == 1u ? K * P.chunks : 0ull;  // per-visit tiles
-    a[1] += mode == 1u ? K : 0ull;             // per-visit probes (accumulators)
-    a[2] += mode == 2u ? K : 0ull;             // table probes
-    a[3] += q_slots(P);                        // Q slots
-    work += K;
-    steps += K * P.R * (unsigned long long)(P.L > 0 ? P.L : 0);
-    visits += 2ull * K * P.R * (unsigned long long)(P.L + 1);
+    a[0] += mode == 1u ? K * P.chunks : 0ull;
+    a[1] += mode == 1u ? K : 0ull;
+    a[2] += mode == 2u ? K : 0ull;
+    a[3] += q_slots(P);
+    a[4] += K * P.R * (unsigned long long)(P.L > 0 ? P.L : 0);
+    a[5] += 2ull * K * P.R * (unsigned long long)(P.L + 1);
+    a[6] += K;
   }
+  unsigned long long incl[kAll];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) sh[j][tid] = a[j];
-  sh_steps[tid] = steps;
-  sh_visits[tid] = visits;
-  sh_work[tid] = work;
-  __syncthreads();
-  if (tid == 0) {
-    unsigned long long run[4] = {0, 0, 0, 0}, st = 0, vi = 0, wk = 0;
-    for (int i = 0; i < nt; ++i) {
+  for (int j = 0; j < kAll; ++j) {
+    unsigned long long x = a[j];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const unsigned long long x = sh[j][i];
-        sh[j][i] = run[j];
-        run[j] += x;
-      }
-      st += sh_steps[i];
-      vi += sh_visits[i];
-      wk += sh_work[i];
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
     }
-    totals->tiles = run[0];
-    totals->visit_probes = run[1];
-    totals->table_probes = run[2];
-    totals->probes = wk;
-    totals->steps = st;
-    totals->visits = vi;
-    prefix[nq] = run[0];
-    prefix[(nq + 1) + nq] = run[2];
-    if (!keep_q) prefix[2 * (nq + 1) + nq] = run[3];
+    incl[j] = x;
+    if (lane == 31) sh[j][warp] = x;
   }
   __syncthreads();
-  unsigned long long o[4];
+  if (warp == 0) {
+    const int nw = (nt + 31) >> 5;
 #pragma unroll
-  for (int j = 0; j < 4; ++j) o[j] = sh[j][tid];
+    for (int j = 0; j < kAll; ++j) {
+      const unsigned long long own = lane < nw ? sh[j][lane] : 0ull;
+      unsigned long long x = own;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      sh[j][lane] = x - own;  // before this warp
+      if (lane == 31) {
+        Totals* T = S.totals;
+        if (j == 0) T->tiles = prefix[nq] = x;
+        if (j == 1) T->visit_probes = x;
+        if (j == 2) T->table_probes = prefix[(nq + 1) + nq] = x;
+        if (j == 3 && !S.keep_q) prefix[2 * (nq + 1) + nq] = x;
+        if (j == 4) T->steps = x;
+        if (j == 5) T->visits = x;
+        if (j == 6) T->probes = x;
+      }
+    }
+  }
+  __syncthreads();
+  unsigned long long o[kScan];
+#pragma unroll
+  for (int j = 0; j < kScan; ++j) o[j] = sh[j][warp] + incl[j] - a[j];
   for (int64_t q = b; q < e; ++q) {
     QPlan& P = plans[q];
     const unsigned long long K = P.K;
     P.tile_begin = o[0];
     P.acc_begin = o[1];
     P.table_begin = o[2];
-    if (!keep_q) {
+    if (!S.keep_q) {
       P.probe_begin = o[3];
       P.q_begin = o[3];
       prefix[2 * (nq + 1) + q] = o[3];
@@ -175,21 +197,111 @@ __global__ void scan_kernel(QPlan* __restrict__ plans, int64_t nq, unsigned long
   }
 }
 
+__global__ void scan_kernel(ScanArgs S, int64_t nq) { scan_plans(S, nq); }
+
+// A small batch's plans and their offsets in one launch of one block.  Up to
+// kFusedPlans queries: the FP64 divisions of more would queue up on one SM.
+constexpr int64_t kFusedPlans = 256;
+__global__ void plan_scan_kernel(int64_t nq, QueryArrays Q, BudgetArgs A, int64_t n, const int4* __restrict__ node,
+                                 QPlan* plans, QPlan* pilot, ScanArgs S) {
+  for (int64_t q = threadIdx.x; q < nq; q += blockDim.x) plan_one(q, Q, A, n, node, plans, pilot);
+  __syncthreads();
+  scan_plans(S, nq);
+}
+
+// True in every thread of the last block of the grid to get here; the other
+// blocks' global writes before the call are then visible to it.
+__device__ bool last_block(unsigned long long* arrived) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(arrived, 1ull) + 1ull == gridDim.x;
+  __syncthreads();
+  if (last) __threadfence();
+  return last;
+}
+
+// PILOT: R >= 4 sigma^2 / theta (Lemma 3.7) from the pilot probes' (S1, S2), a
+// warp per query; then the last block scans all plans.  The terms (three FP64
+// divisions each, at 2 lanes per SM and clock) are computed by all lanes; they
+// are added in the oracle's order, probe after probe, the variances in lane 0
+// and the Q in lane 1.  (One thread per query took 72 us for any batch.)
+constexpr int kPilotThreads = 256;
+__global__ void __launch_bounds__(kPilotThreads)
+pilot_budget_scan_kernel(int64_t nq, QPlan* plans, const QPlan* __restrict__ pilot, const double* __restrict__ pilot_s,
+                         BudgetArgs A, const int4* __restrict__ node, ScanArgs S, unsigned long long* arrived) {
+  constexpr int kWarps = kPilotThreads / 32;
+  __shared__ double terms[kWarps][2][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t q = (int64_t)blockIdx.x * kWarps + warp;
+  if (q < nq && pilot[q].K != 0) {
+    const uint32_t K = pilot[q].K, R = pilot[q].R;
+    const double* ps = pilot_s + 2 * pilot[q].probe_begin;
+    double sum = 0.0;  // lane 0: variances, lane 1: Q
+    for (uint32_t k0 = 0; k0 < K; k0 += 32) {
+      const uint32_t k = k0 + (uint32_t)lane, m = K - k0 < 32u ? K - k0 : 32u;
+      double var = 0.0, Q = 0.0;
+      if (k < K) pilot_accumulate(var, Q, ps[2 * k], ps[2 * k + 1], R);  // 0 + term is the term
+      terms[warp][0][lane] = var;
+      terms[warp][1][lane] = Q;
+      __syncwarp();
+      if (lane < 2)
+        for (uint32_t i = 0; i < m; ++i) sum = __dadd_rn(sum, terms[warp][lane][i]);
+      __syncwarp();
+    }
+    const double sum_q = __shfl_sync(0xffffffffu, sum, 1);
+    if (lane == 0) {
+      QPlan P = plans[q];
+      pilot_finish(P, sum, sum_q, K, node[P.s].z, node[P.t].z, A);
+      plans[q] = P;
+    }
+  }
+  if (last_block(arrived)) scan_plans(S, nq);
+}
+
 // ADAPTIVE, between the stages: each query's B* from its first G B1 values of
 // Q_R; the second stage runs probes G B1 .. G B* - 1 into the Q slots after
-// the first stage's, and the median reads G blocks of B* from q_begin.
-__global__ void adapt_kernel(int64_t nq, QPlan* __restrict__ plans, const double* __restrict__ qbuf, BudgetArgs A,
-                             const int4* __restrict__ node) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= nq) return;
-  QPlan& P = plans[q];
-  if (P.status != PW_OK || P.K == 0 || P.Bmax == 0) return;
-  const uint32_t B1 = P.B, K1 = P.K;
-  const uint32_t Bs = adaptive_B(qbuf + P.q_begin, B1, P.Bmax, P.G, P.eps, A.z, node[P.s].z, node[P.t].z);
-  P.B = Bs;
-  P.k_begin = K1;
-  P.K = P.G * (Bs - B1);
-  P.probe_begin = P.q_begin + K1;
+// the first stage's, and the median reads G blocks of B* from q_begin.  A warp
+// per query: lanes load (and square) 32 values, lane 0 adds them in index
+// order; then the last block scans the plans.
+__global__ void __launch_bounds__(kPilotThreads)
+adapt_scan_kernel(int64_t nq, QPlan* plans, const double* __restrict__ qbuf, BudgetArgs A,
+                  const int4* __restrict__ node, ScanArgs S, unsigned long long* arrived) {
+  constexpr int kWarps = kPilotThreads / 32;
+  __shared__ double terms[kWarps][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t q = (int64_t)blockIdx.x * kWarps + warp;
+  if (q < nq && plans[q].status == PW_OK && plans[q].K != 0 && plans[q].Bmax != 0) {
+    const uint32_t B1 = plans[q].B, G = plans[q].G;
+    const double* x = qbuf + plans[q].q_begin;
+    const uint64_t K1 = (uint64_t)G * B1;
+    double mean = 0.0, sum = 0.0;
+    for (int pass = 0; pass < 2; ++pass) {
+      sum = 0.0;
+      for (uint64_t k0 = 0; k0 < K1; k0 += 32) {
+        const uint64_t k = k0 + (uint64_t)lane;
+        const uint32_t m = K1 - k0 < 32u ? (uint32_t)(K1 - k0) : 32u;
+        double v = k < K1 ? x[k] : 0.0;
+        if (pass == 1) v = adaptive_square(v, mean);
+        terms[warp][lane] = v;
+        __syncwarp();
+        if (lane == 0)
+          for (uint32_t i = 0; i < m; ++i) sum = __dadd_rn(sum, terms[warp][i]);
+        __syncwarp();
+      }
+      if (pass == 0) mean = __shfl_sync(0xffffffffu, __ddiv_rn(sum, (double)K1), 0);
+    }
+    if (lane == 0) {
+      QPlan P = plans[q];
+      const uint32_t Bs = adaptive_B(mean, sum, B1, P.Bmax, G, P.eps, A.z, node[P.s].z, node[P.t].z);
+      P.B = Bs;
+      P.k_begin = P.K;
+      P.probe_begin = P.q_begin + P.K;
+      P.K = G * (Bs - B1);
+      plans[q] = P;
+    }
+  }
+  if (last_block(arrived)) scan_plans(S, nq);
 }
 
 // Accumulators of the per-visit probes start at zero.
@@ -258,6 +370,7 @@ __global__ void __launch_bounds__(kWalkThreads, MINB) walk_kernel(WalkArgs A) {
   const auto gr = GraphOf<SPLIT>::get(A);
   const uint32_t lane = threadIdx.x & 31u;
   const unsigned long long total = A.totals->tiles;
+  if (total == 0ull) return;
   for (;;) {
     unsigned long long tile = 0;
     if (lane == 0) tile = atomicAdd(A.counter, 1ull);
@@ -324,6 +437,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 5 : (THREADS == 512 
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t n = A.n;
   const unsigned long long total = A.totals->table_probes;
+  if (total == 0ull) return;
   for (;;) {
     if (threadIdx.x == 0) {
       sh_probe = atomicAdd(A.counter, 1ull);
@@ -399,10 +513,28 @@ __global__ void debug_exact_sum_kernel(const float* __restrict__ u, int64_t n, d
   }
 }
 
+// Mean of B contiguous values, added in index order; eight loads in flight.
+__device__ __forceinline__ double block_mean(const double* __restrict__ x, uint32_t B) {
+  double sum = 0.0;
+  uint32_t k = 0;
+  for (; k + 8 <= B; k += 8) {
+    double v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = x[k + i];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) sum = __dadd_rn(sum, v[i]);
+  }
+  for (; k < B; ++k) sum = __dadd_rn(sum, x[k]);
+  return __ddiv_rn(sum, (double)B);
+}
+
 // Median of the G block means of B contiguous probes (Eq. final-estimator).
+// The middle values are found by rank (ties in index order), every thread
+// comparing its means with all: one thread's insertion sort took 20 us at G = 37.
 __global__ void mom_kernel(const QPlan* __restrict__ plans, const double* __restrict__ qbuf,
                            double* __restrict__ beta, int32_t* __restrict__ status) {
   __shared__ double means[4096];
+  __shared__ double mid[2];
   const int64_t q = blockIdx.x;
   const QPlan& P = plans[q];
   if (P.status != PW_OK || P.K == 0) {
@@ -412,51 +544,31 @@ __global__ void mom_kernel(const QPlan* __restrict__ plans, const double* __rest
     }
     return;
   }
-  for (uint32_t g = threadIdx.x; g < P.G; g += blockDim.x) {
-    const double* x = qbuf + P.q_begin + (uint64_t)g * P.B;
-    double sum = 0.0;
-    for (uint32_t k = 0; k < P.B; ++k) sum = __dadd_rn(sum, x[k]);
-    means[g] = __ddiv_rn(sum, (double)P.B);
+  const uint32_t G = P.G;
+  for (uint32_t g = threadIdx.x; g < G; g += blockDim.x)
+    means[g] = block_mean(qbuf + P.q_begin + (uint64_t)g * P.B, P.B);
+  __syncthreads();
+  const uint32_t hi = G / 2, lo = (G & 1u) ? hi : hi - 1;
+  for (uint32_t g = threadIdx.x; g < G; g += blockDim.x) {
+    const double v = means[g];
+    uint32_t rank = 0;
+    for (uint32_t j = 0; j < G; ++j) rank += (means[j] < v || (means[j] == v && j < g)) ? 1u : 0u;
+    if (rank == lo) mid[0] = v;
+    if (rank == hi) mid[1] = v;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    const uint32_t G = P.G;
-    for (uint32_t i = 1; i < G; ++i) {  // insertion sort
-      const double v = means[i];
-      uint32_t j = i;
-      while (j > 0 && means[j - 1] > v) {
-        means[j] = means[j - 1];
-        --j;
-      }
-      means[j] = v;
-    }
-    const double med = (G & 1u) ? means[G / 2] : __ddiv_rn(__dadd_rn(means[G / 2 - 1], means[G / 2]), 2.0);
-    beta[q] = med;
+    beta[q] = (G & 1u) ? mid[0] : __ddiv_rn(__dadd_rn(mid[0], mid[1]), 2.0);
     status[q] = PW_OK;
   }
-}
-
-// Sharded query: keep only median-of-means blocks [g0, g1) of query 0; probe
-// indices keep their global values (k_begin), so the walks are those of the
-// whole query.
-__global__ void restrict_blocks_kernel(QPlan* plans, uint32_t g0, uint32_t g1) {
-  QPlan& P = plans[0];
-  if (P.status != PW_OK || P.K == 0) return;
-  P.k_begin = g0 * P.B;
-  P.K = (g1 - g0) * P.B;
-  P.G = g1 - g0;
 }
 
 // Block means of a sharded query (Eq. final-estimator before the median).
 __global__ void block_means_kernel(const QPlan* __restrict__ plans, const double* __restrict__ qbuf,
                                    double* __restrict__ means, int32_t* __restrict__ status) {
   const QPlan& P = plans[0];
-  for (uint32_t g = threadIdx.x; g < P.G; g += blockDim.x) {
-    const double* x = qbuf + P.q_begin + (uint64_t)g * P.B;
-    double sum = 0.0;
-    for (uint32_t k = 0; k < P.B; ++k) sum = __dadd_rn(sum, x[k]);
-    means[g] = __ddiv_rn(sum, (double)P.B);
-  }
+  for (uint32_t g = threadIdx.x; g < P.G; g += blockDim.x)
+    means[g] = block_mean(qbuf + P.q_begin + (uint64_t)g * P.B, P.B);
   if (threadIdx.x == 0) status[0] = P.status;
 }
 
@@ -563,7 +675,10 @@ struct BatchBuffers {
   QPlan* pplans;
   unsigned long long* prefix;    // 6 (nq + 1): main tiles, table probes, probes; then the pilot's three
   Totals* totals;                // [0] main, [1] pilot
-  unsigned long long* counters;  // [0] main per-visit tiles, [1] pilot tiles, [2] table probes
+  // cleared at the start of a batch: [0] main per-visit tiles, [1] pilot tiles,
+  // [2] table probes, [3] blocks done with the pilot budget, [4] and [6] as [0]
+  // and [2] for ADAPTIVE's second stage, [5] blocks done with the stopping rule
+  unsigned long long* counters;
   double* pilot_s;               // (S1, S2) per pilot probe
   double* q;                     // Q_R per probe
   ProbeAcc* acc;                 // per-visit probe accumulators
@@ -587,29 +702,15 @@ static BatchSizes batch_sizes(size_t nq, size_t total_K, const BudgetArgs& ba) {
   return z;
 }
 
-// First stage: counters cleared, plans of every query (and their pilots).
-static pw_status enqueue_budget(pw_graph* g, int64_t count, const int64_t* d_s, const int64_t* d_t, const double* d_eps,
-                                const int32_t* d_L, const uint64_t* d_seeds, const BudgetArgs& ba,
-                                const BatchBuffers& B, cudaStream_t stream) {
-  PW_CUDA_TRY(cudaMemsetAsync(B.counters, 0, 64, stream));
-  const int qthreads = 128;
-  const int qblocks = (int)((count + qthreads - 1) / qthreads);
-  budget_init_kernel<<<qblocks, qthreads, 0, stream>>>(count, d_s, d_t, d_eps, d_L, d_seeds, ba, g->n, g->d_node,
-                                                       B.plans, has_pilot(ba) ? B.pplans : nullptr);
-  count_launch();
-  PW_CUDA_TRY(cudaGetLastError());
-  return PW_OK;
-}
-
-// The rest of the pipeline: pilot, walk kernels, median.  No host
+// The whole pipeline: plans, pilot, walk kernels, median.  No host
 // synchronisation: every size it needs was fixed by batch_sizes.
-static pw_status enqueue_walks(pw_graph* g, int64_t count, const pw_params* params, const BudgetArgs& ba,
-                               const BatchBuffers& B, double* d_beta, int32_t* d_status, cudaStream_t stream,
-                               DebugOut* dbg) {
+static pw_status enqueue_walks(pw_graph* g, int64_t count, const QueryArrays& Q, const pw_params* params,
+                               const BudgetArgs& ba, const BatchBuffers& B, double* d_beta, int32_t* d_status,
+                               cudaStream_t stream, DebugOut* dbg) {
+  if (params && (params->walk_mode < 0 || params->walk_mode > 2))
+    return set_error(PW_ERR_ARG, "walk_mode must be 0, 1 or 2");
   const size_t nq = (size_t)count;
   const bool pilot = has_pilot(ba);
-  const int qthreads = 128;
-  const int qblocks = (int)((count + qthreads - 1) / qthreads);
   unsigned long long* prefix = B.prefix;
   unsigned long long* pprefix = B.prefix + 3 * (nq + 1);
   WalkArgs wa;
@@ -620,10 +721,32 @@ static pw_status enqueue_walks(pw_graph* g, int64_t count, const pw_params* para
   wa.nq = count;
   wa.n = (uint32_t)g->n;
   pw_status st;
-  if (pilot) {
-    ModeArgs pm{1, 0, 0.0, 0.0};
-    scan_kernel<<<1, 1024, 0, stream>>>(B.pplans, count, pprefix, B.totals + 1, pm, 0);
+  const bool sharded = dbg && dbg->g_begin >= 0;
+  const bool table_ok = table_bytes(g) <= kMaxTableBytes;
+  const int forced = params && params->walk_mode ? params->walk_mode : g->walk_policy;
+  const ModeArgs M{forced, table_ok ? 1 : 0, g->table_probe_cost, g->table_visit_gain};
+  ScanArgs main_scan{B.plans, prefix, B.totals, M, 0, sharded ? (int32_t)dbg->g_begin : 0,
+                     sharded ? (int32_t)dbg->g_end : 0};
+  const ScanArgs pilot_scan{B.pplans, pprefix, B.totals + 1, ModeArgs{1, 0, 0.0, 0.0}, 0, 0, 0};
+  // plans and the first offsets: the pilot's, or the main walks' where there is no pilot
+  const ScanArgs& first_scan = pilot ? pilot_scan : main_scan;
+  QPlan* pplans = pilot ? B.pplans : nullptr;
+  PW_CUDA_TRY(cudaMemsetAsync(B.counters, 0, 64, stream));
+  if (count <= kFusedPlans) {
+    const int threads = (int)((count + 31) / 32 * 32);
+    plan_scan_kernel<<<1, threads, 0, stream>>>(count, Q, ba, g->n, g->d_node, B.plans, pplans, first_scan);
     count_launch();
+  } else {
+    const int qthreads = 128;
+    budget_init_kernel<<<(int)((count + qthreads - 1) / qthreads), qthreads, 0, stream>>>(count, Q, ba, g->n, g->d_node,
+                                                                                          B.plans, pplans);
+    count_launch();
+    scan_kernel<<<1, 1024, 0, stream>>>(first_scan, count);
+    count_launch();
+  }
+  PW_CUDA_TRY(cudaGetLastError());
+  const int warp_blocks = (int)((count + kPilotThreads / 32 - 1) / (kPilotThreads / 32));
+  if (pilot) {
     wa.plans = B.pplans;
     wa.tile_prefix = pprefix;
     wa.totals = B.totals + 1;
@@ -636,24 +759,11 @@ static pw_status enqueue_walks(pw_graph* g, int64_t count, const pw_params* para
     if ((st = launch_walk(g, stream, wa, false, true)) != PW_OK) return st;
     prof_end(g, stream, ev, 1);
     if (g->prof.enabled) g->prof.pilot_transitions += 2ull * nq * (uint64_t)ba.K0 * (uint64_t)ba.R0;
-    pilot_budget_kernel<<<qblocks, qthreads, 0, stream>>>(count, B.plans, B.pplans, B.pilot_s, ba, g->d_node);
+    pilot_budget_scan_kernel<<<warp_blocks, kPilotThreads, 0, stream>>>(count, B.plans, B.pplans, B.pilot_s, ba,
+                                                                        g->d_node, main_scan, B.counters + 3);
     count_launch();
     PW_CUDA_TRY(cudaGetLastError());
   }
-  const bool sharded = dbg && dbg->g_begin >= 0;
-  if (sharded) {
-    restrict_blocks_kernel<<<1, 1, 0, stream>>>(B.plans, (uint32_t)dbg->g_begin, (uint32_t)dbg->g_end);
-    count_launch();
-    PW_CUDA_TRY(cudaGetLastError());
-  }
-  const bool table_ok = table_bytes(g) <= kMaxTableBytes;
-  const int forced = params && params->walk_mode ? params->walk_mode : g->walk_policy;
-  ModeArgs M{forced, table_ok ? 1 : 0, g->table_probe_cost, g->table_visit_gain};
-  if (params && (params->walk_mode < 0 || params->walk_mode > 2))
-    return set_error(PW_ERR_ARG, "walk_mode must be 0, 1 or 2");
-  scan_kernel<<<1, 1024, 0, stream>>>(B.plans, count, prefix, B.totals, M, 0);
-  count_launch();
-  PW_CUDA_TRY(cudaGetLastError());
   if (dbg && dbg->budget_only) return PW_OK;
   const bool debug = dbg && (dbg->visits || dbg->u);
   wa.plans = B.plans;
@@ -700,9 +810,11 @@ static pw_status enqueue_walks(pw_graph* g, int64_t count, const pw_params* para
   if (st == PW_OK && ba.mode == PW_BUDGET_ADAPTIVE) {
     // the stopping rule on the first stage's Q_R, then the second stage's
     // probes with their own offsets and totals (Q slots stay in place)
-    adapt_kernel<<<qblocks, qthreads, 0, stream>>>(count, B.plans, B.q, ba, g->d_node);
-    count_launch();
-    scan_kernel<<<1, 1024, 0, stream>>>(B.plans, count, prefix, B.totals + 2, M, 1);
+    ScanArgs second = main_scan;
+    second.totals = B.totals + 2;
+    second.keep_q = 1;
+    adapt_scan_kernel<<<warp_blocks, kPilotThreads, 0, stream>>>(count, B.plans, B.q, ba, g->d_node, second,
+                                                                 B.counters + 5);
     count_launch();
     const cudaError_t e = cudaGetLastError();
     st = e == cudaSuccess ? walk_stage(B.totals + 2, B.counters + 4) : cuda_error(e, "adaptive stage");
@@ -782,8 +894,8 @@ static pw_status device_total_K(pw_graph* g, int64_t count, const int64_t* d_s, 
   if ((st = ensure_buffer(ws.counters, 64)) != PW_OK) return st;
   const int qthreads = 128;
   const int qblocks = (int)((count + qthreads - 1) / qthreads);
-  budget_init_kernel<<<qblocks, qthreads, 0, stream>>>(count, d_s, d_t, d_eps, d_L, d_seeds, ba, g->n, g->d_node,
-                                                       (QPlan*)ws.plans.ptr, nullptr);
+  budget_init_kernel<<<qblocks, qthreads, 0, stream>>>(count, QueryArrays{d_s, d_t, d_eps, d_L, d_seeds}, ba, g->n,
+                                                       g->d_node, (QPlan*)ws.plans.ptr, nullptr);
   count_launch();
   unsigned long long* out = (unsigned long long*)ws.counters.ptr + 7;
   sum_k_kernel<<<1, 1024, 0, stream>>>((const QPlan*)ws.plans.ptr, count, out);
@@ -801,8 +913,8 @@ static pw_status enqueue_batch(pw_graph* g, int64_t count, const int64_t* d_s, c
                                const pw_params* params, const BudgetArgs& ba, const BatchBuffers& B, double* d_beta,
                                int32_t* d_status, cudaStream_t stream, DebugOut* dbg) {
   pw_status st;
-  if ((st = enqueue_budget(g, count, d_s, d_t, d_eps, d_L, d_seeds, ba, B, stream)) != PW_OK) return st;
-  if ((st = enqueue_walks(g, count, params, ba, B, d_beta, d_status, stream, dbg)) != PW_OK) return st;
+  const QueryArrays Q{d_s, d_t, d_eps, d_L, d_seeds};
+  if ((st = enqueue_walks(g, count, Q, params, ba, B, d_beta, d_status, stream, dbg)) != PW_OK) return st;
   PW_CUDA_TRY(cudaMemcpyAsync(g->ws.host_totals, B.totals, sizeof(Totals), cudaMemcpyDeviceToHost, stream));
   st = prof_totals(g, B.totals, stream);
   if (st == PW_OK && ba.mode == PW_BUDGET_ADAPTIVE && !(dbg && dbg->budget_only)) st = prof_totals(g, B.totals + 2, stream);
@@ -1601,8 +1713,8 @@ extern "C" pw_status pw_query_batch_noalloc(pw_graph* g, int64_t count, const in
   PW_CUDA_TRY(cudaStreamWaitEvent(stream, g->ws.last_use, 0));
   const int qthreads = 128;
   const int qblocks = (int)((count + qthreads - 1) / qthreads);
-  budget_init_kernel<<<qblocks, qthreads, 0, stream>>>(count, d_s, d_t, d_eps, d_L, d_seeds, ba, g->n, g->d_node,
-                                                       B.plans, nullptr);
+  const QueryArrays Q{d_s, d_t, d_eps, d_L, d_seeds};
+  budget_init_kernel<<<qblocks, qthreads, 0, stream>>>(count, Q, ba, g->n, g->d_node, B.plans, nullptr);
   count_launch();
   sum_k_kernel<<<1, 1024, 0, stream>>>(B.plans, count, B.counters + 7);
   count_launch();
@@ -1631,8 +1743,7 @@ extern "C" pw_status pw_query_batch_noalloc(pw_graph* g, int64_t count, const in
   B.pilot_s = (double*)(base + o_pilot);
   B.q = (double*)(base + o_q);
   B.acc = (ProbeAcc*)(base + o_acc);
-  if ((st = enqueue_budget(g, count, d_s, d_t, d_eps, d_L, d_seeds, ba, B, stream)) != PW_OK) return st;
-  if ((st = enqueue_walks(g, count, params, ba, B, d_beta_hat, d_status, stream, nullptr)) != PW_OK) return st;
+  if ((st = enqueue_walks(g, count, Q, params, ba, B, d_beta_hat, d_status, stream, nullptr)) != PW_OK) return st;
   PW_CUDA_TRY(cudaMemcpyAsync(g->ws.host_totals, B.totals, sizeof(Totals), cudaMemcpyDeviceToHost, stream));
   PW_CUDA_TRY(cudaEventRecord(g->ws.last_use, stream));
   return PW_OK;
