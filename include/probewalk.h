@@ -303,8 +303,8 @@ pw_status pw_server_collect(pw_server* srv, int64_t cap, uint64_t* tickets, doub
  * pw_server_tune runs the sample (host arrays as in pw_query_batch; seeds may
  * be NULL) through the server as a burst, once to warm up and once timed.
  * When the graph's probe table fits in shared memory it times each policy:
- * 0 the default model (n Feistel passes per table against 2.5 per visit), 1
- * the graph's model fitted by pw_autotune on the batch kernels (skipped when
+ * 0 the default model (2^b Feistel passes per table, 2^b >= n the
+ * permutation's domain, against 1.15 saved per visit), 1 the graph's model fitted by pw_autotune on the batch kernels (skipped when
  * the graph is untuned), 2 every query per-visit, 3 every query with the
  * table, and keeps the fastest.  When the table does not fit, every policy
  * runs the same per-visit jobs; it then times the server kernel at 2 and at 3
@@ -403,12 +403,10 @@ pw_status pw_profile(pw_graph* g, int32_t enable, int32_t reset, pw_profile_stat
  * the policy and window checks below run at the caller's own budget, where a
  * sample of 32 queries or more stands for the batch far better than 8),
  * params' G, and R = 1024 replicas, each run after one untimed
- * warm-up: the per-visit kernel in its two register variants (compiler's
- * choice, or capped for 3 blocks of 256 per SM), keeping the faster; the
- * per-probe shared-memory table with blocks of 256, 512 and 1024 threads,
- * keeping the fastest; and that table kernel again at R = 256 (the same
- * probes, a quarter of the visits).  The kept variants are stored in the
- * graph and used by every later batch.  From the main walk kernels'
+ * warm-up: the per-visit kernel; the per-probe shared-memory table with
+ * blocks of 256, 512 and 1024 threads, keeping the fastest; and that table
+ * kernel again at R = 256 (the same probes, a quarter of the visits).  The
+ * kept block size is stored in the graph and used by every later batch.  From the main walk kernels'
  * CUDA-event time of the kept runs it fits
  *   per-visit:  t = visits * visit_ns
  *   table:      t = probes * table_probe_ns + visits * table_visit_ns
@@ -440,7 +438,7 @@ typedef struct pw_tune_result {
   double sample_ms[3];     /* walk-kernel time of the kept runs (per-visit; table at R = 1024; table at R = 256) */
   int32_t table_available; /* 1 when the probe table fits in shared memory */
   int32_t sample_mode;     /* walk kernel the fitted model picks for the sample: 1 per-visit, 2 table */
-  int32_t visit_occupancy; /* per-visit kernel variant kept: 1 compiler-chosen registers, 3 capped for 3 blocks/SM */
+  int32_t visit_occupancy; /* resident blocks of 256 per SM of the per-visit kernel: 3 */
   int32_t table_threads;   /* table-kernel block size kept: 256, 512 or 1024 (0 when unavailable) */
   double policy_ms[3];     /* walk time of the sample at the caller's budget: per-query model, all per-visit, all table */
   int32_t policy;          /* the policy walk_mode 0 now follows: 0 per-query model, 1 all per-visit, 2 all table */

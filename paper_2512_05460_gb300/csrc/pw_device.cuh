@@ -114,12 +114,14 @@ __host__ __device__ __forceinline__ uint64_t level_seed(uint64_t seed, int32_t L
 // ---- Paired-Sign Probe -------------------------------------------------------
 
 struct Probe {
-  uint32_t n;        // nodes
-  uint32_t n_active; // n - r
-  uint32_t hi, lo;   // Feistel halves: domain 2^(hi + lo) >= n, hi = lo or lo + 1
-  uint32_t rounds;   // 8, or 12 when hi + lo <= 4
-  uint32_t a, b;     // hash parameters, a in [1, p-1], b in [0, p-1]
-  uint32_t key[12];  // round keys
+  uint32_t n;         // nodes
+  uint32_t n_active;  // n - r
+  uint32_t lo;        // Feistel halves hi and lo: domain 2^(hi + lo) >= n, hi = lo or lo + 1
+  uint32_t sh_hi, sh_lo;  // 32 - hi, 32 - lo
+  uint32_t rounds;    // 8, or 12 when hi + lo <= 4
+  uint32_t a, b;      // hash parameters, a in [1, p-1], b in [0, p-1]
+  uint32_t key[12];   // round keys 0 and 1, then key i XOR key i - 2 (feistel_pass)
+  uint32_t out1, out2;  // the last two round keys: out2 of the last round, out1 of the one before
 };
 
 // Domain bits: the smallest b >= 2 with 2^b >= n, with b = 3 raised to 4 (the
@@ -137,54 +139,86 @@ __host__ __device__ __forceinline__ void feistel_bits(uint32_t n, uint32_t& hi, 
 //   words of (k,0,0,tag): a = 1 + (w0|w1<<32) mod (p-1), b = (w2|w3<<32) mod p;
 //   words of (k,1,j,tag), j = 0,1,2: round keys 4j..4j+3;
 //   word 0 of (k,2,0,tag): parity coin r = 2 (bit 0) for even n, r = 1 for odd n.
-__host__ __device__ __forceinline__ Probe make_probe(uint32_t n, uint64_t seed, uint32_t k, uint32_t tag) {
+__host__ __device__ __forceinline__ Probe probe_from_words(uint32_t n, const Philox4& ab, const Philox4& k0,
+                                                           const Philox4& k1, const Philox4& k2, uint32_t coin) {
   Probe P;
   P.n = n;
-  feistel_bits(n, P.hi, P.lo);
-  P.rounds = (P.hi + P.lo <= 4) ? 12u : 8u;
-  const Philox4 ab = philox_seeded(seed, k, 0u, 0u, tag);
+  uint32_t hi;
+  feistel_bits(n, hi, P.lo);
+  P.sh_hi = 32u - hi;
+  P.sh_lo = 32u - P.lo;
+  P.rounds = (hi + P.lo <= 4) ? 12u : 8u;
   const uint64_t wa = (uint64_t)ab.x | ((uint64_t)ab.y << 32);
   const uint64_t wb = (uint64_t)ab.z | ((uint64_t)ab.w << 32);
   P.a = (uint32_t)(1 + wa % (kHashPrime - 1));
   P.b = (uint32_t)(wb % kHashPrime);
+  const uint32_t key[12] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w, k2.x, k2.y, k2.z, k2.w};
+  P.key[0] = key[0];
+  P.key[1] = key[1];
 #pragma unroll
-  for (uint32_t j = 0; j < 3; ++j) {
-    const Philox4 kk = philox_seeded(seed, k, 1u, j, tag);
-    P.key[4 * j + 0] = kk.x;
-    P.key[4 * j + 1] = kk.y;
-    P.key[4 * j + 2] = kk.z;
-    P.key[4 * j + 3] = kk.w;
-  }
-  const Philox4 coin = philox_seeded(seed, k, 2u, 0u, tag);
-  const uint32_t r = (n & 1u) ? 1u : 2u * (coin.x & 1u);
-  P.n_active = n - r;
+  for (int i = 2; i < 12; ++i) P.key[i] = key[i] ^ key[i - 2];
+  P.out1 = P.rounds == 8u ? key[6] : key[10];
+  P.out2 = P.rounds == 8u ? key[7] : key[11];
+  P.n_active = n - ((n & 1u) ? 1u : 2u * (coin & 1u));
   return P;
 }
 
-// Round function: top h bits of ((x ^ key) * C1, xor-folded by 16, * C2).
-__host__ __device__ __forceinline__ uint32_t feistel_f(uint32_t x, uint32_t key, uint32_t h) {
-  uint32_t y = (x ^ key) * 0x9E3779B1u;
+__host__ __device__ __forceinline__ Probe make_probe(uint32_t n, uint64_t seed, uint32_t k, uint32_t tag) {
+  return probe_from_words(n, philox_seeded(seed, k, 0u, 0u, tag), philox_seeded(seed, k, 1u, 0u, tag),
+                          philox_seeded(seed, k, 1u, 1u, tag), philox_seeded(seed, k, 1u, 2u, tag),
+                          philox_seeded(seed, k, 2u, 0u, tag).x);
+}
+
+#ifdef __CUDACC__
+// The same by a whole warp with the same arguments: lanes 0 to 4 evaluate one
+// of the five Philox blocks each and the words go round by shuffles, a quarter
+// of the instructions of five blocks in every lane.
+__device__ __forceinline__ Probe make_probe_warp(uint32_t n, uint64_t seed, uint32_t k, uint32_t tag) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t c1 = lane == 0u ? 0u : (lane <= 3u ? 1u : 2u), c2 = lane == 2u ? 1u : (lane == 3u ? 2u : 0u);
+  const Philox4 own = philox_seeded(seed, k, c1, c2, tag);
+  Philox4 w[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    w[j].x = __shfl_sync(0xffffffffu, own.x, j);
+    w[j].y = __shfl_sync(0xffffffffu, own.y, j);
+    w[j].z = __shfl_sync(0xffffffffu, own.z, j);
+    w[j].w = __shfl_sync(0xffffffffu, own.w, j);
+  }
+  return probe_from_words(n, w[0], w[1], w[2], w[3], __shfl_sync(0xffffffffu, own.x, 4));
+}
+#endif
+
+// Round function of u = x ^ key: top 32 - shift bits of (u * C1, xor-folded by
+// 16, * C2).  (The last shift as a high-word product, to move it off the
+// shift-and-logic pipe, was slower: 64 shifts but 32 high words per SM and clock.)
+__host__ __device__ __forceinline__ uint32_t feistel_f(uint32_t u, uint32_t shift) {
+  uint32_t y = u * 0x9E3779B1u;
   y ^= y >> 16;
   y *= 0x85EBCA6Bu;
-  return y >> (32u - h);
+  return y >> shift;
 }
 
 // One pass of the Feistel network on [2^hi] x [2^lo] (the generalised
 // construction for such domains, Black and Rogaway 2002): a round maps
 // (left, right) to (right, left ^ F(right)) with F as wide as the left half,
 // so the halves trade widths every round; after the even round count the left
-// half has hi bits again.
+// half has hi bits again.  With x_0 = left, x_1 = right and x_{i+1} = x_{i-1} ^
+// F(x_i ^ key), the pass carries u_i = x_i ^ key(i-1): then u_{i+1} = u_{i-1} ^
+// F ^ (key(i-2) ^ key(i)) is one three-input operation a round, where x and x ^
+// key took three.
 template <int ROUNDS>
 __host__ __device__ __forceinline__ uint32_t feistel_pass(const Probe& P, uint32_t x) {
-  uint32_t left = x >> P.lo, right = x & ((1u << P.lo) - 1u);
+  const uint32_t left = x >> P.lo, right = x & ((1u << P.lo) - 1u);
+  uint32_t u0 = right ^ P.key[0];                                   // u_1
+  uint32_t u1 = left ^ feistel_f(u0, P.sh_hi) ^ P.key[1];          // u_2
 #pragma unroll
-  for (int i = 0; i < ROUNDS; ++i) {
-    const uint32_t f = feistel_f(right, P.key[i], (i & 1) ? P.lo : P.hi);
-    const uint32_t nr = left ^ f;
-    left = right;
-    right = nr;
+  for (int i = 2; i < ROUNDS; ++i) {
+    const uint32_t u2 = u0 ^ feistel_f(u1, (i & 1) ? P.sh_hi : P.sh_lo) ^ P.key[i];
+    u0 = u1;
+    u1 = u2;
   }
-  return (left << P.lo) | right;
+  return ((u1 ^ P.out2) << P.lo) | (u0 ^ feistel_f(u1, P.sh_lo) ^ P.out1);
 }
 
 __host__ __device__ __forceinline__ uint32_t feistel_once(const Probe& P, uint32_t x) {
@@ -200,49 +234,36 @@ __host__ __device__ __forceinline__ uint32_t probe_pi(const Probe& P, uint32_t v
   return x;
 }
 
-// (a*u + b) mod (2^31 - 1) by Mersenne folding; a < 2^31, u < 2^31, b < 2^31.
-__host__ __device__ __forceinline__ uint32_t hash_mod_p(uint32_t a, uint32_t u, uint32_t b) {
-  const uint64_t t = (uint64_t)a * (uint64_t)u + (uint64_t)b;  // < 2^62 + 2^31
-  uint64_t m = (t & kHashPrime) + (t >> 31);                    // < 2^32
-  m = (m & kHashPrime) + (m >> 31);                             // <= 2^31
-  if (m >= kHashPrime) m -= kHashPrime;
-  return (uint32_t)m;
+// Parity of (a u + b) mod p, p = 2^31 - 1, for a, b < p and u < 2^30: one
+// Mersenne fold m = (t mod 2^31) + floor(t / 2^31) < 2p, all in 32-bit words;
+// p is odd, so subtracting it when m >= p, that is when m + 1 has bit 31 set,
+// flips the parity.
+__host__ __device__ __forceinline__ uint32_t hash_parity(uint32_t a, uint32_t u, uint32_t b) {
+  const uint64_t t = (uint64_t)a * (uint64_t)u + (uint64_t)b;
+  const uint32_t lo = (uint32_t)t, hi = (uint32_t)(t >> 32);
+#ifdef __CUDA_ARCH__
+  const uint32_t m = (lo & 0x7FFFFFFFu) + __funnelshift_l(lo, hi, 1);
+#else
+  const uint32_t m = (lo & 0x7FFFFFFFu) + ((hi << 1) | (lo >> 31));
+#endif
+  return (m ^ ((m + 1u) >> 31)) & 1u;
 }
 
-// z from pi: 0 on the zero set, else +1 when h(pair) + pi is even.
-__host__ __device__ __forceinline__ int probe_z_from_pi(const Probe& P, uint32_t pi) {
-  if (pi >= P.n_active) return 0;
-  const uint32_t hv = hash_mod_p(P.a, pi >> 1, P.b) & 1u;
-  return ((hv ^ pi) & 1u) ? -1 : 1;
+// Sign of a node outside the zero set (pi < n - r): 1 when h(pair) + pi is odd
+// (z = -1).
+__host__ __device__ __forceinline__ uint32_t probe_negative(const Probe& P, uint32_t pi) {
+  return (hash_parity(P.a, pi >> 1, P.b) ^ pi) & 1u;
 }
 
-__host__ __device__ __forceinline__ int probe_z(const Probe& P, uint32_t v) { return probe_z_from_pi(P, probe_pi(P, v)); }
+__host__ __device__ __forceinline__ int probe_z(const Probe& P, uint32_t v) {
+  const uint32_t pi = probe_pi(P, v);
+  return pi >= P.n_active ? 0 : (probe_negative(P, pi) ? -1 : 1);
+}
 
 // Term z/d in FP32 from the stored correctly rounded reciprocal: +-1/d is the
-// IEEE quotient of +-1 by d and 0/d is +0.
-__device__ __forceinline__ float signed_term(int z, uint32_t inv_bits) {
-  return z == 0 ? 0.0f : __uint_as_float(z > 0 ? inv_bits : (inv_bits ^ 0x80000000u));
-}
-
-// z for two nodes at once: one cycle-walk queue, so a lane runs iter(s)+iter(t)
-// Feistel passes instead of the warp paying max(iter(s)) + max(iter(t)).
-__device__ __forceinline__ void probe_pi_pair(const Probe& P, uint32_t vs, uint32_t vt, uint32_t& pis,
-                                              uint32_t& pit) {
-  uint32_t x = vs;
-  bool second = false;
-  while (true) {
-    x = feistel_once(P, x);
-    if (x < P.n) {
-      if (!second) {
-        pis = x;
-        second = true;
-        x = vt;
-      } else {
-        pit = x;
-        break;
-      }
-    }
-  }
+// IEEE quotient of +-1 by d and 0/d is +0.  `sign`: bit 31 set for z = -1.
+__device__ __forceinline__ float signed_term(bool zero, uint32_t sign, uint32_t inv_bits) {
+  return zero ? 0.0f : __uint_as_float(inv_bits ^ (sign & 0x80000000u));
 }
 
 }  // namespace pw

@@ -272,7 +272,7 @@ static pw_status load_common(int64_t n, const int64_t* rp, const int32_t* col, i
   g->device = device;
   g->n = n;
   g->nnz = nnz;
-  g->table_probe_cost = (double)n;
+  default_walk_model(n, &g->table_probe_cost, &g->table_visit_gain);
   g->d_min = dmn;
   g->d_max = dmx;
   g->bipartite = bip;

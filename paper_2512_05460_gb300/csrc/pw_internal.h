@@ -104,10 +104,9 @@ struct pw_graph {
   int sm_count = 0;
   // Walk-mode cost model: a query's probes run in the probe-table kernel when
   //   K * table_probe_cost < 2 K R (L + 1) * table_visit_gain.
-  // Defaults (set at load): n and 2.5, in units of one Feistel pass per node
-  // (table) against about 2.5 passes per visit (per-visit evaluation);
-  // pw_autotune replaces them by nanoseconds measured on this graph.
-  double table_probe_cost = 0.0, table_visit_gain = 2.5;
+  // Defaults set at load (default_walk_model); pw_autotune replaces them by
+  // nanoseconds measured on this graph.
+  double table_probe_cost = 0.0, table_visit_gain = 0.0;
   int tuned = 0;
   int4* d_rec = nullptr;     // nnz neighbour records (fused layout only)
   int32_t* d_col = nullptr;  // nnz neighbour ids (always)
@@ -115,10 +114,8 @@ struct pw_graph {
   int layout = 1;            // walk access: 1 fused records, 2 col_idx + node records
   cudaStream_t stream = nullptr;
   std::map<std::pair<const void*, size_t>, int> grids;  // persistent grid per walk kernel and shared memory
-  // Kernel variants (pw_autotune): per-visit kernel with compiler-chosen
-  // registers (1) or registers capped for 3 blocks per SM (3); table-kernel
-  // block size (0: by shared memory, else 256, 512 or 1024 threads).
-  int visit_minb = 1;
+  // Table-kernel block size (pw_autotune; 0: by shared memory, else 256, 512
+  // or 1024 threads).
   int table_threads = 0;
   int walk_policy = 0;  // walk_mode 0 means: 0 the cost model per query, 1 all per-visit, 2 all table
   // L2 access-policy window of the walk and server launches
@@ -158,6 +155,17 @@ inline cudaError_t launch_with_window(const pw_graph* g, void (*fn)(K...), int g
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, fn, static_cast<A&&>(args)...);
+}
+
+// The walk-mode cost model of an untuned graph or server, in Feistel passes: a
+// table takes one per element of the permutation's domain 2^b, and a visit
+// that reads the table saves 1.15 (n = 10^5: 333 ns against 2.9 ps; R-MAT 2^20:
+// 3.4 to 5.6 us against 4.2 ps).
+inline void default_walk_model(int64_t n, double* probe_cost, double* visit_gain) {
+  int b = 2;
+  while (b < 31 && ((int64_t)1 << b) < n) ++b;
+  *probe_cost = (double)((int64_t)1 << (b == 3 ? 4 : b));
+  *visit_gain = 1.15;
 }
 
 pw_status set_error(pw_status st, const std::string& msg);

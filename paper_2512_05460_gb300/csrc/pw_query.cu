@@ -362,15 +362,18 @@ struct GraphOf<true> {
   static __device__ __forceinline__ SplitRecords get(const WalkArgs& A) { return SplitRecords{A.col, A.node}; }
 };
 
-// MINB: 1 leaves the registers to the compiler (2 blocks of 256 per SM), 3
-// caps them for 3 blocks per SM (more walks in flight, some spills); the
-// autotuner picks one per graph.
-template <bool DEBUG, bool PILOT, bool SPLIT, int MINB>
-__global__ void __launch_bounds__(kWalkThreads, MINB) walk_kernel(WalkArgs A) {
+// 3 blocks per SM (80 registers, 9 KB of pools each, the rest of the SM's
+// memory caching the graph): 4 blocks (64 registers, some spilled) took 5.9 ps
+// a visit on a 2000^2 grid against 5.3, 6.2 against 5.8 on a 10^5-node graph,
+// and 9.8 against 10.2 on R-MAT 2^20.
+template <bool DEBUG, bool PILOT, bool SPLIT>
+__global__ void __launch_bounds__(kWalkThreads, DEBUG ? 1 : 3) walk_kernel(WalkArgs A) {
   const auto gr = GraphOf<SPLIT>::get(A);
   const uint32_t lane = threadIdx.x & 31u;
   const unsigned long long total = A.totals->tiles;
   if (total == 0ull) return;
+  __shared__ VisitPool pools[kWalkThreads / 32];
+  VisitPool& pool = pools[threadIdx.x >> 5];
   for (;;) {
     unsigned long long tile = 0;
     if (lane == 0) tile = atomicAdd(A.counter, 1ull);
@@ -386,12 +389,13 @@ __global__ void __launch_bounds__(kWalkThreads, MINB) walk_kernel(WalkArgs A) {
     const uint32_t k = P.k_begin + kl;
     SumDigits sum;
     sum_clear(sum);
+    const Probe pr = make_probe_warp(A.n, P.seed, k, A.probe_tag);
+    if (lane == 0) pool.probe = pr;
+    const uint64_t pair = (uint64_t)k * R + p;
+    const uint32_t m = R - c * 32u < 32u ? R - c * 32u : 32u;
+    const float U = walk_pair_visit<DEBUG>(gr, A.visits, A.walk_tag, pool, P.s, P.t, P.L, P.seed, pair, m, lane);
     if (p < R) {
-      const Probe pr = make_probe(A.n, P.seed, k, A.probe_tag);
-      const uint64_t pair = (uint64_t)k * R + p;
-      const ZOnTheFly zp{pr};
-      const float U = walk_pair<DEBUG>(gr, A.visits, A.walk_tag, zp, P.s, P.t, P.L, P.seed, pair);
-      if (DEBUG && A.u_debug && q == 0) A.u_debug[(uint64_t)k * R + p] = U;
+      if (DEBUG && A.u_debug && q == 0) A.u_debug[pair] = U;
       sum_add(sum, U);
     }
     sum_warp_reduce(sum);
@@ -612,15 +616,10 @@ static int default_table_threads(const pw_graph* g) {
 
 using WalkFn = void (*)(WalkArgs);
 
-// The per-visit kernel of a launch (DEBUG builds exist only at MINB 1).
-static WalkFn walk_fn(bool debug, bool pilot, bool split, int minb) {
-  if (debug) return split ? walk_kernel<true, false, true, 1> : walk_kernel<true, false, false, 1>;
-  if (minb == 3) {
-    if (pilot) return split ? walk_kernel<false, true, true, 3> : walk_kernel<false, true, false, 3>;
-    return split ? walk_kernel<false, false, true, 3> : walk_kernel<false, false, false, 3>;
-  }
-  if (pilot) return split ? walk_kernel<false, true, true, 1> : walk_kernel<false, true, false, 1>;
-  return split ? walk_kernel<false, false, true, 1> : walk_kernel<false, false, false, 1>;
+static WalkFn walk_fn(bool debug, bool pilot, bool split) {
+  if (debug) return split ? walk_kernel<true, false, true> : walk_kernel<true, false, false>;
+  if (pilot) return split ? walk_kernel<false, true, true> : walk_kernel<false, true, false>;
+  return split ? walk_kernel<false, false, true> : walk_kernel<false, false, false>;
 }
 
 // The table kernel of a launch (DEBUG builds exist only at 256 threads).
@@ -646,7 +645,7 @@ static int grid_of(pw_graph* g, WalkFn fn, int threads, size_t smem) {
 }
 
 static pw_status launch_walk(pw_graph* g, cudaStream_t stream, const WalkArgs& a, bool debug, bool pilot) {
-  const WalkFn fn = walk_fn(debug, pilot, g->layout == 2, g->visit_minb);
+  const WalkFn fn = walk_fn(debug, pilot, g->layout == 2);
   const cudaError_t e = launch_with_window(g, fn, grid_of(g, fn, kWalkThreads, 0), kWalkThreads, 0, stream, a);
   count_launch();
   PW_CUDA_TRY(e);
@@ -985,7 +984,7 @@ static pw_status graph_batch(pw_graph* g, int64_t count, const char* h, char* ho
     const WalkFn tf = table_fn(false, g->layout == 2, table_threads(g));
     grid_of(g, tf, table_threads(g), table_bytes(g));
   }
-  for (int pilot = 0; pilot < 2; ++pilot) grid_of(g, walk_fn(false, pilot != 0, g->layout == 2, g->visit_minb), kWalkThreads, 0);
+  for (int pilot = 0; pilot < 2; ++pilot) grid_of(g, walk_fn(false, pilot != 0, g->layout == 2), kWalkThreads, 0);
   std::vector<unsigned char> key;
   key_put(key, count);
   key_put(key, total_K);
@@ -993,7 +992,6 @@ static pw_status graph_batch(pw_graph* g, int64_t count, const char* h, char* ho
   key_put(key, params ? params->walk_mode : 0);
   key_put(key, g->table_probe_cost);
   key_put(key, g->table_visit_gain);
-  key_put(key, g->visit_minb);
   key_put(key, g->walk_policy);
   key_put(key, g->table_threads);
   key_put(key, g->l2_window);
@@ -1406,8 +1404,8 @@ pw_status pw_profile(pw_graph* g, int32_t enable, int32_t reset, pw_profile_stat
   return PW_OK;
 }
 
-// Walk-kernel autotuner: time the sample in each walk kernel and its variants,
-// keep the fastest variant of each, and fit the graph's cost model (per-visit:
+// Walk-kernel autotuner: time the sample in each walk kernel,
+// keep the table kernel's fastest block size, and fit the graph's cost model (per-visit:
 // visits * visit_ns; table: probes * probe_ns + visits * table_visit_ns).  The
 // runs use a FIXED budget (B = 4 probes per block, the caller's G, R = 1024 or
 // 256 replicas), so the two table runs have the same probes and visits in the
@@ -1460,19 +1458,8 @@ pw_status pw_autotune(pw_graph* g, int64_t count, const int64_t* s, const int64_
     return PW_OK;
   };
   Run dv, dt, dq;
-  // per-visit kernel: registers left to the compiler or capped for 3 blocks/SM
-  int best_minb = 1;
-  for (int minb : {1, 3}) {
-    g->visit_minb = minb;
-    Run r;
-    if ((st = timed(1, R_hi, &r)) != PW_OK) return st;
-    if (minb == 1 || r.d.walk_ms < dv.d.walk_ms) {
-      dv = r;
-      best_minb = minb;
-    }
-  }
-  g->visit_minb = best_minb;
-  out->visit_occupancy = best_minb;
+  if ((st = timed(1, R_hi, &dv)) != PW_OK) return st;
+  out->visit_occupancy = 3;
   out->sample_ms[0] = dv.d.walk_ms;
   out->visit_ns = dv.n_visits > 0 ? 1e6 * dv.d.walk_ms / dv.n_visits : 0.0;
   out->sample_mode = 1;

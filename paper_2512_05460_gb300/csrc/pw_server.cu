@@ -65,7 +65,7 @@ struct ServerArgs {
   const int32_t* col;  // col_idx (layout 2)
   const int4* node;
   uint32_t n;
-  uint32_t table_words;  // 0: graph too large for a shared-memory table
+  uint32_t has_table;  // 0: graph too large for a shared-memory table
   SlotDev* slots;
   unsigned long long* heads;  // [2]: host ring, device ring
   unsigned long long* dtail;  // producer position of the device ring
@@ -155,17 +155,17 @@ __device__ bool find_job(const ServerArgs& A, uint32_t& slot, uint32_t& stage, u
   return false;
 }
 
-// One per-visit replica (probe entries by Feistel at each visit), compiled as a
-// separate function.  Inlined into the job loop below, the same code ran about
-// 20x slower per walk step on a 4M-node grid (identical results); behind a call
+// One warp tile of per-visit replicas, compiled as a separate function.
+// Inlined into the job loop below, an earlier form of this code ran about 20x
+// slower per walk step on a 4M-node grid (identical results); behind a call
 // boundary it runs at walk_kernel's speed.
 template <class GR>
 __device__ __noinline__ float server_walk_visit(const GR gr, uint32_t n, uint32_t walk_tag, uint32_t probe_tag,
-                                                int32_t s, int32_t t, int32_t L, uint64_t seed, uint32_t k,
-                                                uint64_t pair) {
-  const Probe pr = make_probe(n, seed, k, probe_tag);
-  const ZOnTheFly zp{pr};
-  return walk_pair<false>(gr, nullptr, walk_tag, zp, s, t, L, seed, pair);
+                                                VisitPool* pool, int32_t s, int32_t t, int32_t L, uint64_t seed,
+                                                uint32_t k, uint64_t pair, uint32_t m) {
+  const Probe pr = make_probe_warp(n, seed, k, probe_tag);
+  if ((threadIdx.x & 31u) == 0u) pool->probe = pr;
+  return walk_pair_visit<false>(gr, nullptr, walk_tag, *pool, s, t, L, seed, pair, m, threadIdx.x & 31u);
 }
 
 // TABLE: the graph's probe table fits in shared memory, so main-stage jobs may
@@ -189,8 +189,11 @@ template <bool TABLE, class GR, int MINB>
 __global__ void __launch_bounds__(kServerThreads, MINB) server_kernel(ServerArgs A) {
   const GR gr = server_graph<GR>(A);
   extern __shared__ uint32_t smem[];
+  // one place for the job's table or its warps' pools (a job uses one or the
+  // other) and, after a query's last job, its block means
   uint32_t* tab = smem;
-  double* means = (double*)(smem + A.table_words);  // table_words is a multiple of 4
+  VisitPool* pools = (VisitPool*)smem;
+  double* means = (double*)smem;
   __shared__ unsigned long long j_sum[kJobProbes][kSumDigits];
   __shared__ uint32_t j_slot, j_stage, j_k, j_count, j_valid, j_last, j_tile;
   const uint32_t lane = threadIdx.x & 31u;
@@ -231,17 +234,17 @@ __global__ void __launch_bounds__(kServerThreads, MINB) server_kernel(ServerArgs
       const uint32_t k = k0 + j;
       SumDigits sum;
       sum_clear(sum);
-      if (p < R) {
-        const uint64_t pair = (uint64_t)k * R + p;
-        float U;
-        if (TABLE && table) {
-          const ZTable zp = table_reader(tab, A.n);
-          U = walk_pair_table<false>(gr, nullptr, walk_tag, zp, P.s, P.t, P.L, P.seed, pair);
-        } else {
-          U = server_walk_visit<GR>(gr, A.n, walk_tag, probe_tag, P.s, P.t, P.L, P.seed, k, pair);
-        }
-        sum_add(sum, U);
+      const uint64_t pair = (uint64_t)k * R + p;
+      float U = 0.0f;
+      if (TABLE && table) {
+        const ZTable zp = table_reader(tab, A.n);
+        if (p < R) U = walk_pair_table<false>(gr, nullptr, walk_tag, zp, P.s, P.t, P.L, P.seed, pair);
+      } else {
+        const uint32_t rest = R - (p - lane), m = rest < 32u ? rest : 32u;
+        U = server_walk_visit<GR>(gr, A.n, walk_tag, probe_tag, pools + (threadIdx.x >> 5), P.s, P.t, P.L, P.seed, k,
+                                  pair, m);
       }
+      if (p < R) sum_add(sum, U);
       sum_warp_reduce(sum);
       if (lane == 0) {
 #pragma unroll
@@ -290,7 +293,7 @@ __global__ void __launch_bounds__(kServerThreads, MINB) server_kernel(ServerArgs
           // visit, by the graph's walk-mode cost model
           const double visits = 2.0 * (double)M.R * (double)(P.L + 1);
           const double probe_cost = __ldcg(A.model), visit_gain = __ldcg(A.model + 1);
-          __stcg(&S->use_table, (A.table_words > 0 && probe_cost < visit_gain * visits) ? 1u : 0u);
+          __stcg(&S->use_table, (A.has_table && probe_cost < visit_gain * visits) ? 1u : 0u);
           __threadfence();
           const unsigned long long pos = atomicAdd(A.dtail, 1ull);
           const uint32_t idx = (uint32_t)(pos % A.cap) + A.cap;
@@ -388,6 +391,7 @@ struct pw_server {
   uint64_t host_tail = 0;
   cudaStream_t kstream = nullptr, cstream = nullptr;
   size_t smem = 0;
+  bool has_table = false;  // the graph's probe table fits in shared memory
   int minb = 2;      // occupancy variant of the per-visit-only kernel (server_fn)
   int grid = 0;      // blocks of the persistent kernel: SMs x resident blocks of that variant
   int grids[2] = {0, 0};  // per-visit-only kernel: grid at minb 2, 3
@@ -447,7 +451,7 @@ static ServerArgs server_args(pw_server* sv) {
   a.col = sv->g->d_col;
   a.node = sv->g->d_node;
   a.n = (uint32_t)sv->g->n;
-  a.table_words = (uint32_t)((sv->smem - kServerMeansBytes) / sizeof(uint32_t));
+  a.has_table = sv->has_table ? 1u : 0u;
   a.slots = sv->d_slots;
   a.heads = sv->d_ctl;
   a.dtail = sv->d_ctl + 2;
@@ -508,8 +512,7 @@ static bool admit(pw_server* sv, const Request& rq) {
   h.ps = (double*)(sv->d_pool + off + sizeof(double) * (size_t)P.K);
   if (!pilot) {
     const double visits = 2.0 * (double)P.R * (double)(P.L + 1);
-    const uint32_t words = (uint32_t)((sv->smem - kServerMeansBytes) / sizeof(uint32_t));
-    h.use_table = (words > 0 && sv->table_probe_cost < sv->table_visit_gain * visits) ? 1u : 0u;
+    h.use_table = (sv->has_table && sv->table_probe_cost < sv->table_visit_gain * visits) ? 1u : 0u;
   }
   sv->h_comp[slot].ticket = 0;
   cudaMemcpyAsync(sv->d_slots + slot, &h, sizeof(SlotDev), cudaMemcpyHostToDevice, sv->cstream);
@@ -576,7 +579,7 @@ static void worker_loop(pw_server* sv) {
         cudaStreamWaitEvent(sv->kstream, ev, 0);
         cudaEventDestroy(ev);
         cudaMemsetAsync(sv->d_ctl + 4, 0, sizeof(unsigned long long), sv->kstream);  // exit flag
-        const ServerFn fn = server_fn(args.table_words > 0, sv->g->layout, minb);
+        const ServerFn fn = server_fn(sv->has_table, sv->g->layout, minb);
         const cudaError_t e = launch_with_window(sv->g, fn, grid, kServerThreads, sv->smem, sv->kstream, args);
         count_launch();
         if (e != cudaSuccess) {
@@ -615,13 +618,11 @@ pw_status pw_server_create(pw_graph* g, const pw_params* params, size_t accum_by
   pw_server* sv = new pw_server();
   sv->g = g;
   sv->ba = ba;
-  // The default walk-mode model (n Feistel passes per table against 2.5 per
-  // visit), not the graph's autotuned costs: those are fitted on the batch
-  // kernels, whose per-visit path is faster than the server's (the server's
-  // runs inside the table-capable kernel at its register cap).
-  // pw_server_tune picks the server's own policy by timing it.
-  sv->table_probe_cost = (double)g->n;
-  sv->table_visit_gain = 2.5;
+  // The default walk-mode model, not the graph's autotuned costs: those are
+  // fitted on the batch kernels, and the server's per-visit walks run inside
+  // the table-capable kernel at its register cap.  pw_server_tune picks the
+  // server's own policy by timing it.
+  default_walk_model(g->n, &sv->table_probe_cost, &sv->table_visit_gain);
   sv->S = 4096;
   sv->cap = 4096;
   sv->pool_bytes = accum_bytes;
@@ -661,12 +662,14 @@ pw_status pw_server_create(pw_graph* g, const pw_params* params, size_t accum_by
   sv->slot_range.assign(sv->S, {0, 0});
   sv->slot_submit_ms.assign(sv->S, 0.0);
   for (uint32_t s = 0; s < sv->S; ++s) sv->free_slots.push_back(sv->S - 1 - s);
-  // shared memory: probe table (if it fits next to the block means) + block means
-  const size_t ubytes = kServerMeansBytes;
-  // rounded to 16 bytes so the FP64 block means that follow stay aligned
-  const size_t tbytes = (sizeof(uint32_t) * (size_t)table_words((uint32_t)g->n) + 15) & ~(size_t)15;
-  sv->smem = ubytes + ((tbytes + ubytes <= 200 * 1024) ? tbytes : 0);
-  const bool with_table = sv->smem > ubytes;
+  // shared memory: the probe table (if it fits), the warps' pools and the block
+  // means of a finished query, all at the same place
+  const size_t tbytes = sizeof(uint32_t) * (size_t)table_words((uint32_t)g->n);
+  const size_t pbytes = sizeof(VisitPool) * (kServerThreads / 32);
+  const bool with_table = tbytes + kServerMeansBytes <= 200 * 1024;
+  sv->has_table = with_table;
+  sv->smem = kServerMeansBytes > pbytes ? kServerMeansBytes : pbytes;
+  if (with_table && tbytes > sv->smem) sv->smem = tbytes;
   for (int v = 0; v < (with_table ? 1 : 2); ++v) {
     const ServerFn fn = server_fn(with_table, g->layout, 2 + v);
     if ((e = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sv->smem)) !=
@@ -758,7 +761,7 @@ pw_status pw_server_tune(pw_server* sv, int64_t count, const int64_t* s, const i
   if (!sv || !out || !s || !t || !eps || !L || count <= 0) return set_error(PW_ERR_ARG, "NULL argument or empty sample");
   memset(out, 0, sizeof *out);
   pw_graph* g = sv->g;
-  const bool table = sv->smem > kServerMeansBytes;
+  const bool table = sv->has_table;
   std::vector<uint64_t> tk((size_t)count);
   std::vector<double> ref, got((size_t)count);
   // the sample as a burst, once to warm up and once timed: queries/s; the
@@ -817,7 +820,9 @@ pw_status pw_server_tune(pw_server* sv, int64_t count, const int64_t* s, const i
   // candidate policies {table cost per probe, saving per visit}: the default
   // model, the graph's batch-fitted model, every query per-visit, every query
   // on the table
-  const double cand[4][2] = {{(double)g->n, 2.5}, {g->table_probe_cost, g->table_visit_gain}, {1.0, 0.0}, {0.0, 1.0}};
+  double cost0, gain0;
+  default_walk_model(g->n, &cost0, &gain0);
+  const double cand[4][2] = {{cost0, gain0}, {g->table_probe_cost, g->table_visit_gain}, {1.0, 0.0}, {0.0, 1.0}};
   const bool valid[4] = {true, g->tuned != 0, true, true};
   int best = 0;
   for (int c = 0; c < 4; ++c) {

@@ -1,6 +1,7 @@
 // Walk building blocks shared by the batch kernels and the server kernel:
-// the two ways of reading probe entries (evaluated per visit, or from a
-// per-probe shared-memory table) and one replica of Algorithm 1's inner loop.
+// Algorithm 1's inner loop for the replicas of one probe, with probe entries
+// evaluated at each visit (a warp's pool of visits) or read from a per-probe
+// table in shared memory.
 #pragma once
 #include <stdint.h>
 
@@ -36,93 +37,123 @@ struct SplitRecords {
   }
 };
 
-// Probe entries evaluated on the fly (Section 3.3 generator): one cycle-walk
-// queue for the two walks so a lane pays iter(s) + iter(t) Feistel passes.
-struct ZOnTheFly {
-  const Probe& pr;
-  __device__ __forceinline__ void pair(uint32_t vs, uint32_t vt, int& zs, int& zt) const {
-    uint32_t pis, pit;
-    probe_pi_pair(pr, vs, vt, pis, pit);
-    zs = probe_z_from_pi(pr, pis);
-    zt = probe_z_from_pi(pr, pit);
-  }
-};
-
 // Probe entries read from the block's table of z^(k) (built once per probe):
 // one sign bit per node (set = negative) plus the ids of the r <= 2 nodes of
 // the zero set, which the bits cannot express.
 struct ZTable {
   const uint32_t* tab;
   uint32_t zero0, zero1;  // zero-set nodes, 0xFFFFFFFF when absent
-  __device__ __forceinline__ int from_word(uint32_t word, uint32_t v) const {
-    const int neg = (int)((word >> (v & 31u)) & 1u);
-    return (v == zero0 || v == zero1) ? 0 : 1 - 2 * neg;
-  }
-  __device__ __forceinline__ int one(uint32_t v) const { return from_word(tab[v >> 5], v); }
-  __device__ __forceinline__ void pair(uint32_t vs, uint32_t vt, int& zs, int& zt) const {
-    zs = one(vs);
-    zt = one(vt);
+  __device__ __forceinline__ uint32_t word(uint32_t v) const { return tab[v >> 5]; }
+  // the term z/d of node v from its table word: rotating left by 31 - v mod 32
+  // puts the node's bit in the sign position
+  __device__ __forceinline__ float term(uint32_t word, uint32_t v, uint32_t inv) const {
+    return signed_term(v == zero0 || v == zero1, __funnelshift_l(word, word, ~v), inv);
   }
 };
 
-// One replica: walks from s and t interleaved, a and b summed in FP32 in step
-// order (Eq. hatphi-def), U_p = a - b.  The load of X_{i+1} is issued before
-// the probe entry of X_i is evaluated so the gather latency overlaps the
-// integer work.
-template <bool DEBUG, class GR, class ZP>
-__device__ __forceinline__ float walk_pair(const GR& gr, uint32_t* visits, uint32_t walk_tag, const ZP& zp, int32_t s,
-                                           int32_t t, int32_t L, uint64_t seed, uint64_t pair) {
-  int4 xs = gr.start(s), xt = gr.start(t);
-  int zs, zt;
-  zp.pair((uint32_t)xs.x, (uint32_t)xt.x, zs, zt);
-  float a = signed_term(zs, (uint32_t)xs.w);
-  float b = signed_term(zt, (uint32_t)xt.w);
-  if (DEBUG) {
-    atomicAdd(visits + xs.x, 1u);
-    atomicAdd(visits + xt.x, 1u);
+// Visits per side that a warp walks ahead before it evaluates their probe
+// entries, and the shared memory of one warp's pool (the nodes, then pi, of
+// 2 x 32 walks).  Kept small: what shared memory takes of the SM's 256 KB is
+// not there for the graph and for the lines of gathers in flight (128 B each,
+// 1,500 walks and more per SM): at 50 KB a block the server's walks ran at half
+// speed, and with twice the steps a 2000^2 grid took 6.3 ps a visit, not 5.3.
+constexpr uint32_t kPoolSteps = 4;  // one Philox block of each walk
+struct VisitPool {
+  uint32_t node[2 * kPoolSteps * 32];
+  Probe probe;  // kept here, not in registers, while the warp walks
+};
+
+// pi of every node in pool.node[0..total), in place, by the whole warp.  A
+// lane runs one Feistel pass per iteration and takes the pool's next node when
+// its pass lands in [n], so that the lanes stay busy whatever their
+// cycle-walks' lengths.
+template <int ROUNDS>
+__device__ __forceinline__ void pool_permute(VisitPool& pool, uint32_t total, uint32_t lane) {
+  const Probe pr = pool.probe;
+  const uint32_t below = (1u << lane) - 1u;
+  uint32_t i = lane, next = 32u;  // 32 + nodes done so far
+  uint32_t x = i < total ? pool.node[i] : 0u;
+  while (next < total + 32u) {
+    x = feistel_pass<ROUNDS>(pr, x);
+    const bool done = x < pr.n && i < total;
+    const uint32_t who = __ballot_sync(0xffffffffu, done);
+    if (done) {
+      pool.node[i] = x;
+      i = next + __popc(who & below);
+      if (i < total) x = pool.node[i];
+    }
+    next += __popc(who);
   }
-  if (L == 0) return __fsub_rn(a, b);
+}
+
+// One replica per lane (lanes below m <= 32 of one warp; all lanes call) of the
+// probe in pool.probe: U_p
+// from the walks of pair `pair` from s and t, a and b summed in FP32 in step
+// order (Eq. hatphi-def).  The warp walks both sides kPoolSteps visits ahead
+// into its pool, evaluates the pool's probe entries together, then adds the
+// terms in order.
+//
+// Bound by the shift-and-logic pipe: a visit costs 2^b / n passes of 26 such
+// operations and 16 products, a quarter of a Philox block, and about 20 more.
+// Evaluating each step's two nodes in their lane, the warp waited for the
+// longest of 32 pairs of cycle-walks: 7.3 passes a step against 3.3 on average
+// at n = 0.62 2^b, 3.1 against 2.1 at 0.95 2^b.  Per visit, before and with the
+// pool: 10.9 -> 5.8 ps (n = 10^5 in L2), 16.5 -> 10.2 (R-MAT 2^20), 7.4 -> 5.3
+// (2000^2 grid).
+template <bool DEBUG, class GR>
+__device__ __forceinline__ float walk_pair_visit(const GR& gr, uint32_t* visits, uint32_t walk_tag, VisitPool& pool,
+                                                 int32_t s, int32_t t, int32_t L, uint64_t seed, uint64_t pair,
+                                                 uint32_t m, uint32_t lane) {
+  const bool active = lane < m;
+  int4 xs = gr.start(s), xt = gr.start(t);
+  float a = 0.0f, b = 0.0f;
   const uint64_t ws = 2 * pair, wt = ws + 1;
-  // Philox key schedule computed inside each call: this path already holds the
-  // probe's Feistel keys, so hoisting the ten round keys would cost registers
-  const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
-  Philox4 rs = philox4x32_10((uint32_t)ws, (uint32_t)(ws >> 32), 0u, walk_tag, k0, k1);
-  Philox4 rt = philox4x32_10((uint32_t)wt, (uint32_t)(wt >> 32), 0u, walk_tag, k0, k1);
-  int4 ns = gr.next(xs, rs.y);
-  int4 nt = gr.next(xt, rt.y);
-  for (uint32_t blk = 0;; ++blk) {
+  uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
+  const uint32_t count = (uint32_t)L + 1u;
+  for (uint32_t v0 = 0; v0 < count; v0 += kPoolSteps) {
+    const uint32_t steps = count - v0 < kPoolSteps ? count - v0 : kPoolSteps;
+    uint32_t inv_s[kPoolSteps], inv_t[kPoolSteps];
+    if (active) {
+      asm volatile("" : "+r"(k0), "+r"(k1));  // keeps the 20 round keys from being held over the pool's phase
+      const Philox4 rs = philox4x32_10((uint32_t)ws, (uint32_t)(ws >> 32), v0 >> 2, walk_tag, k0, k1);
+      const Philox4 rt = philox4x32_10((uint32_t)wt, (uint32_t)(wt >> 32), v0 >> 2, walk_tag, k0, k1);
 #pragma unroll
-    for (int w = 0; w < 4; ++w) {
-      if (w == 0 && blk == 0) continue;
-      const uint32_t i = blk * 4u + (uint32_t)w;  // ns, nt hold X_i
-      const bool more = i < (uint32_t)L;
-      int4 ns2 = ns, nt2 = nt;
-      if (more) {
-        uint32_t wsw, wtw;
-        if (w == 3) {
-          rs = philox4x32_10((uint32_t)ws, (uint32_t)(ws >> 32), blk + 1u, walk_tag, k0, k1);
-          rt = philox4x32_10((uint32_t)wt, (uint32_t)(wt >> 32), blk + 1u, walk_tag, k0, k1);
-          wsw = rs.x;
-          wtw = rt.x;
-        } else {
-          wsw = (w == 0) ? rs.y : (w == 1) ? rs.z : rs.w;
-          wtw = (w == 0) ? rt.y : (w == 1) ? rt.z : rt.w;
+      for (uint32_t j = 0; j < kPoolSteps; ++j) {
+        if (j < steps) {
+          if (j != 0 || v0 != 0) {
+            xs = gr.next(xs, j == 0u ? rs.x : (j == 1u ? rs.y : (j == 2u ? rs.z : rs.w)));
+            xt = gr.next(xt, j == 0u ? rt.x : (j == 1u ? rt.y : (j == 2u ? rt.z : rt.w)));
+          }
+          pool.node[2u * j * m + lane] = (uint32_t)xs.x;
+          pool.node[(2u * j + 1u) * m + lane] = (uint32_t)xt.x;
+          inv_s[j] = (uint32_t)xs.w;
+          inv_t[j] = (uint32_t)xt.w;
+          if (DEBUG) {
+            atomicAdd(visits + xs.x, 1u);
+            atomicAdd(visits + xt.x, 1u);
+          }
         }
-        ns2 = gr.next(ns, wsw);
-        nt2 = gr.next(nt, wtw);
       }
-      zp.pair((uint32_t)ns.x, (uint32_t)nt.x, zs, zt);
-      a = __fadd_rn(a, signed_term(zs, (uint32_t)ns.w));
-      b = __fadd_rn(b, signed_term(zt, (uint32_t)nt.w));
-      if (DEBUG) {
-        atomicAdd(visits + ns.x, 1u);
-        atomicAdd(visits + nt.x, 1u);
+    }
+    __syncwarp();
+    if (pool.probe.rounds == 8u)
+      pool_permute<8>(pool, 2u * steps * m, lane);
+    else
+      pool_permute<12>(pool, 2u * steps * m, lane);
+    __syncwarp();
+    if (active) {
+      const Probe pr = pool.probe;
+#pragma unroll
+      for (uint32_t j = 0; j < kPoolSteps; ++j) {
+        if (j < steps) {
+          const uint32_t ps = pool.node[2u * j * m + lane], pt = pool.node[(2u * j + 1u) * m + lane];
+          a = __fadd_rn(a, signed_term(ps >= pr.n_active, probe_negative(pr, ps) << 31, inv_s[j]));
+          b = __fadd_rn(b, signed_term(pt >= pr.n_active, probe_negative(pr, pt) << 31, inv_t[j]));
+        }
       }
-      if (!more) return __fsub_rn(a, b);
-      ns = ns2;
-      nt = nt2;
     }
   }
+  return __fsub_rn(a, b);
 }
 
 // Words of the per-probe table: one sign bit per node, then two words for
@@ -133,13 +164,13 @@ __host__ __device__ __forceinline__ uint32_t table_words(uint32_t n) { return (n
 // pipelined: at step i the gather of X_{i+1} and the table read of X_i are
 // issued, and the term of X_{i-1} (whose table word was read one step
 // earlier) is added.  The additions keep step order, so the result equals
-// walk_pair's bit for bit.
+// walk_pair_visit's bit for bit.
 template <bool DEBUG, class GR>
 __device__ __forceinline__ float walk_pair_table(const GR& gr, uint32_t* visits, uint32_t walk_tag, const ZTable& zt,
                                                  int32_t s, int32_t t, int32_t L, uint64_t seed, uint64_t pair) {
   const int4 xs = gr.start(s), xt = gr.start(t);
-  float a = signed_term(zt.one((uint32_t)xs.x), (uint32_t)xs.w);
-  float b = signed_term(zt.one((uint32_t)xt.x), (uint32_t)xt.w);
+  float a = zt.term(zt.word((uint32_t)xs.x), (uint32_t)xs.x, (uint32_t)xs.w);
+  float b = zt.term(zt.word((uint32_t)xt.x), (uint32_t)xt.x, (uint32_t)xt.w);
   if (DEBUG) {
     atomicAdd(visits + xs.x, 1u);
     atomicAdd(visits + xt.x, 1u);
@@ -175,10 +206,10 @@ __device__ __forceinline__ float walk_pair_table(const GR& gr, uint32_t* visits,
         ns2 = gr.next(ns, wsw);
         nt2 = gr.next(nt, wtw);
       }
-      const uint32_t cs_word = zt.tab[(uint32_t)ns.x >> 5], ct_word = zt.tab[(uint32_t)nt.x >> 5];
+      const uint32_t cs_word = zt.word((uint32_t)ns.x), ct_word = zt.word((uint32_t)nt.x);
       if (pending) {
-        a = __fadd_rn(a, signed_term(zt.from_word(ps_word, ps_v), ps_inv));
-        b = __fadd_rn(b, signed_term(zt.from_word(pt_word, pt_v), pt_inv));
+        a = __fadd_rn(a, zt.term(ps_word, ps_v, ps_inv));
+        b = __fadd_rn(b, zt.term(pt_word, pt_v, pt_inv));
       }
       if (DEBUG) {
         atomicAdd(visits + ns.x, 1u);
@@ -192,8 +223,8 @@ __device__ __forceinline__ float walk_pair_table(const GR& gr, uint32_t* visits,
       pt_inv = (uint32_t)nt.w;
       pending = true;
       if (!more) {
-        a = __fadd_rn(a, signed_term(zt.from_word(ps_word, ps_v), ps_inv));
-        b = __fadd_rn(b, signed_term(zt.from_word(pt_word, pt_v), pt_inv));
+        a = __fadd_rn(a, zt.term(ps_word, ps_v, ps_inv));
+        b = __fadd_rn(b, zt.term(pt_word, pt_v, pt_inv));
         return __fsub_rn(a, b);
       }
       ns = ns2;
@@ -216,9 +247,8 @@ __device__ __forceinline__ void build_probe_table(const Probe& pr, uint32_t* tab
   while (w < nwords) {
     x = feistel_once(pr, x);
     if (x < n) {
-      const int z = probe_z_from_pi(pr, x);
-      if (z == 0) zero[x - pr.n_active] = v;
-      acc |= (uint32_t)(z < 0) << (v & 31u);
+      if (x >= pr.n_active) zero[x - pr.n_active] = v;  // its bit is not read
+      acc |= probe_negative(pr, x) << (v & 31u);
       ++v;
       if ((v & 31u) == 0 || v >= n) {
         tab[w] = acc;

@@ -1,0 +1,86 @@
+"""Edges of the kernels' work splits: the sizes at which a tile, a pool, a
+segment or a launch rule begins and ends, each against the oracle or against
+the form of the same call that takes the other path."""
+
+import numpy as np
+import pytest
+
+import oracle
+from pw_inputs import barabasi_albert, complete_graph, cycle_graph, er_cycle, query_seeds, uniform_pairs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pw():
+    from paper_2512_05460_gb300 import build
+
+    build.build()
+    from paper_2512_05460_gb300 import probewalk
+
+    probewalk.lib()
+    return probewalk
+
+
+# n = 5, 16: the 12-round permutation; 17: the smallest 8-round one; 33: n just
+# above 2^b / 2, where cycle-walks are longest; 65: odd, one zero node
+GRAPHS = [lambda: complete_graph(5), lambda: cycle_graph(16), lambda: complete_graph(17), lambda: er_cycle(33, 0.2, 3),
+          lambda: er_cycle(65, 0.1, 4)]
+
+
+@pytest.mark.parametrize("graph_fn", GRAPHS)
+def test_visit_pool_edges(pw, oracle_lib, graph_fn):
+    """Per-visit walks in warp pools of 4 visits a side: walk lengths around the
+    pool's, replica counts around a warp's, every U_p and visit against the oracle."""
+    host = graph_fn()
+    with pw.Graph(host.row_ptr, host.col_idx) as g:
+        for L in (0, 1, 2, 3, 4, 7, 8):
+            for R in (2, 31, 32, 33):
+                params = pw.make_params(budget_mode=pw.PW_BUDGET_FIXED, B=2, G=3, R=R, walk_mode=1)
+                cfg = oracle.budget_cfg(mode=oracle.MODE_FIXED, B=2, G=3, R=R)
+                dev = pw.pw_debug_query(g.handle, host.n, 0, 3, 0.3, L, 77 + L, params, q_cap=64, u_cap=4096,
+                                        want_visits=True)
+                orc = oracle.query(host, 0, 3, 0.3, L, 77 + L, cfg, want_q=True, want_u=True, want_visits=True)
+                np.testing.assert_array_equal(dev["u"], orc["u"])
+                np.testing.assert_array_equal(dev["visits"], orc["visits"])
+                np.testing.assert_array_equal(dev["q"], orc["q"])
+                assert dev["beta"] == orc["beta"]
+                assert pw.pw_query(g.handle, 0, 3, 0.3, L, 77 + L, params) == orc["beta"]
+
+
+@pytest.mark.parametrize("mode", ["pilot", "fixed", "adaptive"])
+def test_plans_across_the_fused_launch(pw, oracle_lib, mode):
+    """Up to 256 queries are planned and scanned in one launch, more in two; a
+    batch of either kind gives each query, the invalid ones among them, what it
+    gets in smaller batches."""
+    host = er_cycle(200, 8 / 199, 0)
+    budget = {"pilot": {}, "fixed": {"budget_mode": pw.PW_BUDGET_FIXED, "B": 2, "G": 3, "R": 5},
+              "adaptive": {"budget_mode": pw.PW_BUDGET_ADAPTIVE}}[mode]
+    params = pw.make_params(**budget)
+    count = 1100  # more than one query per thread of the scan
+    s, t = uniform_pairs(host.n, count, 7)
+    seeds = query_seeds(count, 8)
+    eps = np.full(count, 0.45)
+    t[5], s[300] = s[5], -1
+    eps[256] = 2.0
+    with pw.Graph(host.row_ptr, host.col_idx) as g:
+        whole, st = pw.pw_query_batch(g.handle, s, t, eps, 9, seeds, params)
+        assert st[300] == st[256] == pw.PW_ERR_ARG and np.count_nonzero(st) == 2 and whole[5] == 0.0
+        for lo, hi in ((0, 1), (1, 33), (33, 289), (289, 546), (546, 1100)):
+            part, pst = pw.pw_query_batch(g.handle, s[lo:hi], t[lo:hi], eps[lo:hi], 9, seeds[lo:hi], params)
+            np.testing.assert_array_equal(part, whole[lo:hi])
+            np.testing.assert_array_equal(pst, st[lo:hi])
+    if mode == "pilot":
+        want, _, _ = oracle.query_many(host, s[:4], t[:4], 0.45, 9, seeds[:4])
+        np.testing.assert_array_equal(whole[:4], want)
+
+
+@pytest.mark.parametrize("G", [1, 2, 5, 24, 129, 300])
+def test_median_by_rank(pw, oracle_lib, G):
+    """Even and odd block counts below and above the block's 128 threads."""
+    host = barabasi_albert(400, 3, 5)
+    params = pw.make_params(budget_mode=pw.PW_BUDGET_FIXED, B=9, G=G, R=3)
+    cfg = oracle.budget_cfg(mode=oracle.MODE_FIXED, B=9, G=G, R=3)
+    with pw.Graph(host.row_ptr, host.col_idx) as g:
+        for s, t in ((1, 2), (0, 399)):
+            assert pw.pw_query(g.handle, s, t, 0.3, 6, 5, params) == oracle.query(host, s, t, 0.3, 6, 5, cfg)["beta"]
