@@ -86,6 +86,14 @@ struct GraphCache {
   uint64_t launches = 0;  // kernel launches in one replay
 };
 
+// Layout of the series steps on a graph: its heavy rows' segments, built by the
+// first pw_series_batch, and scratch kept between calls.
+struct SeriesPlan {
+  DeviceBuffer segs, heavy, arrived, scratch;
+  int32_t nseg = 0, nheavy = 0;
+  bool ready = false;
+};
+
 struct Workspace {
   DeviceBuffer plans, pilot_plans, tile_prefix, pilot_s, acc, q, totals, counters, queries, results, u_debug;
   Totals* host_totals = nullptr;  // pinned: totals of the latest batch (valid once last_use has completed)
@@ -130,6 +138,7 @@ struct pw_graph {
   pw::GraphCache gcache;
   pw::Workspace ws;
   pw::ProfileState prof;
+  pw::SeriesPlan series;
 };
 
 namespace pw {

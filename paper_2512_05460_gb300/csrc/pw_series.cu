@@ -9,14 +9,21 @@
 // error-free transformations (TwoSum, and TwoProd by fused multiply-add), each
 // a handful of FP32 operations; the final reduction to beta is FP64.
 //
-// 32 queries per pass, one warp lane per query column.  x, y and h are n x 32
-// row-major (a node's 32 pairs are one 256-byte row), so gathering x over a
-// node's neighbours reads whole lines.  Iteration i adds x_i to h and forms
-// x_{i+1} = P x_i with (P x)_v = (sum_{u in N(v)} x_u) * (1/d_v), neighbours
-// read from col_idx (4 bytes per entry).  Rows of at most 1024
-// entries take one warp each and add in CSR order; longer rows (the hubs of
-// power-law graphs) are cut into 1024-entry segments whose partial sums are
-// added in segment order, so one hub does not hold up a whole step.
+// C = 4, 8, 16 or 32 queries per pass (the fewest columns that hold what is left
+// of a group of equal L), one warp lane per query column and 32 / C rows per
+// warp.  x, y and h are n x C row-major, so gathering x over a node's neighbours
+// reads whole sectors (C = 32: two lines a row).  Iteration i forms x_{i+1} =
+// P x_i with (P x)_v = (sum_{u in N(v)} x_u) * (1/d_v), neighbours read from
+// col_idx (4 bytes per entry); every second iteration adds x_i and x_{i+1} to h,
+// which halves the traffic of h.
+//
+// Rows of at most 64 entries take one warp's lanes and add in CSR order; longer
+// rows are cut into segments of 64 or of about the root of their degree, whose
+// partial sums are added in segment order by the warp that finishes the row's
+// last one.  An addition of pairs is a chain of about 50 clocks, so a row's
+// length is its latency: with 1024-entry segments, and the heavy rows in two
+// launches after the light ones, a step on a 10^5-node power-law graph waited
+// 155 us for its two hubs where all other rows took 20.
 #include <math.h>
 #include <string.h>
 
@@ -29,8 +36,13 @@
 
 namespace pw {
 
-constexpr int kSeriesCols = 32;
-constexpr int32_t kSeriesSegEdges = 1024;  // rows with more entries are split into segments of this size
+constexpr int kSeriesCols = 32;       // most queries per pass
+constexpr int32_t kSeriesRow = 64;    // rows with more entries are cut into segments
+constexpr int64_t kSeriesSegment = 64;  // entries of a segment, or about the root of the row's if more
+constexpr int kSeriesThreads = 256;
+// Scratch up to this size stays with the graph until it is freed (cudaMalloc and
+// cudaFree wait for the device); larger is allocated and freed by each call.
+constexpr size_t kSeriesKeptBytes = (size_t)256 << 20;
 
 // ---- double-float arithmetic (value = hi + lo) -----------------------------
 // TwoSum (Knuth): s + e == a + b exactly.
@@ -69,30 +81,15 @@ __device__ __forceinline__ float2 df_from_double(double v) {
   return make_float2(hi, __double2float_rn(v - (double)hi));
 }
 
-__global__ void series_init_kernel(float2* __restrict__ x, float2* __restrict__ h, uint32_t n) {
-  const size_t total = (size_t)n * kSeriesCols;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    x[i] = make_float2(0.f, 0.f);
-    h[i] = make_float2(0.f, 0.f);
-  }
-}
-
-// Per-pass control block, written by the host before each pass (so one
-// captured graph serves every pass of the same L).
-struct SeriesCtl {
-  int2 st[kSeriesCols];  // (s, t) of each column
-  int32_t ncols;
-  int32_t pad;
-};
-
-__global__ void series_seed_kernel(float2* __restrict__ x, const SeriesCtl* __restrict__ ctl,
+// Start vectors D^{-1} (e_s - e_t) of a pass, into zeroed x.
+__global__ void series_seed_kernel(float2* __restrict__ x, const int2* __restrict__ st, int ncols, int cols,
                                    const int4* __restrict__ node) {
   const int c = threadIdx.x;
-  if (c >= ctl->ncols) return;
-  const int s = ctl->st[c].x, t = ctl->st[c].y;
+  if (c >= ncols) return;
+  const int s = st[c].x, t = st[c].y;
   if (s == t) return;
-  x[(size_t)s * kSeriesCols + c] = df_from_double(1.0 / (double)node[s].z);
-  x[(size_t)t * kSeriesCols + c] = df_from_double(-1.0 / (double)node[t].z);
+  x[(size_t)s * cols + c] = df_from_double(1.0 / (double)node[s].z);
+  x[(size_t)t * cols + c] = df_from_double(-1.0 / (double)node[t].z);
 }
 
 // 1/d_v as a pair, once per call.
@@ -101,115 +98,291 @@ __global__ void series_inv_degree_kernel(const int4* __restrict__ node, float2* 
     inv[v] = df_from_double(1.0 / (double)__ldg(&node[v].z));
 }
 
-// Sum of x_u (column = lane) over the neighbour entries [e0, e1) of one row,
-// added in CSR order.  A warp loads 32 neighbour ids with one coalesced load
-// and keeps 8 row loads in flight before adding them in order.
+struct SeriesArgs {
+  const float2* x;
+  float2* y;
+  float2* h;
+  const int32_t* col;
+  const int4* node;
+  const float2* inv;
+  const int4* segs;       // {heavy row, e_begin, e_end, partial slot}
+  const int4* heavy;      // {row, first partial slot, partial count, -}
+  float2* partial;        // nseg x C
+  unsigned int* arrived;  // per heavy row: segments done in this step (wraps to 0)
+  uint32_t n;
+  int32_t nseg;
+};
+
+// Sum of many pairs: the high parts by TwoSum, their errors and the low parts
+// in FP32 sums of their own, normalised now and then (fold) and at the end.  8
+// operations a pair and a chain of one addition, against df_add's 20 and a
+// chain of 12; the roundings are 2^-25 of sums of terms 2^-25 of the first, as
+// df_add's are.
+struct PairSum {
+  float hi = 0.f, err = 0.f, low = 0.f;
+  __device__ __forceinline__ void add(float2 v) {
+    float s, e;
+    two_sum(hi, v.x, s, e);
+    hi = s;
+    err = __fadd_rn(err, e);
+    low = __fadd_rn(low, v.y);
+  }
+  __device__ __forceinline__ void fold() {
+    const float t = __fadd_rn(err, low);
+    float s;
+    two_sum(hi, t, s, low);
+    hi = s;
+    err = 0.f;
+  }
+  __device__ __forceinline__ float2 value() {
+    fold();
+    return make_float2(hi, low);
+  }
+};
+
+// The first C neighbour ids of a row of len entries, one per lane of its part.
+template <int C>
+__device__ __forceinline__ int32_t series_ids(const int32_t* __restrict__ col, int32_t e0, int32_t len, uint32_t sub) {
+  return (int32_t)sub < len ? __ldg(col + e0 + (int32_t)sub) : 0;
+}
+
+// Sum of x_u (column = lane mod C) over the entries [e0, e0 + len) of one row,
+// in CSR order; every lane of the warp calls, 32 / C rows at once.  `mine`: the
+// row's first ids (series_ids), the next C come with one coalesced load; up to 8
+// row loads are in flight.  Rows shorter than the warp's longest add zeros,
+// which leaves a sum unchanged.
+template <int C>
 __device__ __forceinline__ float2 series_row_sum(const float2* __restrict__ x, const int32_t* __restrict__ col,
-                                                 int32_t e0, int32_t e1, uint32_t lane) {
-  float2 acc = make_float2(0.f, 0.f);
-  for (int32_t b = e0; b < e1; b += 32) {
-    const int cnt = e1 - b < 32 ? e1 - b : 32;
-    const int u_l = (int)lane < cnt ? __ldg(&col[b + (int)lane]) : 0;
-    int j = 0;
-    for (; j + 8 <= cnt; j += 8) {
+                                                 int32_t mine, int32_t e0, int32_t len, uint32_t sub) {
+  PairSum acc;
+  const int32_t longest = C == 32 ? len : __reduce_max_sync(0xffffffffu, len);
+  for (int32_t b = 0; b < longest; b += C) {
+    const int32_t cnt = len - b;
+    const int32_t lim = longest - b < C ? longest - b : C;  // the same in the whole warp
+    const int32_t next = b + C < longest ? series_ids<C>(col, e0 + b + C, cnt - C, sub) : 0;
+    for (int32_t j = 0; j < lim; j += 8) {
       float2 v[8];
+      auto load = [&](int q) {
+        const int32_t u = __shfl_sync(0xffffffffu, mine, j + q, C);
+        v[q] = j + q < cnt ? __ldg(x + (size_t)(uint32_t)u * C + sub) : make_float2(0.f, 0.f);
+      };
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int u = __shfl_sync(0xffffffffu, u_l, j + q);
-        v[q] = __ldg(x + (size_t)u * kSeriesCols + lane);
+      for (int q = 0; q < 4; ++q) load(q);
+      const bool more = C > 4 && j + 4 < lim;
+      if (more) {
+#pragma unroll
+        for (int q = 4; q < 8; ++q) load(q);
       }
 #pragma unroll
-      for (int q = 0; q < 8; ++q) acc = df_add(acc, v[q]);
+      for (int q = 0; q < 4; ++q) acc.add(v[q]);
+      if (more) {
+#pragma unroll
+        for (int q = 4; q < 8; ++q) acc.add(v[q]);
+      }
+      if (j + 8 < lim) acc.fold();
     }
-    for (; j < cnt; ++j) {
-      const int u = __shfl_sync(0xffffffffu, u_l, j);
-      acc = df_add(acc, __ldg(x + (size_t)u * kSeriesCols + lane));
+    if (b + C < longest) acc.fold();
+    mine = next;
+  }
+  return acc.value();
+}
+
+// One iteration over all rows.  ACC: 0 leaves h, 1 adds x_i and then x_{i+1},
+// 2 starts h as their sum.  The segments of heavy rows come first.
+// Bound by the latency of a row's loads on graphs in L2 and by L2 and HBM
+// bandwidth beyond; 5 blocks per SM (48 registers) against 4 (58) or 6 (40): 268,
+// 388 and 307 us a step on a 1000^2 grid.  Microseconds a step, before -> now:
+// 10^5-node power-law graph, 32 / 16 / 4 columns 168 -> 47 / 175 -> 29 / 168 ->
+// 19; R-MAT 2^20, 32 / 8 columns 1,498 -> 1,244 / 1,499 -> 377; 2000^2 grid, 32
+// columns 1,540 -> 1,142.
+template <int C, int ACC>
+__global__ void __launch_bounds__(kSeriesThreads, 5) series_step_kernel(SeriesArgs A) {
+  constexpr uint32_t kRows = 32 / C;
+  const uint32_t lane = threadIdx.x & 31u, sub = lane % C, part = lane / C;
+  const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
+  const uint32_t seg_groups = ((uint32_t)A.nseg + kRows - 1) / kRows;
+  const uint32_t row_groups = (A.n + kRows - 1) / kRows;
+  const float2 zero = make_float2(0.f, 0.f);
+  auto finish = [&](size_t at, float2 sum, float2 inv, float2 x, float2 h) {
+    const float2 y = df_mul(sum, inv);
+    A.y[at] = y;
+    if (ACC == 1) A.h[at] = df_add(df_add(h, x), y);
+    if (ACC == 2) A.h[at] = df_add(x, y);
+  };
+  uint32_t g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  for (; g < seg_groups; g += warps) {
+    const uint32_t i = g * kRows + part;
+    const bool valid = i < (uint32_t)A.nseg;
+    const int4 sg = valid ? __ldg(A.segs + i) : make_int4(0, 0, 0, 0);
+    const int32_t len = sg.z - sg.y;
+    const float2 sum = series_row_sum<C>(A.x, A.col, series_ids<C>(A.col, sg.y, len, sub), sg.y, len, sub);
+    if (valid) __stcg(A.partial + (size_t)sg.w * C + sub, sum);
+    __threadfence();
+    __syncwarp();
+    const int4 hr = valid ? __ldg(A.heavy + sg.x) : make_int4(0, 0, 0, 0);
+    unsigned int before = 0;
+    if (valid && sub == 0) before = atomicInc(A.arrived + sg.x, (unsigned int)hr.z - 1u);
+    before = __shfl_sync(0xffffffffu, before, part * C);
+    if (valid && before + 1u == (unsigned int)hr.z) {
+      __threadfence();
+      const size_t at = (size_t)(uint32_t)hr.x * C + sub;
+      const float2 inv = __ldg(A.inv + hr.x), x = ACC ? A.x[at] : zero, h = ACC == 1 ? A.h[at] : zero;
+      PairSum acc;
+      const float2* p = A.partial + (size_t)hr.y * C + sub;
+      int32_t k = 0;
+      for (; k + 8 <= hr.z; k += 8) {
+        float2 v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = __ldcg(p + (size_t)(k + q) * C);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) acc.add(v[q]);
+        acc.fold();
+      }
+      for (; k < hr.z; ++k) acc.add(__ldcg(p + (size_t)k * C));
+      finish(at, acc.value(), inv, x, h);
     }
+    __syncwarp();
   }
-  return acc;
-}
-
-// Rows of degree <= kSeriesSegEdges, one warp per row (grid-stride, the next
-// row's record fetched while this one is summed):
-// h_v += x_v; y_v = (sum over neighbours of x_u) * (1/d_v).  Heavier rows
-// are left to the segment kernels below.
-__global__ void __launch_bounds__(256) series_light_kernel(const float2* __restrict__ x, float2* __restrict__ y,
-                                                           float2* __restrict__ h, const int32_t* __restrict__ col,
-                                                           const int4* __restrict__ node,
-                                                           const float2* __restrict__ inv, uint32_t n, int last) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-  uint32_t v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int4 nv = v < n ? __ldg(node + v) : make_int4(0, 0, 0, 0);
-  for (; v < n; v += warps) {
-    const uint32_t vn = v + warps;
-    const int4 nv_next = vn < n ? __ldg(node + vn) : make_int4(0, 0, 0, 0);  // in flight during this row
-    if (nv.z <= kSeriesSegEdges) {
-      const size_t row = (size_t)v * kSeriesCols + lane;
-      h[row] = df_add(h[row], x[row]);
-      if (!last) y[row] = df_mul(series_row_sum(x, col, nv.y, nv.y + nv.z, lane), __ldg(inv + v));
-    }
-    nv = nv_next;
-  }
-}
-
-// One warp per segment of a heavy row: the partial sum of its entries.
-__global__ void __launch_bounds__(256) series_segment_kernel(const float2* __restrict__ x,
-                                                             float2* __restrict__ partial,
-                                                             const int32_t* __restrict__ col,
-                                                             const int4* __restrict__ segs, int32_t nseg) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-  for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < (uint32_t)nseg; i += warps) {
-    const int4 sg = __ldg(segs + i);  // {row, e_begin, e_end, partial slot}
-    partial[(size_t)sg.w * kSeriesCols + lane] = series_row_sum(x, col, sg.y, sg.z, lane);
+  // A row's own values are loaded before its neighbours', its first neighbour
+  // ids one row ahead and its record two rows ahead.
+  g -= seg_groups;
+  uint32_t v = g * kRows + part;
+  const uint32_t step = warps * kRows;
+  auto record = [&](uint32_t u) {  // {row start, entries}; rows of other warps and heavy ones have none
+    const int4 r = u < A.n ? __ldg(A.node + u) : make_int4(0, 0, 0, 0);
+    return make_int2(r.y, u < A.n ? (r.z <= kSeriesRow ? r.z : -1) : -1);
+  };
+  int2 r0 = record(v), r1 = record(v + step);
+  int32_t ids = series_ids<C>(A.col, r0.x, r0.y, sub);
+  for (; g < row_groups; g += warps) {
+    const bool light = r0.y >= 0;
+    const size_t at = (size_t)v * C + sub;
+    const float2 inv = light ? __ldg(A.inv + v) : zero;
+    const float2 x = ACC && light ? A.x[at] : zero, h = ACC == 1 && light ? A.h[at] : zero;
+    const int32_t ids_next = series_ids<C>(A.col, r1.x, r1.y, sub);
+    const int2 r2 = record(v + 2 * step);
+    const float2 sum = series_row_sum<C>(A.x, A.col, ids, r0.x, light ? r0.y : 0, sub);
+    if (light) finish(at, sum, inv, x, h);
+    r0 = r1;
+    r1 = r2;
+    ids = ids_next;
+    v += step;
   }
 }
 
-// One warp per heavy row: h_v += x_v; y_v = (partials in segment order) * (1/d_v).
-__global__ void __launch_bounds__(256) series_heavy_finish_kernel(const float2* __restrict__ x,
-                                                                  float2* __restrict__ y, float2* __restrict__ h,
-                                                                  const float2* __restrict__ partial,
-                                                                  const int4* __restrict__ rows, int32_t nrows,
-                                                                  const float2* __restrict__ inv, int last) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-  for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < (uint32_t)nrows; i += warps) {
-    const int4 hr = __ldg(rows + i);  // {row, first partial slot, partial count, -}
-    const size_t row = (size_t)hr.x * kSeriesCols + lane;
-    h[row] = df_add(h[row], x[row]);
-    if (last) continue;
-    float2 acc = make_float2(0.f, 0.f);
-    for (int32_t p = 0; p < hr.z; ++p) acc = df_add(acc, partial[(size_t)(hr.y + p) * kSeriesCols + lane]);
-    y[row] = df_mul(acc, __ldg(inv + hr.x));
-  }
-}
-
-// Per column: sum of h^2 and of h over nodes in FP64 (fixed order: per-thread
-// strided partial sums, then a shared-memory tree), then beta = sq - tot^2 / n.
-__global__ void series_reduce_kernel(const float2* __restrict__ h, uint32_t n, const SeriesCtl* __restrict__ ctl,
-                                     double* __restrict__ out) {
-  __shared__ double ssq[256], stot[256];
-  const int c = blockIdx.x;
-  if (c >= ctl->ncols) return;
+// beta of each column: sums of h^2 and of h over the nodes in FP64, then
+// sq - tot^2 / n.  h is A.h (use_h) plus A.x (use_x: the last x when its step
+// did not add it).  Every block sums its rows and a tree its threads; the last
+// block adds the blocks' sums, each in a fixed order.
+template <int C>
+__global__ void __launch_bounds__(8 * C) series_reduce_kernel(const float2* __restrict__ h,
+                                                                       const float2* __restrict__ x, int use_h,
+                                                                       int use_x, uint32_t n, int ncols,
+                                                                       double* block_sums, unsigned int* arrived,
+                                                                       double* __restrict__ out) {
+  constexpr uint32_t kRows = 8;  // rows at once per block, for every C: the order of the sums is the same
+  __shared__ double ssq[kRows * C], stot[kRows * C];
+  __shared__ bool last;
+  const uint32_t tid = threadIdx.x, c = tid % C;
   double sq = 0.0, tot = 0.0;
-  for (uint32_t v = threadIdx.x; v < n; v += blockDim.x) {
-    const float2 p = h[(size_t)v * kSeriesCols + c];
-    const double x = (double)p.x + (double)p.y;
-    sq += x * x;
-    tot += x;
+  for (uint64_t v = (uint64_t)blockIdx.x * kRows + tid / C; v < n; v += (uint64_t)gridDim.x * kRows) {
+    const size_t at = (size_t)v * C + c;
+    float2 p = use_h ? h[at] : make_float2(0.f, 0.f);
+    if (use_x) p = use_h ? df_add(p, x[at]) : x[at];
+    const double d = (double)p.x + (double)p.y;
+    sq += d * d;
+    tot += d;
   }
-  ssq[threadIdx.x] = sq;
-  stot[threadIdx.x] = tot;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) {
-      ssq[threadIdx.x] += ssq[threadIdx.x + w];
-      stot[threadIdx.x] += stot[threadIdx.x + w];
-    }
+  auto tree = [&]() {
+    ssq[tid] = sq;
+    stot[tid] = tot;
     __syncthreads();
+    for (uint32_t w = kRows * C / 2; w >= (uint32_t)C; w >>= 1) {
+      if (tid < w) {
+        ssq[tid] += ssq[tid + w];
+        stot[tid] += stot[tid + w];
+      }
+      __syncthreads();
+    }
+  };
+  tree();
+  if (tid < (uint32_t)C) {
+    __stcg(block_sums + ((size_t)blockIdx.x * C + c) * 2, ssq[tid]);
+    __stcg(block_sums + ((size_t)blockIdx.x * C + c) * 2 + 1, stot[tid]);
   }
-  if (threadIdx.x == 0) out[c] = ssq[0] - stot[0] * stot[0] / (double)n;
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) last = atomicInc(arrived, gridDim.x - 1u) + 1u == gridDim.x;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  sq = tot = 0.0;
+  for (uint32_t b = tid / C; b < gridDim.x; b += kRows) {
+    sq += __ldcg(block_sums + ((size_t)b * C + c) * 2);
+    tot += __ldcg(block_sums + ((size_t)b * C + c) * 2 + 1);
+  }
+  tree();
+  if ((int)tid < ncols) out[tid] = ssq[tid] - stot[tid] * stot[tid] / (double)n;
+}
+
+using SeriesStepFn = void (*)(SeriesArgs);
+template <int C>
+static SeriesStepFn series_step_fn(int acc) {
+  return acc == 0 ? series_step_kernel<C, 0> : (acc == 1 ? series_step_kernel<C, 1> : series_step_kernel<C, 2>);
+}
+
+// One pass of `ncols` <= C queries of equal L, enqueued on `stream`; returns
+// the number of kernels.  x_buf and y_buf alternate.
+template <int C>
+static int series_pass(SeriesArgs A, float2* x_buf, float2* y_buf, const int2* st, int ncols, int32_t L, int grid,
+                       int reduce_grid, double* block_sums, unsigned int* reduce_arrived, double* out,
+                       cudaStream_t stream) {
+  cudaMemsetAsync(x_buf, 0, sizeof(float2) * (size_t)A.n * C, stream);
+  series_seed_kernel<<<1, kSeriesCols, 0, stream>>>(x_buf, st, ncols, C, A.node);
+  float2 *x = x_buf, *y = y_buf;
+  for (int32_t i = 0; i < L; ++i) {
+    A.x = x;
+    A.y = y;
+    series_step_fn<C>((i & 1) ? 0 : (i == 0 ? 2 : 1))<<<grid, kSeriesThreads, 0, stream>>>(A);
+    std::swap(x, y);
+  }
+  series_reduce_kernel<C><<<reduce_grid, 8 * C, 0, stream>>>(A.h, x, L > 0, (L & 1) == 0, A.n, ncols,
+                                                                      block_sums, reduce_arrived, out);
+  return L + 2;
+}
+
+// Heavy rows' segments, laid out once per graph (they depend on its degrees only).
+static pw_status series_plan(pw_graph* g) {
+  SeriesPlan& P = g->series;
+  if (P.ready) return PW_OK;
+  std::vector<int4> segs, heavy;
+  int64_t start = 0;
+  int32_t slot = 0;
+  for (int64_t v = 0; v < g->n; ++v) {
+    const int32_t d = g->deg[(size_t)v];
+    if (d > kSeriesRow) {
+      int64_t size = kSeriesSegment;
+      while (size * size < d) size *= 2;
+      const int32_t first = slot;
+      for (int64_t e = start; e < start + d; e += size)
+        segs.push_back(make_int4((int)heavy.size(), (int)e, (int)std::min<int64_t>(e + size, start + d), slot++));
+      heavy.push_back(make_int4((int)v, first, slot - first, 0));
+    }
+    start += d;
+  }
+  pw_status st;
+  if ((st = ensure_buffer(P.segs, sizeof(int4) * segs.size())) != PW_OK) return st;
+  if ((st = ensure_buffer(P.heavy, sizeof(int4) * heavy.size())) != PW_OK) return st;
+  if ((st = ensure_buffer(P.arrived, sizeof(unsigned int) * (heavy.size() + 1))) != PW_OK) return st;
+  PW_CUDA_TRY(cudaMemcpyAsync(P.segs.ptr, segs.data(), sizeof(int4) * segs.size(), cudaMemcpyHostToDevice, g->stream));
+  PW_CUDA_TRY(cudaMemcpyAsync(P.heavy.ptr, heavy.data(), sizeof(int4) * heavy.size(), cudaMemcpyHostToDevice,
+                              g->stream));
+  PW_CUDA_TRY(cudaMemsetAsync(P.arrived.ptr, 0, sizeof(unsigned int) * (heavy.size() + 1), g->stream));
+  PW_CUDA_TRY(cudaStreamSynchronize(g->stream));
+  P.nseg = (int32_t)segs.size();
+  P.nheavy = (int32_t)heavy.size();
+  P.ready = true;
+  return PW_OK;
 }
 
 }  // namespace pw
@@ -228,151 +401,101 @@ extern "C" pw_status pw_series_batch(pw_graph* g, int64_t count, const int64_t* 
   std::lock_guard<std::mutex> guard(g->lock);
   PW_CUDA_TRY(cudaSetDevice(g->device));
   const size_t n = (size_t)g->n;
-  const size_t bytes = sizeof(float2) * n * kSeriesCols;
-  // rows of more than kSeriesSegEdges entries: segments {row, e_begin, e_end,
-  // partial slot} and rows {row, first slot, slot count}, in CSR order
-  std::vector<int4> segs, heavy;
-  {
-    int64_t start = 0;
-    int32_t slot = 0;
-    for (int64_t v = 0; v < g->n; ++v) {
-      const int32_t d = g->deg[(size_t)v];
-      if (d > kSeriesSegEdges) {
-        const int32_t first = slot;
-        for (int64_t e = start; e < start + d; e += kSeriesSegEdges) {
-          const int64_t e1 = std::min<int64_t>(e + kSeriesSegEdges, start + d);
-          segs.push_back(make_int4((int)v, (int)e, (int)e1, slot++));
-        }
-        heavy.push_back(make_int4((int)v, first, slot - first, 0));
-      }
-      start += d;
-    }
-  }
-  DeviceBuffer xb, yb, hb, sb, ob, segb, rowb, partb, invb;
-  pw_status st;
-  auto release = [&]() {
-    free_buffer(xb);
-    free_buffer(yb);
-    free_buffer(hb);
-    free_buffer(sb);
-    free_buffer(ob);
-    free_buffer(segb);
-    free_buffer(rowb);
-    free_buffer(partb);
-    free_buffer(invb);
-  };
-  if ((st = ensure_buffer(xb, bytes)) != PW_OK || (st = ensure_buffer(yb, bytes)) != PW_OK ||
-      (st = ensure_buffer(hb, bytes)) != PW_OK || (st = ensure_buffer(sb, sizeof(SeriesCtl))) != PW_OK ||
-      (st = ensure_buffer(ob, sizeof(double) * kSeriesCols)) != PW_OK ||
-      (st = ensure_buffer(invb, sizeof(float2) * n)) != PW_OK ||
-      (!segs.empty() && ((st = ensure_buffer(segb, sizeof(int4) * segs.size())) != PW_OK ||
-                         (st = ensure_buffer(rowb, sizeof(int4) * heavy.size())) != PW_OK ||
-                         (st = ensure_buffer(partb, sizeof(float2) * kSeriesCols * segs.size())) != PW_OK))) {
-    release();
-    return st;
-  }
   cudaStream_t stream = g->stream;
-  const int threads = 256;
-  int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, series_light_kernel, threads, 0) != cudaSuccess || occ < 1)
-    occ = 1;
-  const int grid = g->sm_count * occ;
-  const int32_t nseg = (int32_t)segs.size(), nheavy = (int32_t)heavy.size();
-  const int seg_grid = (int)std::min<int64_t>((int64_t)grid, ((int64_t)nseg * 32 + threads - 1) / threads);
-  const int heavy_grid = (int)std::min<int64_t>((int64_t)grid, ((int64_t)nheavy * 32 + threads - 1) / threads);
-  cudaError_t e = cudaSuccess;
-  const float2* inv = (const float2*)invb.ptr;
-  series_inv_degree_kernel<<<grid, threads, 0, stream>>>(g->d_node, (float2*)invb.ptr, (uint32_t)n);
-  count_launch();
-  if (nseg > 0) {
-    e = cudaMemcpyAsync(segb.ptr, segs.data(), sizeof(int4) * segs.size(), cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(rowb.ptr, heavy.data(), sizeof(int4) * heavy.size(), cudaMemcpyHostToDevice, stream);
-  }
-  // One pass (init, seed, L + 1 steps, reduce) enqueued on the stream; returns
-  // the number of kernels.  A pass of L + 1 steps is one to three launches
-  // per step, so it is captured once per distinct L as a CUDA graph and the
-  // graph is replayed for every 32-query group of that L.
-  const SeriesCtl* ctl_d = (const SeriesCtl*)sb.ptr;
-  auto enqueue_pass = [&](int32_t Lc) -> int {
-    int kernels = 0;
-    float2* x = (float2*)xb.ptr;
-    float2* y = (float2*)yb.ptr;
-    float2* h = (float2*)hb.ptr;
-    series_init_kernel<<<grid, threads, 0, stream>>>(x, h, (uint32_t)n);
-    series_seed_kernel<<<1, kSeriesCols, 0, stream>>>(x, ctl_d, g->d_node);
-    kernels += 2;
-    for (int32_t i = 0; i <= Lc; ++i) {
-      const int last = i == Lc;
-      series_light_kernel<<<grid, threads, 0, stream>>>(x, y, h, g->d_col, g->d_node, inv, (uint32_t)n, last);
-      ++kernels;
-      if (nheavy > 0) {
-        if (!last) {
-          series_segment_kernel<<<seg_grid, threads, 0, stream>>>(x, (float2*)partb.ptr, g->d_col,
-                                                                  (const int4*)segb.ptr, nseg);
-          ++kernels;
-        }
-        series_heavy_finish_kernel<<<heavy_grid, threads, 0, stream>>>(x, y, h, (const float2*)partb.ptr,
-                                                                       (const int4*)rowb.ptr, nheavy, inv, last);
-        ++kernels;
-      }
-      std::swap(x, y);
-    }
-    series_reduce_kernel<<<kSeriesCols, 256, 0, stream>>>(h, (uint32_t)n, ctl_d, (double*)ob.ptr);
-    return kernels + 1;
-  };
-  cudaGraphExec_t exec = nullptr;
-  int32_t exec_L = -1;
-  int exec_kernels = 0;
+  pw_status st = series_plan(g);
+  if (st != PW_OK) return st;
+  SeriesPlan& P = g->series;
   // queries with the same L share a pass: group by L in input order
   std::vector<int64_t> order((size_t)count);
   for (int64_t i = 0; i < count; ++i) order[(size_t)i] = i;
   std::stable_sort(order.begin(), order.end(), [&](int64_t a, int64_t b) { return L[a] < L[b]; });
-  for (size_t pos = 0; pos < order.size() && e == cudaSuccess;) {
-    const int32_t Lc = L[order[pos]];
-    SeriesCtl ctl;
-    memset(&ctl, 0, sizeof ctl);
-    std::vector<int64_t> idx;
-    while (pos < order.size() && ctl.ncols < kSeriesCols && L[order[pos]] == Lc) {
-      const int64_t i = order[pos++];
-      ctl.st[ctl.ncols++] = make_int2((int)s[i], (int)t[i]);
-      idx.push_back(i);
-    }
-    e = cudaMemcpyAsync(sb.ptr, &ctl, sizeof ctl, cudaMemcpyHostToDevice, stream);
+  struct Pass {
+    size_t begin;
+    int ncols, cols;
+  };
+  std::vector<Pass> passes;
+  int most = 0;  // columns of the widest pass
+  for (size_t pos = 0; pos < order.size();) {
+    size_t end = pos;
+    while (end < order.size() && end - pos < (size_t)kSeriesCols && L[order[end]] == L[order[pos]]) ++end;
+    const int ncols = (int)(end - pos);
+    const int cols = ncols <= 4 ? 4 : (ncols <= 8 ? 8 : (ncols <= 16 ? 16 : 32));
+    passes.push_back({pos, ncols, cols});
+    most = std::max(most, cols);
+    pos = end;
+  }
+  int occ = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, series_step_kernel<32, 1>, kSeriesThreads, 0) != cudaSuccess ||
+      occ < 1)
+    occ = 1;
+  const int reduce_grid = g->sm_count * 4;
+  // x, y, h, 1/d, partial sums, the reduction's block sums, (s, t) and results
+  auto align = [](size_t b) { return (b + 255) & ~(size_t)255; };
+  const size_t b_vec = align(sizeof(float2) * n * (size_t)most), b_inv = align(sizeof(float2) * n);
+  const size_t b_part = align(sizeof(float2) * (size_t)most * (size_t)P.nseg);
+  const size_t b_sums = align(sizeof(double) * 2 * (size_t)most * (size_t)reduce_grid);
+  const size_t b_st = align(sizeof(int2) * (size_t)count), b_out = align(sizeof(double) * (size_t)count);
+  const size_t bytes = 3 * b_vec + b_inv + b_part + b_sums + b_st + b_out;
+  DeviceBuffer own;
+  DeviceBuffer& buf = bytes <= kSeriesKeptBytes ? P.scratch : own;
+  if ((st = ensure_buffer(buf, bytes)) != PW_OK) return st;
+  char* at = (char*)buf.ptr;
+  auto take = [&](size_t b) {
+    char* p = at;
+    at += b;
+    return p;
+  };
+  float2* xb = (float2*)take(b_vec);
+  float2* yb = (float2*)take(b_vec);
+  SeriesArgs A;
+  memset(&A, 0, sizeof A);
+  A.h = (float2*)take(b_vec);
+  float2* inv = (float2*)take(b_inv);
+  A.partial = (float2*)take(b_part);
+  double* sums = (double*)take(b_sums);
+  int2* d_st = (int2*)take(b_st);
+  double* d_out = (double*)take(b_out);
+  A.inv = inv;
+  A.col = g->d_col;
+  A.node = g->d_node;
+  A.segs = (const int4*)P.segs.ptr;
+  A.heavy = (const int4*)P.heavy.ptr;
+  A.arrived = (unsigned int*)P.arrived.ptr;
+  unsigned int* reduce_arrived = A.arrived + P.nheavy;
+  A.n = (uint32_t)n;
+  A.nseg = P.nseg;
+  std::vector<int2> h_st((size_t)count);
+  for (size_t j = 0; j < order.size(); ++j) h_st[j] = make_int2((int)s[order[j]], (int)t[order[j]]);
+  cudaError_t e = cudaMemcpyAsync(d_st, h_st.data(), sizeof(int2) * (size_t)count, cudaMemcpyHostToDevice, stream);
+  series_inv_degree_kernel<<<g->sm_count * occ, kSeriesThreads, 0, stream>>>(g->d_node, inv, (uint32_t)n);
+  count_launch();
+  for (const Pass& p : passes) {
     if (e != cudaSuccess) break;
-    if (exec_L != Lc) {
-      if (exec) cudaGraphExecDestroy(exec);
-      exec = nullptr;
-      cudaGraph_t graph = nullptr;
-      e = cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal);
-      if (e != cudaSuccess) break;
-      exec_kernels = enqueue_pass(Lc);
-      const cudaError_t e_launch = cudaGetLastError();
-      e = cudaStreamEndCapture(stream, &graph);  // always ends the capture
-      if (e == cudaSuccess) e = e_launch;
-      if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
-      if (graph) cudaGraphDestroy(graph);
-      if (e != cudaSuccess) break;
-      exec_L = Lc;
-    }
+    const int32_t Lc = L[order[p.begin]];
+    // as many warps as the pass has rows and segments to hand out, at most the resident ones
+    const int64_t groups = (int64_t)(n * (size_t)p.cols + 31) / 32 + ((int64_t)P.nseg * p.cols + 31) / 32;
+    const int grid = (int)std::min<int64_t>((int64_t)g->sm_count * occ,
+                                            (groups * 32 + kSeriesThreads - 1) / kSeriesThreads);
     cudaEvent_t ev = nullptr;
     prof_begin(g, stream, &ev);
-    e = cudaGraphLaunch(exec, stream);
-    for (int k = 0; k < exec_kernels; ++k) count_launch();
+    const auto pass = p.cols == 4 ? series_pass<4> : (p.cols == 8 ? series_pass<8> : (p.cols == 16 ? series_pass<16> : series_pass<32>));
+    const int kernels = pass(A, xb, yb, d_st + p.begin, p.ncols, Lc, grid, reduce_grid, sums, reduce_arrived,
+                             d_out + p.begin, stream);
+    count_launches(kernels);
     prof_end(g, stream, ev, 3);
-    if (e != cudaSuccess) break;
     if (g->prof.enabled) g->prof.series_steps += (uint64_t)Lc + 1;
-    std::vector<double> res((size_t)ctl.ncols);
-    e = cudaMemcpyAsync(res.data(), ob.ptr, sizeof(double) * ctl.ncols, cudaMemcpyDeviceToHost, stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-    for (int c = 0; c < ctl.ncols && e == cudaSuccess; ++c) {
-      const int64_t i = idx[(size_t)c];
-      beta_L[i] = s[i] == t[i] ? 0.0 : res[(size_t)c];
-    }
+    e = cudaGetLastError();
   }
-  if (exec) cudaGraphExecDestroy(exec);
-  release();
+  std::vector<double> res((size_t)count);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(res.data(), d_out, sizeof(double) * (size_t)count, cudaMemcpyDeviceToHost, stream);
+  const cudaError_t e_sync = cudaStreamSynchronize(stream);  // also before `own` and the host arrays go
+  if (e == cudaSuccess) e = e_sync;
+  free_buffer(own);
   if (e != cudaSuccess) return cuda_error(e, "series");
-  PW_CUDA_TRY(cudaGetLastError());
+  for (size_t j = 0; j < order.size(); ++j) {
+    const int64_t i = order[j];
+    beta_L[i] = s[i] == t[i] ? 0.0 : res[j];
+  }
   return PW_OK;
 }

@@ -84,3 +84,33 @@ def test_median_by_rank(pw, oracle_lib, G):
     with pw.Graph(host.row_ptr, host.col_idx) as g:
         for s, t in ((1, 2), (0, 399)):
             assert pw.pw_query(g.handle, s, t, 0.3, 6, 5, params) == oracle.query(host, s, t, 0.3, 6, 5, cfg)["beta"]
+
+
+def _hub_graph(n, degrees):
+    """A ring whose first nodes also link to `degrees` others."""
+    from pw_inputs import from_edges
+
+    u, v = [np.arange(n)], [(np.arange(n) + 1) % n]
+    for i, d in enumerate(degrees):
+        u.append(np.full(d, i))
+        v.append((np.arange(d) * ((n - 40) // d) + 20 + i) % n)
+    return from_edges(n, np.concatenate(u), np.concatenate(v), name="hubs", keep_lcc=False)
+
+
+@pytest.mark.parametrize("count", [1, 4, 5, 8, 9, 16, 17, 33])
+def test_series_column_widths(pw, count):
+    """4, 8, 16 or 32 columns a pass, odd and even lengths (h takes two steps at
+    a time), rows of one segment, of several and of more than 64: FP64's values
+    to 1e-9, and each query's bits whatever it shares the pass with."""
+    from oracle import exact
+
+    host = _hub_graph(6000, [62, 63, 64, 130, 4500])
+    s, t = uniform_pairs(host.n, count, 50 + count)
+    s[0] = 4
+    with pw.Graph(host.row_ptr, host.col_idx) as g:
+        for L in (0, 1, 2, 7):
+            got = pw.pw_series_batch(g.handle, s, t, L)
+            want = exact.series_beta_many(host.row_ptr, host.col_idx, host.n, s, t, L)
+            np.testing.assert_allclose(got, want, rtol=1e-9, atol=0)
+            alone = [pw.pw_series_batch(g.handle, s[i : i + 1], t[i : i + 1], L)[0] for i in (0, count - 1)]
+            np.testing.assert_array_equal(alone, got[[0, count - 1]])
