@@ -118,6 +118,7 @@ struct Probe {
   uint32_t n_active;  // n - r
   uint32_t lo;        // Feistel halves hi and lo: domain 2^(hi + lo) >= n, hi = lo or lo + 1
   uint32_t sh_hi, sh_lo;  // 32 - hi, 32 - lo
+  uint32_t pow_lo, mask_lo;  // 2^lo, 2^lo - 1
   uint32_t rounds;    // 8, or 12 when hi + lo <= 4
   uint32_t a, b;      // hash parameters, a in [1, p-1], b in [0, p-1]
   uint32_t key[12];   // round keys 0 and 1, then key i XOR key i - 2 (feistel_pass)
@@ -147,6 +148,8 @@ __host__ __device__ __forceinline__ Probe probe_from_words(uint32_t n, const Phi
   feistel_bits(n, hi, P.lo);
   P.sh_hi = 32u - hi;
   P.sh_lo = 32u - P.lo;
+  P.pow_lo = 1u << P.lo;
+  P.mask_lo = P.pow_lo - 1u;
   P.rounds = (hi + P.lo <= 4) ? 12u : 8u;
   const uint64_t wa = (uint64_t)ab.x | ((uint64_t)ab.y << 32);
   const uint64_t wb = (uint64_t)ab.z | ((uint64_t)ab.w << 32);
@@ -209,7 +212,7 @@ __host__ __device__ __forceinline__ uint32_t feistel_f(uint32_t u, uint32_t shif
 // key took three.
 template <int ROUNDS>
 __host__ __device__ __forceinline__ uint32_t feistel_pass(const Probe& P, uint32_t x) {
-  const uint32_t left = x >> P.lo, right = x & ((1u << P.lo) - 1u);
+  const uint32_t left = x >> P.lo, right = x & P.mask_lo;
   uint32_t u0 = right ^ P.key[0];                                   // u_1
   uint32_t u1 = left ^ feistel_f(u0, P.sh_hi) ^ P.key[1];          // u_2
 #pragma unroll
@@ -218,7 +221,8 @@ __host__ __device__ __forceinline__ uint32_t feistel_pass(const Probe& P, uint32
     u0 = u1;
     u1 = u2;
   }
-  return ((u1 ^ P.out2) << P.lo) | (u0 ^ feistel_f(u1, P.sh_lo) ^ P.out1);
+  // the halves do not overlap: a product and a sum join them off the shift-and-logic pipe
+  return (u1 ^ P.out2) * P.pow_lo + (u0 ^ feistel_f(u1, P.sh_lo) ^ P.out1);
 }
 
 __host__ __device__ __forceinline__ uint32_t feistel_once(const Probe& P, uint32_t x) {
@@ -234,36 +238,33 @@ __host__ __device__ __forceinline__ uint32_t probe_pi(const Probe& P, uint32_t v
   return x;
 }
 
-// Parity of (a u + b) mod p, p = 2^31 - 1, for a, b < p and u < 2^30: one
-// Mersenne fold m = (t mod 2^31) + floor(t / 2^31) < 2p, all in 32-bit words;
-// p is odd, so subtracting it when m >= p, that is when m + 1 has bit 31 set,
-// flips the parity.
-__host__ __device__ __forceinline__ uint32_t hash_parity(uint32_t a, uint32_t u, uint32_t b) {
-  const uint64_t t = (uint64_t)a * (uint64_t)u + (uint64_t)b;
+// Sign of a node outside the zero set (pi < n - r), in bit 31: set (z = -1) when
+// h(pi / 2) + pi is odd, h the parity of (a u + b) mod p, p = 2^31 - 1, for
+// a, b < p and u < 2^30.  One Mersenne fold m = (t mod 2^31) + floor(t / 2^31) <
+// 2p stays in 32 bits; p is odd, so subtracting it when m >= p, that is when
+// m + 1 has bit 31 set, flips the parity.  The other bits are not meaningful.
+__host__ __device__ __forceinline__ uint32_t probe_sign(const Probe& P, uint32_t pi) {
+  const uint64_t t = (uint64_t)P.a * (uint64_t)(pi >> 1) + (uint64_t)P.b;
   const uint32_t lo = (uint32_t)t, hi = (uint32_t)(t >> 32);
 #ifdef __CUDA_ARCH__
   const uint32_t m = (lo & 0x7FFFFFFFu) + __funnelshift_l(lo, hi, 1);
 #else
   const uint32_t m = (lo & 0x7FFFFFFFu) + ((hi << 1) | (lo >> 31));
 #endif
-  return (m ^ ((m + 1u) >> 31)) & 1u;
-}
-
-// Sign of a node outside the zero set (pi < n - r): 1 when h(pair) + pi is odd
-// (z = -1).
-__host__ __device__ __forceinline__ uint32_t probe_negative(const Probe& P, uint32_t pi) {
-  return (hash_parity(P.a, pi >> 1, P.b) ^ pi) & 1u;
+  return ((m ^ pi) * 0x80000000u) ^ (m + 1u);
 }
 
 __host__ __device__ __forceinline__ int probe_z(const Probe& P, uint32_t v) {
   const uint32_t pi = probe_pi(P, v);
-  return pi >= P.n_active ? 0 : (probe_negative(P, pi) ? -1 : 1);
+  return pi >= P.n_active ? 0 : ((probe_sign(P, pi) >> 31) ? -1 : 1);
 }
 
-// Term z/d in FP32 from the stored correctly rounded reciprocal: +-1/d is the
-// IEEE quotient of +-1 by d and 0/d is +0.  `sign`: bit 31 set for z = -1.
-__device__ __forceinline__ float signed_term(bool zero, uint32_t sign, uint32_t inv_bits) {
-  return zero ? 0.0f : __uint_as_float(inv_bits ^ (sign & 0x80000000u));
+// sum + z/d in FP32 from the stored correctly rounded reciprocal: +-1/d is the
+// IEEE quotient of +-1 by d, and 0/d = +0 leaves the sum (never -0: it starts at
+// +0).  `sign`: bit 31 set for z = -1; its other bits are ignored.
+__device__ __forceinline__ float add_term(float sum, bool zero, uint32_t sign, uint32_t inv_bits) {
+  const float next = __fadd_rn(sum, __uint_as_float(inv_bits ^ (sign & 0x80000000u)));
+  return zero ? sum : next;
 }
 
 }  // namespace pw

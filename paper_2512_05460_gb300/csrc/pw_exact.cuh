@@ -60,11 +60,17 @@ __device__ __forceinline__ void sum_add(SumDigits& a, float U) {
   digits_add<kS2Digits>(a.d + kS1Digits, M * M, 2 * sh, false);
 }
 
+// Digits summed over the warp, for digits below 2^42 in magnitude (a lane's own
+// value has digits below 2^32): low 16 bits and the rest each by one 32-bit warp
+// reduction, 22 instructions where shuffles took 110 and as many 64-bit
+// additions.
 __device__ __forceinline__ void sum_warp_reduce(SumDigits& a) {
 #pragma unroll
-  for (int j = 0; j < kSumDigits; ++j)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a.d[j] += __shfl_xor_sync(0xffffffffu, a.d[j], o);
+  for (int j = 0; j < kSumDigits; ++j) {
+    const int lo = __reduce_add_sync(0xffffffffu, (int)(a.d[j] & 0xFFFFll));
+    const int hi = __reduce_add_sync(0xffffffffu, (int)(a.d[j] >> 16));
+    a.d[j] = (long long)lo + ((long long)hi << 16);
+  }
 }
 
 // atomics on 64-bit words add modulo 2^64, which is exact for signed digit sums

@@ -41,7 +41,8 @@ struct Totals {
   unsigned long long probes;        // all probes (Q slots)
   unsigned long long steps;         // sum of K * R * L (walk pairs times length)
   unsigned long long visits;        // sum of 2 K R (L + 1)
-  unsigned long long pad[2];
+  unsigned long long team;          // warps per probe of the team table kernel (1, 2, 4 or 8)
+  unsigned long long pad[1];
 };
 
 struct ProfileState {

@@ -88,6 +88,9 @@ struct ModeArgs {
   double visit_gain;  // saving per visit when entries come from the table
 };
 
+// Graphs of up to this many nodes run their table probes in the team kernel.
+constexpr int64_t kTeamNodes = 4096;
+
 struct ScanArgs {
   QPlan* plans;
   unsigned long long* prefix;
@@ -95,6 +98,7 @@ struct ScanArgs {
   ModeArgs M;
   int32_t keep_q;      // the second stage of ADAPTIVE queries: the Q slots stay where the first stage put them
   int32_t g0, g1;      // g1 > 0: a sharded query keeps only median-of-means blocks [g0, g1)
+  int32_t warps;       // resident warps of the team table kernel
 };
 
 // Walk mode and offsets of every query, by one block of at most 1024 threads.
@@ -102,7 +106,7 @@ struct ScanArgs {
 // warp shuffles, then over the warps.  (One thread adding 1024 partials from
 // shared memory took 37 us, whatever the batch; this takes 4 to 6.)
 __device__ void scan_plans(const ScanArgs& S, int64_t nq) {
-  constexpr int kScan = 4, kSums = 3, kAll = kScan + kSums;
+  constexpr int kScan = 4, kSums = 4, kAll = kScan + kSums;
   __shared__ unsigned long long sh[kAll][32];
   QPlan* plans = S.plans;
   unsigned long long* prefix = S.prefix;
@@ -111,8 +115,8 @@ __device__ void scan_plans(const ScanArgs& S, int64_t nq) {
   const int64_t per = (nq + nt - 1) / nt;
   const int64_t b0 = per * tid, b = b0 < nq ? b0 : nq, e = b + per < nq ? b + per : nq;
   // scanned: per-visit tiles, per-visit probes (accumulators), table probes, Q
-  // slots; summed: steps, visits, probes
-  unsigned long long a[kAll] = {0, 0, 0, 0, 0, 0, 0};
+  // slots; summed: steps, visits, probes, tiles of the table probes
+  unsigned long long a[kAll] = {0, 0, 0, 0, 0, 0, 0, 0};
   for (int64_t q = b; q < e; ++q) {
     QPlan& P = plans[q];
     // a sharded query (a batch of one): probe indices keep their global values
@@ -135,6 +139,7 @@ __device__ void scan_plans(const ScanArgs& S, int64_t nq) {
     a[4] += K * P.R * (unsigned long long)(P.L > 0 ? P.L : 0);
     a[5] += 2ull * K * P.R * (unsigned long long)(P.L + 1);
     a[6] += K;
+    a[7] += mode == 2u ? K * P.chunks : 0ull;
   }
   unsigned long long incl[kAll];
 #pragma unroll
@@ -151,6 +156,7 @@ __device__ void scan_plans(const ScanArgs& S, int64_t nq) {
   __syncthreads();
   if (warp == 0) {
     const int nw = (nt + 31) >> 5;
+    unsigned long long table_probes = 0;
 #pragma unroll
     for (int j = 0; j < kAll; ++j) {
       const unsigned long long own = lane < nw ? sh[j][lane] : 0ull;
@@ -170,6 +176,14 @@ __device__ void scan_plans(const ScanArgs& S, int64_t nq) {
         if (j == 4) T->steps = x;
         if (j == 5) T->visits = x;
         if (j == 6) T->probes = x;
+        if (j == 2) table_probes = x;
+        if (j == 7) {
+          // warps per table probe: the fewest that make four waves of probes over
+          // the resident warps, and no more than a probe has tiles
+          unsigned long long team = 1;
+          while (team < 8 && table_probes * team < 4ull * S.warps && table_probes * team < x) team *= 2;
+          T->team = team;
+        }
       }
     }
   }
@@ -197,12 +211,12 @@ __device__ void scan_plans(const ScanArgs& S, int64_t nq) {
   }
 }
 
-__global__ void scan_kernel(ScanArgs S, int64_t nq) { scan_plans(S, nq); }
+__global__ void __launch_bounds__(1024) scan_kernel(ScanArgs S, int64_t nq) { scan_plans(S, nq); }
 
 // A small batch's plans and their offsets in one launch of one block.  Up to
 // kFusedPlans queries: the FP64 divisions of more would queue up on one SM.
 constexpr int64_t kFusedPlans = 256;
-__global__ void plan_scan_kernel(int64_t nq, QueryArrays Q, BudgetArgs A, int64_t n, const int4* __restrict__ node,
+__global__ void __launch_bounds__(kFusedPlans) plan_scan_kernel(int64_t nq, QueryArrays Q, BudgetArgs A, int64_t n, const int4* __restrict__ node,
                                  QPlan* plans, QPlan* pilot, ScanArgs S) {
   for (int64_t q = threadIdx.x; q < nq; q += blockDim.x) plan_one(q, Q, A, n, node, plans, pilot);
   __syncthreads();
@@ -342,6 +356,7 @@ struct WalkArgs {
   int64_t nq;
   uint32_t n;
   uint32_t walk_tag, probe_tag;
+  int32_t pilot;  // team kernel: write (S1, S2)
 };
 
 // Persistent per-visit walk kernel: each warp pops tiles (query, probe k, 32
@@ -490,6 +505,86 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 5 : (THREADS == 512 
       A.q[P.probe_begin + kl] = u_statistic(S1, S2, R);
     }
     __syncthreads();
+  }
+}
+
+// Table kernel of graphs of few nodes (kTeamNodes): a team of 1, 2, 4 or 8 of a
+// block's warps (Totals::team) claims a probe, builds its table through the
+// warps' pools and runs its tiles.  With a block per probe, seven of 256 threads
+// built a 200-node table one after another, warps without a tile waited at three
+// barriers a probe (66 % of the stalls), and tiles of few steps paid for 110
+// shuffles each: 64 queries on a 200-node graph took 1.28 ms, 0.84 with teams (a
+// probe's table 18 ns of the GPU, 2.6 with teams).  Up to 4,096 nodes the eight
+// tables of a block take 4 KB.  Also the pilot walks of graphs of up to
+// kTeamPilotNodes, (S1, S2) per probe: one query 113 us, 93 so; building 1,024
+// entries takes a warp as long as 20 steps of per-visit walks.
+constexpr int64_t kTeamPilotNodes = 1024;
+constexpr uint32_t kTeamWarps = 8;
+template <bool DEBUG, bool SPLIT>
+__global__ void __launch_bounds__(kTeamWarps * 32, DEBUG ? 1 : 4) walk_team_kernel(WalkArgs A) {
+  const auto gr = GraphOf<SPLIT>::get(A);
+  __shared__ VisitPool pools[kTeamWarps];
+  __shared__ uint32_t tabs[kTeamWarps][kTeamNodes / 32 + 2];
+  __shared__ unsigned long long sums[kTeamWarps][kSumDigits];
+  __shared__ unsigned long long claims[kTeamWarps];
+  const unsigned long long total = A.totals->table_probes;
+  if (total == 0ull) return;
+  const uint32_t lane = threadIdx.x & 31u, size = (uint32_t)A.totals->team;
+  const uint32_t team = (threadIdx.x >> 5) / size, warp = (threadIdx.x >> 5) % size;
+  VisitPool& pool = pools[threadIdx.x >> 5];
+  uint32_t* tab = tabs[team];
+  unsigned long long* sum_of = sums[team];
+  const uint32_t n = A.n;
+  auto sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(team + 1u), "r"(size * 32u) : "memory"); };
+  for (;;) {
+    if (warp == 0) {
+      if (lane == 0) claims[team] = atomicAdd(A.counter, 1ull);
+      if (lane < kSumDigits) sum_of[lane] = 0ull;
+      if (lane < 2) tab[(n + 31u) / 32u + lane] = 0xFFFFFFFFu;
+    }
+    sync();
+    const unsigned long long j = claims[team];
+    if (j >= total) return;  // the whole team
+    const int64_t q = find_segment(A.table_prefix, A.nq, j);
+    const QPlan& P = A.plans[q];
+    const uint32_t kl = (uint32_t)(j - P.table_begin);
+    const uint32_t k = P.k_begin + kl;
+    const Probe pr = make_probe_warp(n, P.seed, k, A.probe_tag);
+    if (lane == 0) pool.probe = pr;
+    __syncwarp();
+    build_probe_table_team(pool, tab, n, warp, size, lane);
+    sync();
+    const ZTable zp = table_reader(tab, n);
+    const uint32_t R = P.R, chunks = P.chunks;
+    for (uint32_t c = warp; c < chunks; c += size) {
+      const uint32_t p = c * 32u + lane;
+      SumDigits sum;
+      sum_clear(sum);
+      if (p < R) {
+        const uint64_t pair = (uint64_t)k * R + p;
+        const float U = walk_pair_table<DEBUG>(gr, A.visits, A.walk_tag, zp, P.s, P.t, P.L, P.seed, pair);
+        if (DEBUG && A.u_debug && q == 0) A.u_debug[pair] = U;
+        sum_add(sum, U);
+      }
+      __syncwarp();
+      sum_warp_reduce(sum);
+      if (lane == 0) sum_atomic_add(sum_of, sum);
+    }
+    sync();
+    if (warp == 0 && lane == 0) {
+      long long d[kSumDigits];
+#pragma unroll
+      for (int i = 0; i < kSumDigits; ++i) d[i] = (long long)sum_of[i];
+      double S1, S2;
+      sum_round(d, S1, S2);
+      if (A.pilot) {
+        A.q[2 * (P.probe_begin + kl)] = S1;
+        A.q[2 * (P.probe_begin + kl) + 1] = S2;
+      } else {
+        A.q[P.probe_begin + kl] = u_statistic(S1, S2, R);
+      }
+    }
+    __syncwarp();
   }
 }
 
@@ -656,7 +751,22 @@ static int table_threads(const pw_graph* g) {
   return g->table_threads ? g->table_threads : default_table_threads(g);
 }
 
+// The team table kernel of a graph, its grid, and whether the graph uses it.
+static WalkFn team_fn(bool debug, bool split) {
+  if (debug) return split ? walk_team_kernel<true, true> : walk_team_kernel<true, false>;
+  return split ? walk_team_kernel<false, true> : walk_team_kernel<false, false>;
+}
+static int team_grid(pw_graph* g) { return grid_of(g, team_fn(false, g->layout == 2), kTeamWarps * 32, 0); }
+
 static pw_status launch_table(pw_graph* g, cudaStream_t stream, const WalkArgs& a, bool debug) {
+  if (g->n <= kTeamNodes) {
+    const WalkFn fn = team_fn(debug, g->layout == 2);
+    const cudaError_t e =
+        launch_with_window(g, fn, grid_of(g, fn, kTeamWarps * 32, 0), kTeamWarps * 32, 0, stream, a);
+    count_launch();
+    PW_CUDA_TRY(e);
+    return PW_OK;
+  }
   const size_t smem = table_bytes(g);
   const int threads = debug ? 256 : table_threads(g);
   const WalkFn fn = table_fn(debug, g->layout == 2, threads);
@@ -724,9 +834,12 @@ static pw_status enqueue_walks(pw_graph* g, int64_t count, const QueryArrays& Q,
   const bool table_ok = table_bytes(g) <= kMaxTableBytes;
   const int forced = params && params->walk_mode ? params->walk_mode : g->walk_policy;
   const ModeArgs M{forced, table_ok ? 1 : 0, g->table_probe_cost, g->table_visit_gain};
+  const bool team_pilot = g->n <= kTeamPilotNodes;
+  const int warps = g->n <= kTeamNodes ? team_grid(g) * (int)kTeamWarps : 0;
   ScanArgs main_scan{B.plans, prefix, B.totals, M, 0, sharded ? (int32_t)dbg->g_begin : 0,
-                     sharded ? (int32_t)dbg->g_end : 0};
-  const ScanArgs pilot_scan{B.pplans, pprefix, B.totals + 1, ModeArgs{1, 0, 0.0, 0.0}, 0, 0, 0};
+                     sharded ? (int32_t)dbg->g_end : 0, warps};
+  const ScanArgs pilot_scan{B.pplans, pprefix, B.totals + 1, ModeArgs{team_pilot ? 2 : 1, team_pilot ? 1 : 0, 0.0, 0.0},
+                            0, 0, 0, warps};
   // plans and the first offsets: the pilot's, or the main walks' where there is no pilot
   const ScanArgs& first_scan = pilot ? pilot_scan : main_scan;
   QPlan* pplans = pilot ? B.pplans : nullptr;
@@ -755,7 +868,11 @@ static pw_status enqueue_walks(pw_graph* g, int64_t count, const QueryArrays& Q,
     wa.probe_tag = kTagProbePilot;
     cudaEvent_t ev;
     prof_begin(g, stream, &ev);
-    if ((st = launch_walk(g, stream, wa, false, true)) != PW_OK) return st;
+    wa.pilot = 1;
+    wa.table_prefix = pprefix + (nq + 1);
+    if ((st = team_pilot ? launch_table(g, stream, wa, false) : launch_walk(g, stream, wa, false, true)) != PW_OK)
+      return st;
+    wa.pilot = 0;
     prof_end(g, stream, ev, 1);
     if (g->prof.enabled) g->prof.pilot_transitions += 2ull * nq * (uint64_t)ba.K0 * (uint64_t)ba.R0;
     pilot_budget_scan_kernel<<<warp_blocks, kPilotThreads, 0, stream>>>(count, B.plans, B.pplans, B.pilot_s, ba,
@@ -980,7 +1097,9 @@ static pw_status graph_batch(pw_graph* g, int64_t count, const char* h, char* ho
   pw_status st = batch_buffers(g, (size_t)count, total_K, ba, &B);  // allocations stay outside the capture
   if (st != PW_OK) return st;
   const bool table_ok = table_bytes(g) <= kMaxTableBytes;
-  if (table_ok) {  // occupancy queries stay outside the capture
+  if (g->n <= kTeamNodes) {  // occupancy queries stay outside the capture
+    team_grid(g);
+  } else if (table_ok) {
     const WalkFn tf = table_fn(false, g->layout == 2, table_threads(g));
     grid_of(g, tf, table_threads(g), table_bytes(g));
   }

@@ -161,11 +161,13 @@ __device__ bool find_job(const ServerArgs& A, uint32_t& slot, uint32_t& stage, u
 // boundary it runs at walk_kernel's speed.
 template <class GR>
 __device__ __noinline__ float server_walk_visit(const GR gr, uint32_t n, uint32_t walk_tag, uint32_t probe_tag,
-                                                VisitPool* pool, int32_t s, int32_t t, int32_t L, uint64_t seed,
-                                                uint32_t k, uint64_t pair, uint32_t m) {
+                                                int32_t s, int32_t t, int32_t L, uint64_t seed, uint32_t k,
+                                                uint64_t pair, uint32_t m) {
+  extern __shared__ uint32_t smem[];  // the warps' pools
+  VisitPool& pool = ((VisitPool*)smem)[threadIdx.x >> 5];
   const Probe pr = make_probe_warp(n, seed, k, probe_tag);
-  if ((threadIdx.x & 31u) == 0u) pool->probe = pr;
-  return walk_pair_visit<false>(gr, nullptr, walk_tag, *pool, s, t, L, seed, pair, m, threadIdx.x & 31u);
+  if ((threadIdx.x & 31u) == 0u) pool.probe = pr;
+  return walk_pair_visit<false>(gr, nullptr, walk_tag, pool, s, t, L, seed, pair, m, threadIdx.x & 31u);
 }
 
 // TABLE: the graph's probe table fits in shared memory, so main-stage jobs may
@@ -189,10 +191,9 @@ template <bool TABLE, class GR, int MINB>
 __global__ void __launch_bounds__(kServerThreads, MINB) server_kernel(ServerArgs A) {
   const GR gr = server_graph<GR>(A);
   extern __shared__ uint32_t smem[];
-  // one place for the job's table or its warps' pools (a job uses one or the
-  // other) and, after a query's last job, its block means
+  // one place for the job's table or its warps' pools (server_walk_visit; a job
+  // uses one or the other) and, after a query's last job, its block means
   uint32_t* tab = smem;
-  VisitPool* pools = (VisitPool*)smem;
   double* means = (double*)smem;
   __shared__ unsigned long long j_sum[kJobProbes][kSumDigits];
   __shared__ uint32_t j_slot, j_stage, j_k, j_count, j_valid, j_last, j_tile;
@@ -241,8 +242,7 @@ __global__ void __launch_bounds__(kServerThreads, MINB) server_kernel(ServerArgs
         if (p < R) U = walk_pair_table<false>(gr, nullptr, walk_tag, zp, P.s, P.t, P.L, P.seed, pair);
       } else {
         const uint32_t rest = R - (p - lane), m = rest < 32u ? rest : 32u;
-        U = server_walk_visit<GR>(gr, A.n, walk_tag, probe_tag, pools + (threadIdx.x >> 5), P.s, P.t, P.L, P.seed, k,
-                                  pair, m);
+        U = server_walk_visit<GR>(gr, A.n, walk_tag, probe_tag, P.s, P.t, P.L, P.seed, k, pair, m);
       }
       if (p < R) sum_add(sum, U);
       sum_warp_reduce(sum);

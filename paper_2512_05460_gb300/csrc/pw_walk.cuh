@@ -38,16 +38,17 @@ struct SplitRecords {
 };
 
 // Probe entries read from the block's table of z^(k) (built once per probe):
-// one sign bit per node (set = negative) plus the ids of the r <= 2 nodes of
-// the zero set, which the bits cannot express.
+// one sign bit per node (set = negative; node v in bit 31 - v mod 32 of its
+// word) plus the ids of the r <= 2 nodes of the zero set, which the bits cannot
+// express.
 struct ZTable {
   const uint32_t* tab;
   uint32_t zero0, zero1;  // zero-set nodes, 0xFFFFFFFF when absent
   __device__ __forceinline__ uint32_t word(uint32_t v) const { return tab[v >> 5]; }
-  // the term z/d of node v from its table word: rotating left by 31 - v mod 32
-  // puts the node's bit in the sign position
-  __device__ __forceinline__ float term(uint32_t word, uint32_t v, uint32_t inv) const {
-    return signed_term(v == zero0 || v == zero1, __funnelshift_l(word, word, ~v), inv);
+  // sum + z/d of node v from its table word: rotating left by v mod 32 puts the
+  // node's bit in the sign position
+  __device__ __forceinline__ float add(float sum, uint32_t word, uint32_t v, uint32_t inv) const {
+    return add_term(sum, v == zero0 || v == zero1, __funnelshift_l(word, word, v), inv);
   }
 };
 
@@ -71,18 +72,25 @@ template <int ROUNDS>
 __device__ __forceinline__ void pool_permute(VisitPool& pool, uint32_t total, uint32_t lane) {
   const Probe pr = pool.probe;
   const uint32_t below = (1u << lane) - 1u;
-  uint32_t i = lane, next = 32u;  // 32 + nodes done so far
-  uint32_t x = i < total ? pool.node[i] : 0u;
-  while (next < total + 32u) {
+  // byte offsets into pool.node: of this lane's node, of the next one to take
+  const uint32_t end = 4u * total;
+  uint32_t at = 4u * lane, next = 128u;
+  auto node = [&](uint32_t offset) -> uint32_t& { return *(uint32_t*)((char*)pool.node + offset); };
+  uint32_t limit = at < end ? pr.n : 0u;  // no pass of a lane without a node is done
+  uint32_t x = at < end ? node(at) : 0u;
+  while (next < end + 128u) {  // until as many were done as there are
     x = feistel_pass<ROUNDS>(pr, x);
-    const bool done = x < pr.n && i < total;
+    const bool done = x < limit;
     const uint32_t who = __ballot_sync(0xffffffffu, done);
     if (done) {
-      pool.node[i] = x;
-      i = next + __popc(who & below);
-      if (i < total) x = pool.node[i];
+      node(at) = x;
+      at = next + 4u * (uint32_t)__popc(who & below);
+      if (at < end)
+        x = node(at);
+      else
+        limit = 0u;
     }
-    next += __popc(who);
+    next += 4u * (uint32_t)__popc(who);
   }
 }
 
@@ -107,7 +115,7 @@ __device__ __forceinline__ float walk_pair_visit(const GR& gr, uint32_t* visits,
   const bool active = lane < m;
   int4 xs = gr.start(s), xt = gr.start(t);
   float a = 0.0f, b = 0.0f;
-  const uint64_t ws = 2 * pair, wt = ws + 1;
+  const uint64_t ws = 2 * pair;
   uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
   const uint32_t count = (uint32_t)L + 1u;
   for (uint32_t v0 = 0; v0 < count; v0 += kPoolSteps) {
@@ -115,8 +123,9 @@ __device__ __forceinline__ float walk_pair_visit(const GR& gr, uint32_t* visits,
     uint32_t inv_s[kPoolSteps], inv_t[kPoolSteps];
     if (active) {
       asm volatile("" : "+r"(k0), "+r"(k1));  // keeps the 20 round keys from being held over the pool's phase
+      // ws is even, so the walks share the high word, and with it the second round's first product
       const Philox4 rs = philox4x32_10((uint32_t)ws, (uint32_t)(ws >> 32), v0 >> 2, walk_tag, k0, k1);
-      const Philox4 rt = philox4x32_10((uint32_t)wt, (uint32_t)(wt >> 32), v0 >> 2, walk_tag, k0, k1);
+      const Philox4 rt = philox4x32_10((uint32_t)ws + 1u, (uint32_t)(ws >> 32), v0 >> 2, walk_tag, k0, k1);
 #pragma unroll
       for (uint32_t j = 0; j < kPoolSteps; ++j) {
         if (j < steps) {
@@ -147,8 +156,8 @@ __device__ __forceinline__ float walk_pair_visit(const GR& gr, uint32_t* visits,
       for (uint32_t j = 0; j < kPoolSteps; ++j) {
         if (j < steps) {
           const uint32_t ps = pool.node[2u * j * m + lane], pt = pool.node[(2u * j + 1u) * m + lane];
-          a = __fadd_rn(a, signed_term(ps >= pr.n_active, probe_negative(pr, ps) << 31, inv_s[j]));
-          b = __fadd_rn(b, signed_term(pt >= pr.n_active, probe_negative(pr, pt) << 31, inv_t[j]));
+          a = add_term(a, ps >= pr.n_active, probe_sign(pr, ps), inv_s[j]);
+          b = add_term(b, pt >= pr.n_active, probe_sign(pr, pt), inv_t[j]);
         }
       }
     }
@@ -169,17 +178,17 @@ template <bool DEBUG, class GR>
 __device__ __forceinline__ float walk_pair_table(const GR& gr, uint32_t* visits, uint32_t walk_tag, const ZTable& zt,
                                                  int32_t s, int32_t t, int32_t L, uint64_t seed, uint64_t pair) {
   const int4 xs = gr.start(s), xt = gr.start(t);
-  float a = zt.term(zt.word((uint32_t)xs.x), (uint32_t)xs.x, (uint32_t)xs.w);
-  float b = zt.term(zt.word((uint32_t)xt.x), (uint32_t)xt.x, (uint32_t)xt.w);
+  float a = zt.add(0.0f, zt.word((uint32_t)xs.x), (uint32_t)xs.x, (uint32_t)xs.w);
+  float b = zt.add(0.0f, zt.word((uint32_t)xt.x), (uint32_t)xt.x, (uint32_t)xt.w);
   if (DEBUG) {
     atomicAdd(visits + xs.x, 1u);
     atomicAdd(visits + xt.x, 1u);
   }
   if (L == 0) return __fsub_rn(a, b);
-  const uint64_t ws = 2 * pair, wt = ws + 1;
+  const uint64_t ws = 2 * pair;  // even: both walks have its high word
   const PhiloxKeys keys = philox_keys(seed);
   Philox4 rs = philox4x32_10((uint32_t)ws, (uint32_t)(ws >> 32), 0u, walk_tag, keys);
-  Philox4 rt = philox4x32_10((uint32_t)wt, (uint32_t)(wt >> 32), 0u, walk_tag, keys);
+  Philox4 rt = philox4x32_10((uint32_t)ws + 1u, (uint32_t)(ws >> 32), 0u, walk_tag, keys);
   int4 ns = gr.next(xs, rs.y);
   int4 nt = gr.next(xt, rt.y);
   // pending term: table word, node and reciprocal of the previous step's nodes
@@ -196,7 +205,7 @@ __device__ __forceinline__ float walk_pair_table(const GR& gr, uint32_t* visits,
         uint32_t wsw, wtw;
         if (w == 3) {
           rs = philox4x32_10((uint32_t)ws, (uint32_t)(ws >> 32), blk + 1u, walk_tag, keys);
-          rt = philox4x32_10((uint32_t)wt, (uint32_t)(wt >> 32), blk + 1u, walk_tag, keys);
+          rt = philox4x32_10((uint32_t)ws + 1u, (uint32_t)(ws >> 32), blk + 1u, walk_tag, keys);
           wsw = rs.x;
           wtw = rt.x;
         } else {
@@ -208,8 +217,8 @@ __device__ __forceinline__ float walk_pair_table(const GR& gr, uint32_t* visits,
       }
       const uint32_t cs_word = zt.word((uint32_t)ns.x), ct_word = zt.word((uint32_t)nt.x);
       if (pending) {
-        a = __fadd_rn(a, zt.term(ps_word, ps_v, ps_inv));
-        b = __fadd_rn(b, zt.term(pt_word, pt_v, pt_inv));
+        a = zt.add(a, ps_word, ps_v, ps_inv);
+        b = zt.add(b, pt_word, pt_v, pt_inv);
       }
       if (DEBUG) {
         atomicAdd(visits + ns.x, 1u);
@@ -223,8 +232,8 @@ __device__ __forceinline__ float walk_pair_table(const GR& gr, uint32_t* visits,
       pt_inv = (uint32_t)nt.w;
       pending = true;
       if (!more) {
-        a = __fadd_rn(a, zt.term(ps_word, ps_v, ps_inv));
-        b = __fadd_rn(b, zt.term(pt_word, pt_v, pt_inv));
+        a = zt.add(a, ps_word, ps_v, ps_inv);
+        b = zt.add(b, pt_word, pt_v, pt_inv);
         return __fsub_rn(a, b);
       }
       ns = ns2;
@@ -244,20 +253,45 @@ __device__ __forceinline__ void build_probe_table(const Probe& pr, uint32_t* tab
   if (threadIdx.x < 2) zero[threadIdx.x] = 0xFFFFFFFFu;
   __syncthreads();
   uint32_t w = threadIdx.x, v = w * 32u, x = v, acc = 0;
+  uint32_t stop = n - v < 32u ? n : v + 32u;  // end of the word's nodes
   while (w < nwords) {
     x = feistel_once(pr, x);
     if (x < n) {
       if (x >= pr.n_active) zero[x - pr.n_active] = v;  // its bit is not read
-      acc |= probe_negative(pr, x) << (v & 31u);
-      ++v;
-      if ((v & 31u) == 0 || v >= n) {
-        tab[w] = acc;
-        acc = 0;
+      acc = __funnelshift_l(probe_sign(pr, x), acc, 1);
+      if (++v == stop) {
+        tab[w] = acc << ((w + 1u) * 32u - stop);  // a last word may hold fewer nodes
         w += blockDim.x;
         v = w * 32u;
+        stop = n - v < 32u ? n : v + 32u;
       }
       x = v;
     }
+  }
+}
+
+// The same for a graph of few nodes by `warps` warps, of which this is number
+// `warp`, each taking up to 256 nodes at a time through its pool.
+__device__ __forceinline__ void build_probe_table_team(VisitPool& pool, uint32_t* tab, uint32_t n, uint32_t warp,
+                                                       uint32_t warps, uint32_t lane) {
+  constexpr uint32_t kBatch = 2u * kPoolSteps * 32u;
+  const uint32_t n_active = pool.probe.n_active;
+  for (uint32_t base = warp * kBatch; base < n; base += warps * kBatch) {
+    const uint32_t count = n - base < kBatch ? n - base : kBatch;
+    for (uint32_t i = lane; i < count; i += 32u) pool.node[i] = base + i;
+    __syncwarp();
+    if (pool.probe.rounds == 8u)
+      pool_permute<8>(pool, count, lane);
+    else
+      pool_permute<12>(pool, count, lane);
+    __syncwarp();
+    for (uint32_t i = lane; i - lane < count; i += 32u) {
+      const uint32_t pi = i < count ? pool.node[i] : 0u;
+      if (i < count && pi >= n_active) tab[(n + 31u) / 32u + pi - n_active] = base + i;
+      const uint32_t word = __ballot_sync(0xffffffffu, (int32_t)probe_sign(pool.probe, pi) < 0);
+      if (lane == 0) tab[(base + i) >> 5] = __brev(word);
+    }
+    __syncwarp();
   }
 }
 

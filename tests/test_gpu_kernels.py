@@ -114,3 +114,31 @@ def test_series_column_widths(pw, count):
             np.testing.assert_allclose(got, want, rtol=1e-9, atol=0)
             alone = [pw.pw_series_batch(g.handle, s[i : i + 1], t[i : i + 1], L)[0] for i in (0, count - 1)]
             np.testing.assert_array_equal(alone, got[[0, count - 1]])
+
+
+@pytest.mark.parametrize("n", [5, 16, 17, 33, 255, 257, 1024, 1025, 4095, 4096, 4097])
+def test_team_tables(pw, oracle_lib, n):
+    """Table walks of small graphs by teams of one to eight warps: node counts
+    around a word, a warp's batch of 256, the pilot's limit and the kernel's;
+    probe counts that make teams of eight, of few and of one.  The per-visit
+    kernel gives the same estimates, the oracle the single query's replicas."""
+    host = complete_graph(n) if n < 17 else (cycle_graph(n) if n > 1025 else er_cycle(n, min(0.2, 8 / n), 3))
+    s, t = np.array([0, 1, 2]), np.array([n - 1, 3, 4])
+    seeds = query_seeds(3, n)
+    with pw.Graph(host.row_ptr, host.col_idx) as g:
+        for B, G, R, L in ((1, 3, 300, 5), (7, 150, 65, 3), (40, 200, 33, 2), (40, 200, 2, 0)):
+            got = []
+            for mode in (1, 2):
+                params = pw.make_params(budget_mode=pw.PW_BUDGET_FIXED, B=B, G=G, R=R, walk_mode=mode)
+                beta, st = pw.pw_query_batch(g.handle, s, t, 0.3, L, seeds, params)
+                assert np.all(st == 0)
+                got.append(beta)
+            np.testing.assert_array_equal(got[0], got[1])
+        params = pw.make_params(budget_mode=pw.PW_BUDGET_FIXED, B=1, G=2, R=70, walk_mode=2)
+        dev = pw.pw_debug_query(g.handle, host.n, 0, n - 1, 0.3, 6, 9, params, q_cap=8, u_cap=256, want_visits=True)
+        orc = oracle.query(host, 0, n - 1, 0.3, 6, 9, oracle.budget_cfg(mode=oracle.MODE_FIXED, B=1, G=2, R=70),
+                           want_q=True, want_u=True, want_visits=True)
+        np.testing.assert_array_equal(dev["u"], orc["u"])
+        np.testing.assert_array_equal(dev["visits"], orc["visits"])
+        b = oracle.budget(host, 0, n - 1, 0.3, 6, 9)
+        assert pw.pw_budget(g.handle, 0, n - 1, 0.3, 6, 9) == {k: b[k] for k in "BGKR"}
