@@ -9,6 +9,7 @@
 
 #include "pw_device.cuh"
 #include "pw_internal.h"
+#include "pw_walk.cuh"
 
 namespace pw {
 
@@ -29,6 +30,22 @@ __global__ void build_records_kernel(const int32_t* __restrict__ row_ptr, const 
     else
       node[e - nnz] = r;
   }
+}
+
+// The arrays of RankedRecords: neighbours' ranks three to a word, node records by rank.
+__global__ void build_ranked_kernel(const int32_t* __restrict__ col, const int4* __restrict__ node,
+                                    const int32_t* __restrict__ rank, int64_t n, int64_t nnz,
+                                    uint64_t* __restrict__ packed, int4* __restrict__ ranked) {
+  const int64_t words = (nnz + 2) / 3;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += (int64_t)gridDim.x * blockDim.x) {
+    uint64_t w = 0;
+    for (int j = 0; j < 3 && 3 * i + j < nnz; ++j)
+      w |= (uint64_t)(uint32_t)rank[col[3 * i + j]] << (RankedRecords::kBits * j);
+    packed[i] = w;
+    if (i < n) ranked[rank[i]] = node[i];
+  }
+  for (int64_t v = words + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
+    ranked[rank[v]] = node[v];
 }
 
 __global__ void debug_philox_kernel(uint4 ctr, uint2 key, uint4* out) {
@@ -64,11 +81,10 @@ __global__ void debug_walk_kernel(const int32_t* __restrict__ col, const int4* _
 // gathers with the walk's access per step (the next index depends on the
 // loaded value, as in a walk), 8 independent chains per thread, no other work.
 // Fused layout: one 16-B record uniform over the record array.  Split layout:
-// a 4-B col_idx entry uniform over col_idx, then the node record it names.
-template <bool SPLIT>
-__global__ void __launch_bounds__(256) gather_peak_kernel(const int4* __restrict__ rec, const int32_t* __restrict__ col,
-                                                         const int4* __restrict__ node, uint32_t nnz, uint32_t iters,
-                                                         uint32_t* sink) {
+// a col_idx entry uniform over col_idx (4 B, or packed), then the node record it
+// names.
+template <class GR>
+__global__ void __launch_bounds__(256) gather_peak_kernel(GR gr, uint32_t nnz, uint32_t iters, uint32_t* sink) {
   const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x;
   uint32_t x[8];
 #pragma unroll
@@ -77,8 +93,7 @@ __global__ void __launch_bounds__(256) gather_peak_kernel(const int4* __restrict
   for (uint32_t it = 0; it < iters; ++it) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      const uint32_t e = __umulhi(x[j], nnz);
-      const int4 r = SPLIT ? __ldg(node + __ldg(col + e)) : __ldg(rec + e);
+      const int4 r = gr.next(make_int4(0, 0, (int)nnz, 0), x[j]);
       x[j] = x[j] * 1664525u + 1013904223u + (uint32_t)r.y;
       acc += (uint32_t)r.x;
     }
@@ -180,9 +195,31 @@ static pw_status upload(pw_graph* g, const int64_t* rp64, const int32_t* col) {
   const int blocks = (int)std::min<int64_t>((work + threads - 1) / threads, (int64_t)g->sm_count * 32);
   build_records_kernel<<<blocks, threads, 0, g->stream>>>(d_rp, d_col, g->n, g->nnz, g->d_rec, g->d_node);
   count_launch();
+  int32_t* d_rank = nullptr;
+  std::vector<int32_t> rank;  // by degree, the largest first, in node order among equals
+  if (g->access == WalkAccess::kRanked) {
+    std::vector<int32_t> first((size_t)g->d_max + 2, 0);
+    for (int32_t d : g->deg) ++first[(size_t)d];
+    int32_t at = 0;
+    for (int32_t d = g->d_max; d >= 0; --d) {
+      const int32_t c = first[(size_t)d];
+      first[(size_t)d] = at;
+      at += c;
+    }
+    rank.resize((size_t)g->n);
+    for (int64_t v = 0; v < g->n; ++v) rank[(size_t)v] = first[(size_t)g->deg[(size_t)v]]++;
+    PW_CUDA_TRY(cudaMalloc(&g->d_packed, sizeof(uint64_t) * (size_t)((g->nnz + 2) / 3)));
+    PW_CUDA_TRY(cudaMalloc(&g->d_ranked, sizeof(int4) * (size_t)g->n));
+    PW_CUDA_TRY(cudaMalloc(&d_rank, sizeof(int32_t) * (size_t)g->n));
+    PW_CUDA_TRY(cudaMemcpyAsync(d_rank, rank.data(), sizeof(int32_t) * (size_t)g->n, cudaMemcpyHostToDevice, g->stream));
+    build_ranked_kernel<<<blocks, threads, 0, g->stream>>>(d_col, g->d_node, d_rank, g->n, g->nnz, g->d_packed,
+                                                           g->d_ranked);
+    count_launch();
+  }
   PW_CUDA_TRY(cudaGetLastError());
   PW_CUDA_TRY(cudaStreamSynchronize(g->stream));
   cudaFree(d_rp);
+  if (d_rank) cudaFree(d_rank);
   PW_CUDA_TRY(cudaMallocHost(&g->ws.host_totals, sizeof(Totals)));
   PW_CUDA_TRY(cudaEventCreateWithFlags(&g->ws.last_use, cudaEventDisableTiming));
   return PW_OK;
@@ -209,13 +246,13 @@ pw_status set_l2_window(pw_graph* g, int which) {
   void* base = nullptr;
   size_t bytes = 0;
   if (which == 1 && g->layout == 2) {
-    base = g->d_col;
-    bytes = sizeof(int32_t) * (size_t)g->nnz;
+    base = g->d_packed ? (void*)g->d_packed : (void*)g->d_col;
+    bytes = g->d_packed ? sizeof(uint64_t) * (size_t)((g->nnz + 2) / 3) : sizeof(int32_t) * (size_t)g->nnz;
   } else if (which == 1) {
     base = g->d_rec;
     bytes = sizeof(int4) * (size_t)g->nnz;
   } else {
-    base = g->d_node;
+    base = g->d_ranked ? g->d_ranked : g->d_node;
     bytes = sizeof(int4) * (size_t)g->n;
   }
   const size_t num = bytes < (size_t)max_window ? bytes : (size_t)max_window;
@@ -254,6 +291,8 @@ static void destroy(pw_graph* g) {
   if (g->d_rec) cudaFree(g->d_rec);
   if (g->d_col) cudaFree(g->d_col);
   if (g->d_node) cudaFree(g->d_node);
+  if (g->d_packed) cudaFree(g->d_packed);
+  if (g->d_ranked) cudaFree(g->d_ranked);
   if (g->stream) cudaStreamDestroy(g->stream);
   delete g;
 }
@@ -289,6 +328,10 @@ static pw_status load_common(int64_t n, const int64_t* rp, const int32_t* col, i
     g->layout = 2;
   else
     g->layout = (fused_bytes > (double)((size_t)64 << 20) && split_bytes <= (double)((size_t)160 << 20)) ? 2 : 1;
+  if (g->layout == 2)
+    g->access = split_bytes > (double)((size_t)64 << 20) && n <= (int64_t)1 << RankedRecords::kBits
+                    ? WalkAccess::kRanked
+                    : WalkAccess::kSplit;
   st = upload(g, rp, col);
   if (st != PW_OK) {
     destroy(g);
@@ -380,9 +423,11 @@ pw_status pw_debug_gather_peak(pw_graph* g, int32_t iters, double* sectors_per_s
   pw_status st = pw::ensure_buffer(b, 64);
   if (st != PW_OK) return st;
   int nb = 0;
-  const bool split = g->layout == 2;
-  PW_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      &nb, split ? pw::gather_peak_kernel<true> : pw::gather_peak_kernel<false>, 256, 0));
+  const pw::WalkAccess access = g->access;
+  const void* fn = access == pw::WalkAccess::kFused   ? (const void*)pw::gather_peak_kernel<pw::FusedRecords>
+                   : access == pw::WalkAccess::kSplit ? (const void*)pw::gather_peak_kernel<pw::SplitRecords>
+                                                      : (const void*)pw::gather_peak_kernel<pw::RankedRecords>;
+  PW_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, 256, 0));
   const int blocks = g->sm_count * (nb > 0 ? nb : 1);
   cudaEvent_t e0, e1;
   PW_CUDA_TRY(cudaEventCreate(&e0));
@@ -390,12 +435,15 @@ pw_status pw_debug_gather_peak(pw_graph* g, int32_t iters, double* sectors_per_s
   double best = 0.0;
   for (int rep = 0; rep < 3; ++rep) {
     PW_CUDA_TRY(cudaEventRecord(e0, g->stream));
-    if (split)
-      pw::gather_peak_kernel<true><<<blocks, 256, 0, g->stream>>>(g->d_rec, g->d_col, g->d_node, (uint32_t)g->nnz,
-                                                                  (uint32_t)iters, (uint32_t*)b.ptr);
+    if (access == pw::WalkAccess::kFused)
+      pw::gather_peak_kernel<<<blocks, 256, 0, g->stream>>>(pw::FusedRecords{g->d_rec, g->d_node}, (uint32_t)g->nnz,
+                                                            (uint32_t)iters, (uint32_t*)b.ptr);
+    else if (access == pw::WalkAccess::kSplit)
+      pw::gather_peak_kernel<<<blocks, 256, 0, g->stream>>>(pw::SplitRecords{g->d_col, g->d_node}, (uint32_t)g->nnz,
+                                                            (uint32_t)iters, (uint32_t*)b.ptr);
     else
-      pw::gather_peak_kernel<false><<<blocks, 256, 0, g->stream>>>(g->d_rec, g->d_col, g->d_node, (uint32_t)g->nnz,
-                                                                   (uint32_t)iters, (uint32_t*)b.ptr);
+      pw::gather_peak_kernel<<<blocks, 256, 0, g->stream>>>(pw::RankedRecords{g->d_packed, g->d_node, g->d_ranked}, (uint32_t)g->nnz,
+                                                            (uint32_t)iters, (uint32_t*)b.ptr);
     pw::count_launch();
     PW_CUDA_TRY(cudaGetLastError());
     PW_CUDA_TRY(cudaEventRecord(e1, g->stream));

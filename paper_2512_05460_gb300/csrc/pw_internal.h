@@ -13,6 +13,9 @@
 
 namespace pw {
 
+// How a walk reads the graph (pw_walk.cuh).
+enum class WalkAccess { kFused, kSplit, kRanked };
+
 // Per-query plan, one per query of a batch, resident in device memory.
 struct QPlan {
   uint64_t seed;
@@ -120,7 +123,10 @@ struct pw_graph {
   int4* d_rec = nullptr;     // nnz neighbour records (fused layout only)
   int32_t* d_col = nullptr;  // nnz neighbour ids (always)
   int4* d_node = nullptr;    // n node records
-  int layout = 1;            // walk access: 1 fused records, 2 col_idx + node records
+  uint64_t* d_packed = nullptr;  // neighbours' ranks by degree, three to a word (kRanked only)
+  int4* d_ranked = nullptr;      // node records by rank (kRanked only)
+  int layout = 1;            // walk layout: 1 fused records, 2 col_idx + node records
+  pw::WalkAccess access = pw::WalkAccess::kFused;  // the layout's form that walks read
   cudaStream_t stream = nullptr;
   std::map<std::pair<const void*, size_t>, int> grids;  // persistent grid per walk kernel and shared memory
   // Table-kernel block size (pw_autotune; 0: by shared memory, else 256, 512

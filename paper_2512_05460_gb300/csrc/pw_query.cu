@@ -341,9 +341,11 @@ __device__ __forceinline__ int64_t find_segment(const unsigned long long* __rest
 }
 
 struct WalkArgs {
-  const int4* rec;   // fused records (layout 1)
-  const int32_t* col;  // col_idx (layout 2)
+  const int4* rec;        // fused records
+  const int32_t* col;     // col_idx (split)
+  const uint64_t* packed;  // neighbours' ranks, three to a word (ranked)
   const int4* node;
+  const int4* ranked;     // node records by rank (ranked)
   const QPlan* plans;
   const unsigned long long* tile_prefix;   // per-visit tiles
   const unsigned long long* table_prefix;  // table-kernel probes
@@ -365,25 +367,29 @@ struct WalkArgs {
 // its tile's replicas exactly; a pilot tile is a whole probe (R0 <= 32) and
 // writes (S1, S2); a main tile adds its digits to the probe's accumulator and
 // the probe's last tile computes Q_R.
-// The graph access of a launch: fused records, or col_idx plus node records.
-template <bool SPLIT>
+// The graph access of a launch.
+template <WalkAccess ACCESS>
 struct GraphOf;
 template <>
-struct GraphOf<false> {
+struct GraphOf<WalkAccess::kFused> {
   static __device__ __forceinline__ FusedRecords get(const WalkArgs& A) { return FusedRecords{A.rec, A.node}; }
 };
 template <>
-struct GraphOf<true> {
+struct GraphOf<WalkAccess::kSplit> {
   static __device__ __forceinline__ SplitRecords get(const WalkArgs& A) { return SplitRecords{A.col, A.node}; }
+};
+template <>
+struct GraphOf<WalkAccess::kRanked> {
+  static __device__ __forceinline__ RankedRecords get(const WalkArgs& A) { return RankedRecords{A.packed, A.node, A.ranked}; }
 };
 
 // 3 blocks per SM (80 registers, 9 KB of pools each, the rest of the SM's
 // memory caching the graph): 4 blocks (64 registers, some spilled) took 5.9 ps
 // a visit on a 2000^2 grid against 5.3, 6.2 against 5.8 on a 10^5-node graph,
 // and 9.8 against 10.2 on R-MAT 2^20.
-template <bool DEBUG, bool PILOT, bool SPLIT>
+template <bool DEBUG, bool PILOT, WalkAccess ACCESS>
 __global__ void __launch_bounds__(kWalkThreads, DEBUG ? 1 : 3) walk_kernel(WalkArgs A) {
-  const auto gr = GraphOf<SPLIT>::get(A);
+  const auto gr = GraphOf<ACCESS>::get(A);
   const uint32_t lane = threadIdx.x & 31u;
   const unsigned long long total = A.totals->tiles;
   if (total == 0ull) return;
@@ -446,9 +452,9 @@ __global__ void __launch_bounds__(kWalkThreads, DEBUG ? 1 : 3) walk_kernel(WalkA
 // domain has (2 R (L+1) > 2^b).
 // THREADS: 256 (five blocks per SM for small tables), 512 or 1024 (one or two
 // blocks per SM with up to 200 KB of table, still 32 warps).
-template <bool DEBUG, bool SPLIT, int THREADS>
+template <bool DEBUG, WalkAccess ACCESS, int THREADS>
 __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 5 : (THREADS == 512 ? 2 : 1)) walk_table_kernel(WalkArgs A) {
-  const auto gr = GraphOf<SPLIT>::get(A);
+  const auto gr = GraphOf<ACCESS>::get(A);
   extern __shared__ uint32_t tab[];
   __shared__ unsigned long long sh_probe;
   __shared__ unsigned long long sh_sum[kSumDigits];
@@ -520,9 +526,9 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 5 : (THREADS == 512 
 // entries takes a warp as long as 20 steps of per-visit walks.
 constexpr int64_t kTeamPilotNodes = 1024;
 constexpr uint32_t kTeamWarps = 8;
-template <bool DEBUG, bool SPLIT>
+template <bool DEBUG, WalkAccess ACCESS>
 __global__ void __launch_bounds__(kTeamWarps * 32, DEBUG ? 1 : 4) walk_team_kernel(WalkArgs A) {
-  const auto gr = GraphOf<SPLIT>::get(A);
+  const auto gr = GraphOf<ACCESS>::get(A);
   __shared__ VisitPool pools[kTeamWarps];
   __shared__ uint32_t tabs[kTeamWarps][kTeamNodes / 32 + 2];
   __shared__ unsigned long long sums[kTeamWarps][kSumDigits];
@@ -701,28 +707,40 @@ void prof_end(pw_graph* g, cudaStream_t stream, cudaEvent_t a, int kind) {
 static size_t table_bytes(const pw_graph* g) { return sizeof(uint32_t) * (size_t)table_words((uint32_t)g->n); }
 static constexpr size_t kMaxTableBytes = 200 * 1024;
 
-// Table-kernel block size by shared memory: 256 threads while five tables fit
-// per SM (then registers limit it to five blocks), 512 while two fit, else 1024.
+// Table-kernel block size by shared memory: 256 threads up to 32 KB a table (five
+// blocks per SM; at 41 KB and R = 1024 five tables left the gathers 20 KB of L1
+// and took 64 ms where two blocks of 512 took 30, at 24 KB 7.8 against 8.0), 512
+// while two tables fit, else 1024.
 static int default_table_threads(const pw_graph* g) {
   const size_t per_block = table_bytes(g) + 2048;
-  const size_t fit = ((size_t)228 << 10) / per_block;
-  return fit >= 5 ? 256 : (fit >= 2 ? 512 : 1024);
+  return per_block <= ((size_t)34 << 10) ? 256 : (2 * per_block <= ((size_t)228 << 10) ? 512 : 1024);
 }
 
 using WalkFn = void (*)(WalkArgs);
 
-static WalkFn walk_fn(bool debug, bool pilot, bool split) {
-  if (debug) return split ? walk_kernel<true, false, true> : walk_kernel<true, false, false>;
-  if (pilot) return split ? walk_kernel<false, true, true> : walk_kernel<false, true, false>;
-  return split ? walk_kernel<false, false, true> : walk_kernel<false, false, false>;
+template <WalkAccess ACCESS>
+static WalkFn walk_fn_of(bool debug, bool pilot) {
+  return debug ? walk_kernel<true, false, ACCESS>
+               : (pilot ? walk_kernel<false, true, ACCESS> : walk_kernel<false, false, ACCESS>);
+}
+static WalkFn walk_fn(bool debug, bool pilot, WalkAccess access) {
+  return access == WalkAccess::kFused   ? walk_fn_of<WalkAccess::kFused>(debug, pilot)
+         : access == WalkAccess::kSplit ? walk_fn_of<WalkAccess::kSplit>(debug, pilot)
+                                        : walk_fn_of<WalkAccess::kRanked>(debug, pilot);
 }
 
 // The table kernel of a launch (DEBUG builds exist only at 256 threads).
-static WalkFn table_fn(bool debug, bool split, int threads) {
-  if (debug) return split ? walk_table_kernel<true, true, 256> : walk_table_kernel<true, false, 256>;
-  if (threads == 1024) return split ? walk_table_kernel<false, true, 1024> : walk_table_kernel<false, false, 1024>;
-  if (threads == 512) return split ? walk_table_kernel<false, true, 512> : walk_table_kernel<false, false, 512>;
-  return split ? walk_table_kernel<false, true, 256> : walk_table_kernel<false, false, 256>;
+template <WalkAccess ACCESS>
+static WalkFn table_fn_of(bool debug, int threads) {
+  if (debug) return walk_table_kernel<true, ACCESS, 256>;
+  return threads == 1024  ? walk_table_kernel<false, ACCESS, 1024>
+         : threads == 512 ? walk_table_kernel<false, ACCESS, 512>
+                          : walk_table_kernel<false, ACCESS, 256>;
+}
+static WalkFn table_fn(bool debug, WalkAccess access, int threads) {
+  return access == WalkAccess::kFused   ? table_fn_of<WalkAccess::kFused>(debug, threads)
+         : access == WalkAccess::kSplit ? table_fn_of<WalkAccess::kSplit>(debug, threads)
+                                        : table_fn_of<WalkAccess::kRanked>(debug, threads);
 }
 
 // Persistent grid: SMs x resident blocks, measured once per kernel and
@@ -740,7 +758,7 @@ static int grid_of(pw_graph* g, WalkFn fn, int threads, size_t smem) {
 }
 
 static pw_status launch_walk(pw_graph* g, cudaStream_t stream, const WalkArgs& a, bool debug, bool pilot) {
-  const WalkFn fn = walk_fn(debug, pilot, g->layout == 2);
+  const WalkFn fn = walk_fn(debug, pilot, g->access);
   const cudaError_t e = launch_with_window(g, fn, grid_of(g, fn, kWalkThreads, 0), kWalkThreads, 0, stream, a);
   count_launch();
   PW_CUDA_TRY(e);
@@ -752,15 +770,18 @@ static int table_threads(const pw_graph* g) {
 }
 
 // The team table kernel of a graph, its grid, and whether the graph uses it.
-static WalkFn team_fn(bool debug, bool split) {
-  if (debug) return split ? walk_team_kernel<true, true> : walk_team_kernel<true, false>;
-  return split ? walk_team_kernel<false, true> : walk_team_kernel<false, false>;
+static WalkFn team_fn(bool debug, WalkAccess access) {  // ranked arrays belong to larger graphs
+  if (debug)
+    return access == WalkAccess::kFused ? walk_team_kernel<true, WalkAccess::kFused>
+                                        : walk_team_kernel<true, WalkAccess::kSplit>;
+  return access == WalkAccess::kFused ? walk_team_kernel<false, WalkAccess::kFused>
+                                      : walk_team_kernel<false, WalkAccess::kSplit>;
 }
-static int team_grid(pw_graph* g) { return grid_of(g, team_fn(false, g->layout == 2), kTeamWarps * 32, 0); }
+static int team_grid(pw_graph* g) { return grid_of(g, team_fn(false, g->access), kTeamWarps * 32, 0); }
 
 static pw_status launch_table(pw_graph* g, cudaStream_t stream, const WalkArgs& a, bool debug) {
   if (g->n <= kTeamNodes) {
-    const WalkFn fn = team_fn(debug, g->layout == 2);
+    const WalkFn fn = team_fn(debug, g->access);
     const cudaError_t e =
         launch_with_window(g, fn, grid_of(g, fn, kTeamWarps * 32, 0), kTeamWarps * 32, 0, stream, a);
     count_launch();
@@ -769,7 +790,7 @@ static pw_status launch_table(pw_graph* g, cudaStream_t stream, const WalkArgs& 
   }
   const size_t smem = table_bytes(g);
   const int threads = debug ? 256 : table_threads(g);
-  const WalkFn fn = table_fn(debug, g->layout == 2, threads);
+  const WalkFn fn = table_fn(debug, g->access, threads);
   const cudaError_t e = launch_with_window(g, fn, grid_of(g, fn, threads, smem), threads, smem, stream, a);
   count_launch();
   PW_CUDA_TRY(e);
@@ -826,6 +847,8 @@ static pw_status enqueue_walks(pw_graph* g, int64_t count, const QueryArrays& Q,
   memset(&wa, 0, sizeof wa);
   wa.rec = g->d_rec;
   wa.col = g->d_col;
+  wa.packed = g->d_packed;
+  wa.ranked = g->d_ranked;
   wa.node = g->d_node;
   wa.nq = count;
   wa.n = (uint32_t)g->n;
@@ -1100,10 +1123,10 @@ static pw_status graph_batch(pw_graph* g, int64_t count, const char* h, char* ho
   if (g->n <= kTeamNodes) {  // occupancy queries stay outside the capture
     team_grid(g);
   } else if (table_ok) {
-    const WalkFn tf = table_fn(false, g->layout == 2, table_threads(g));
+    const WalkFn tf = table_fn(false, g->access, table_threads(g));
     grid_of(g, tf, table_threads(g), table_bytes(g));
   }
-  for (int pilot = 0; pilot < 2; ++pilot) grid_of(g, walk_fn(false, pilot != 0, g->layout == 2), kWalkThreads, 0);
+  for (int pilot = 0; pilot < 2; ++pilot) grid_of(g, walk_fn(false, pilot != 0, g->access), kWalkThreads, 0);
   std::vector<unsigned char> key;
   key_put(key, count);
   key_put(key, total_K);

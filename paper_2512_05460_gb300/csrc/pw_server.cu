@@ -61,9 +61,11 @@ struct Completion {
 };
 
 struct ServerArgs {
-  const int4* rec;     // fused records (layout 1)
-  const int32_t* col;  // col_idx (layout 2)
+  const int4* rec;        // fused records
+  const int32_t* col;     // col_idx (split)
+  const uint64_t* packed;  // neighbours' ranks, three to a word (ranked)
   const int4* node;
+  const int4* ranked;     // node records by rank (ranked)
   uint32_t n;
   uint32_t has_table;  // 0: graph too large for a shared-memory table
   SlotDev* slots;
@@ -175,7 +177,7 @@ __device__ __noinline__ float server_walk_visit(const GR gr, uint32_t n, uint32_
 // occupancy the registers are capped for: 2 blocks/SM (the registers the
 // per-visit path asks for) or 3 (fewer registers, some spilled), whichever
 // pw_server_tune finds faster on the graph.
-// The graph access of the server: fused records, or col_idx plus node records.
+// The graph access of the server.
 template <class GR>
 __device__ __forceinline__ GR server_graph(const ServerArgs& A);
 template <>
@@ -185,6 +187,10 @@ __device__ __forceinline__ FusedRecords server_graph<FusedRecords>(const ServerA
 template <>
 __device__ __forceinline__ SplitRecords server_graph<SplitRecords>(const ServerArgs& A) {
   return SplitRecords{A.col, A.node};
+}
+template <>
+__device__ __forceinline__ RankedRecords server_graph<RankedRecords>(const ServerArgs& A) {
+  return RankedRecords{A.packed, A.node, A.ranked};
 }
 
 template <bool TABLE, class GR, int MINB>
@@ -336,13 +342,14 @@ __global__ void __launch_bounds__(kServerThreads, MINB) server_kernel(ServerArgs
 
 using ServerFn = void (*)(ServerArgs);
 // minb: 2 or 3 blocks/SM for the per-visit-only kernel (the table kernel is 4)
-static ServerFn server_fn(bool table, int layout, int minb) {
-  if (layout == 2) {
-    if (table) return server_kernel<true, SplitRecords, 4>;
-    return minb == 3 ? server_kernel<false, SplitRecords, 3> : server_kernel<false, SplitRecords, 2>;
-  }
-  if (table) return server_kernel<true, FusedRecords, 4>;
-  return minb == 3 ? server_kernel<false, FusedRecords, 3> : server_kernel<false, FusedRecords, 2>;
+template <class GR>
+static ServerFn server_fn_of(bool table, int minb) {
+  return table ? server_kernel<true, GR, 4> : (minb == 3 ? server_kernel<false, GR, 3> : server_kernel<false, GR, 2>);
+}
+static ServerFn server_fn(bool table, WalkAccess access, int minb) {
+  return access == WalkAccess::kFused   ? server_fn_of<FusedRecords>(table, minb)
+         : access == WalkAccess::kSplit ? server_fn_of<SplitRecords>(table, minb)
+                                        : server_fn_of<RankedRecords>(table, minb);
 }
 
 struct Request {
@@ -449,6 +456,8 @@ static ServerArgs server_args(pw_server* sv) {
   ServerArgs a;
   a.rec = sv->g->d_rec;
   a.col = sv->g->d_col;
+  a.packed = sv->g->d_packed;
+  a.ranked = sv->g->d_ranked;
   a.node = sv->g->d_node;
   a.n = (uint32_t)sv->g->n;
   a.has_table = sv->has_table ? 1u : 0u;
@@ -579,7 +588,7 @@ static void worker_loop(pw_server* sv) {
         cudaStreamWaitEvent(sv->kstream, ev, 0);
         cudaEventDestroy(ev);
         cudaMemsetAsync(sv->d_ctl + 4, 0, sizeof(unsigned long long), sv->kstream);  // exit flag
-        const ServerFn fn = server_fn(sv->has_table, sv->g->layout, minb);
+        const ServerFn fn = server_fn(sv->has_table, sv->g->access, minb);
         const cudaError_t e = launch_with_window(sv->g, fn, grid, kServerThreads, sv->smem, sv->kstream, args);
         count_launch();
         if (e != cudaSuccess) {
@@ -671,7 +680,7 @@ pw_status pw_server_create(pw_graph* g, const pw_params* params, size_t accum_by
   sv->smem = kServerMeansBytes > pbytes ? kServerMeansBytes : pbytes;
   if (with_table && tbytes > sv->smem) sv->smem = tbytes;
   for (int v = 0; v < (with_table ? 1 : 2); ++v) {
-    const ServerFn fn = server_fn(with_table, g->layout, 2 + v);
+    const ServerFn fn = server_fn(with_table, g->access, 2 + v);
     if ((e = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sv->smem)) !=
         cudaSuccess)
       return fail(cuda_error(e, "server smem attribute"));

@@ -142,3 +142,37 @@ def test_team_tables(pw, oracle_lib, n):
         np.testing.assert_array_equal(dev["visits"], orc["visits"])
         b = oracle.budget(host, 0, n - 1, 0.3, 6, 9)
         assert pw.pw_budget(g.handle, 0, n - 1, 0.3, 6, 9) == {k: b[k] for k in "BGKR"}
+
+
+def test_ranked_records(pw):
+    """A power-law graph whose col_idx and node records exceed 64 MB: walks read
+    packed ranks by degree, and give the fused layout's trajectories and estimates
+    in both walk kernels and the server."""
+    from pw_inputs import rmat_native
+
+    host = rmat_native(18, 80, (0.57, 0.19, 0.19, 0.05), 6)
+    assert 4 * host.nnz + 16 * host.n > 64 << 20 and host.n <= 1 << 21
+    s, t = uniform_pairs(host.n, 5, 71)
+    s[0] = int(np.argmax(np.diff(host.row_ptr)))
+    seeds = query_seeds(5, 72)
+    flags = pw.LOAD_NO_CONNECTIVITY
+    with pw.Graph(host.row_ptr, host.col_idx, flags=flags) as g, \
+            pw.Graph(host.row_ptr, host.col_idx, flags=flags | pw.LOAD_FUSED) as f:
+        assert pw.pw_profile(g.handle, enable=False)["layout"] == 2
+        want, _ = pw.pw_query_batch(f.handle, s, t, 0.3, 21, seeds)
+        for mode in (0, 1, 2):
+            got, st = pw.pw_query_batch(g.handle, s, t, 0.3, 21, seeds, pw.make_params(walk_mode=mode))
+            assert np.all(st == 0)
+            np.testing.assert_array_equal(got, want)
+        params = pw.make_params(budget_mode=pw.PW_BUDGET_FIXED, B=1, G=2, R=40, walk_mode=1)
+        q = [pw.pw_debug_query(h.handle, host.n, int(s[0]), int(t[0]), 0.3, 21, 5, params, q_cap=8, u_cap=128,
+                               want_visits=True) for h in (g, f)]
+        np.testing.assert_array_equal(q[0]["u"], q[1]["u"])
+        np.testing.assert_array_equal(q[0]["visits"], q[1]["visits"])
+        srv = pw.pw_server_create(g.handle, None, 1 << 24)
+        try:
+            tickets = [pw.pw_server_submit(srv, int(s[i]), int(t[i]), 0.3, 21, int(seeds[i])) for i in range(5)]
+            pw.pw_server_drain(srv, 60000)
+            np.testing.assert_array_equal([pw.pw_server_poll(srv, x)[1] for x in tickets], want)
+        finally:
+            pw.pw_server_destroy(srv)
