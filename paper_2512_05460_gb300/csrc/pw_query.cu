@@ -240,14 +240,17 @@ __device__ bool last_block(unsigned long long* arrived) {
 // divisions each, at 2 lanes per SM and clock) are computed by all lanes; they
 // are added in the oracle's order, probe after probe, the variances in lane 0
 // and the Q in lane 1.  (One thread per query took 72 us for any batch.)
+// Blocks of two warps for batches of up to 2,048 queries: eight warps' divisions
+// queued on one SM for 11 of 19 us.
 constexpr int kPilotThreads = 256;
+static int pilot_threads(int64_t nq) { return nq <= 2048 ? 64 : kPilotThreads; }
 __global__ void __launch_bounds__(kPilotThreads)
 pilot_budget_scan_kernel(int64_t nq, QPlan* plans, const QPlan* __restrict__ pilot, const double* __restrict__ pilot_s,
                          BudgetArgs A, const int4* __restrict__ node, ScanArgs S, unsigned long long* arrived) {
   constexpr int kWarps = kPilotThreads / 32;
   __shared__ double terms[kWarps][2][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t q = (int64_t)blockIdx.x * kWarps + warp;
+  const int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
   if (q < nq && pilot[q].K != 0) {
     const uint32_t K = pilot[q].K, R = pilot[q].R;
     const double* ps = pilot_s + 2 * pilot[q].probe_begin;
@@ -284,7 +287,7 @@ adapt_scan_kernel(int64_t nq, QPlan* plans, const double* __restrict__ qbuf, Bud
   constexpr int kWarps = kPilotThreads / 32;
   __shared__ double terms[kWarps][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t q = (int64_t)blockIdx.x * kWarps + warp;
+  const int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
   if (q < nq && plans[q].status == PW_OK && plans[q].K != 0 && plans[q].Bmax != 0) {
     const uint32_t B1 = plans[q].B, G = plans[q].G;
     const double* x = qbuf + plans[q].q_begin;
@@ -327,15 +330,18 @@ __global__ void zero_acc_kernel(ProbeAcc* __restrict__ acc, const Totals* __rest
     w[i] = 0ull;
 }
 
+// Last q with prefix[q] <= x, by a whole warp: 32 ways a round, so one load's
+// latency for up to 32 queries and two for 1,024.
 __device__ __forceinline__ int64_t find_segment(const unsigned long long* __restrict__ prefix, int64_t nq,
                                                 unsigned long long x) {
-  int64_t lo = 0, hi = nq;  // last q with prefix[q] <= x
-  while (hi - lo > 1) {
-    const int64_t mid = (lo + hi) >> 1;
-    if (prefix[mid] <= x)
-      lo = mid;
-    else
-      hi = mid;
+  const int64_t lane = (int64_t)(threadIdx.x & 31u);
+  int64_t lo = 0, n = nq;  // in [lo, lo + n), prefix[lo] <= x
+  while (n > 1) {
+    const int64_t step = (n + 31) / 32, at = lane * step;
+    const uint32_t le = __ballot_sync(0xffffffffu, at < n && prefix[lo + at] <= x);  // lanes 0 to some lane
+    const int64_t skip = (int64_t)(__popc(le) - 1) * step;
+    lo += skip;
+    n = n - skip < step ? n - skip : step;
   }
   return lo;
 }
@@ -395,11 +401,16 @@ __global__ void __launch_bounds__(kWalkThreads, DEBUG ? 1 : 3) walk_kernel(WalkA
   if (total == 0ull) return;
   __shared__ VisitPool pools[kWalkThreads / 32];
   VisitPool& pool = pools[threadIdx.x >> 5];
+  // Short tiles (up to 64 steps) of a launch with several for each warp are
+  // claimed one ahead: the claim's latency was a tenth of such a tile.
+  const unsigned long long warps = (unsigned long long)gridDim.x * (kWalkThreads / 32);
+  const bool ahead = total >= 4ull * warps && A.totals->visits <= 4096ull * total;
+  auto claim = [&]() { return lane == 0 ? atomicAdd(A.counter, 1ull) : 0ull; };
+  unsigned long long next = claim();
   for (;;) {
-    unsigned long long tile = 0;
-    if (lane == 0) tile = atomicAdd(A.counter, 1ull);
-    tile = __shfl_sync(0xffffffffu, tile, 0);
+    const unsigned long long tile = __shfl_sync(0xffffffffu, next, 0);
     if (tile >= total) return;
+    if (ahead) next = claim();
     const int64_t q = find_segment(A.tile_prefix, A.nq, tile);
     const QPlan& P = A.plans[q];
     const uint32_t chunks = P.chunks, R = P.R;
@@ -420,12 +431,17 @@ __global__ void __launch_bounds__(kWalkThreads, DEBUG ? 1 : 3) walk_kernel(WalkA
       sum_add(sum, U);
     }
     sum_warp_reduce(sum);
+    if (!ahead) next = claim();
     if (lane != 0) continue;
     if (PILOT) {
       double S1, S2;
       sum_round(sum.d, S1, S2);
       A.q[2 * (P.probe_begin + kl)] = S1;
       A.q[2 * (P.probe_begin + kl) + 1] = S2;
+    } else if (chunks == 1u) {  // the tile is the probe
+      double S1, S2;
+      sum_round(sum.d, S1, S2);
+      A.q[P.probe_begin + kl] = u_statistic(S1, S2, R);
     } else {
       ProbeAcc* pa = A.acc + P.acc_begin + kl;
       sum_atomic_add(pa->d, sum);
@@ -440,6 +456,50 @@ __global__ void __launch_bounds__(kWalkThreads, DEBUG ? 1 : 3) walk_kernel(WalkA
         A.q[P.probe_begin + kl] = u_statistic(S1, S2, R);
       }
     }
+  }
+}
+
+// Pilot of a few queries: a block's eight warps take 4 of a pilot probe's 32
+// replicas each.  64 probes a query leave the GPU nearly empty, so a tile's
+// latency is the stage's time; with 4 replicas a warp's pool holds one node a
+// lane, about 4 Feistel passes for 4 steps instead of 12.  One query on a
+// 10^5-node graph, L = 200: 349 us with a warp per probe, 110 so.
+template <WalkAccess ACCESS>
+__global__ void __launch_bounds__(kWalkThreads, 2) pilot_spread_kernel(WalkArgs A) {
+  const auto gr = GraphOf<ACCESS>::get(A);
+  __shared__ VisitPool pools[kWalkThreads / 32];
+  __shared__ unsigned long long sums[kSumDigits];
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  VisitPool& pool = pools[warp];
+  const unsigned long long total = A.totals->tiles;  // a tile is a probe
+  for (unsigned long long tile = blockIdx.x; tile < total; tile += gridDim.x) {
+    if (threadIdx.x < kSumDigits) sums[threadIdx.x] = 0ull;
+    __syncthreads();
+    const int64_t q = find_segment(A.tile_prefix, A.nq, tile);
+    const QPlan& P = A.plans[q];
+    const uint32_t R = P.R, k = (uint32_t)(tile - P.tile_begin);
+    const Probe pr = make_probe_warp(A.n, P.seed, k, A.probe_tag);
+    if (lane == 0) pool.probe = pr;
+    const uint32_t share = (R + 7u) / 8u, first = warp * share;
+    const uint32_t m = first >= R ? 0u : (R - first < share ? R - first : share);
+    const uint64_t pair = (uint64_t)k * R + first + lane;
+    const float U = walk_pair_visit<false>(gr, nullptr, A.walk_tag, pool, P.s, P.t, P.L, P.seed, pair, m, lane);
+    SumDigits sum;
+    sum_clear(sum);
+    if (lane < m) sum_add(sum, U);
+    sum_warp_reduce(sum);
+    if (lane == 0) sum_atomic_add(sums, sum);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      long long d[kSumDigits];
+#pragma unroll
+      for (int j = 0; j < kSumDigits; ++j) d[j] = (long long)sums[j];
+      double S1, S2;
+      sum_round(d, S1, S2);
+      A.q[2 * (P.probe_begin + k)] = S1;
+      A.q[2 * (P.probe_begin + k) + 1] = S2;
+    }
+    __syncthreads();
   }
 }
 
@@ -633,12 +693,23 @@ __device__ __forceinline__ double block_mean(const double* __restrict__ x, uint3
   return __ddiv_rn(sum, (double)B);
 }
 
+// Monotone 64-bit key of a finite double; -0 and +0 have one key.
+__device__ __forceinline__ long long order_key(double v) {
+  const long long b = __double_as_longlong(__dadd_rn(v, 0.0));
+  return b >= 0 ? b : (long long)(0x8000000000000000ull - (unsigned long long)b);
+}
+
 // Median of the G block means of B contiguous probes (Eq. final-estimator).
 // The middle values are found by rank (ties in index order), every thread
-// comparing its means with all: one thread's insertion sort took 20 us at G = 37.
+// comparing its means with all, as integers: FP64 compares go through a pipe of
+// 2 lanes per clock.  A query's values pass through shared memory when they fit
+// (coalesced loads; the additions keep index order).  One thread's insertion
+// sort took 20 us at G = 37; the whole kernel takes 5.
+constexpr uint32_t kMomStaged = 1920;
 __global__ void mom_kernel(const QPlan* __restrict__ plans, const double* __restrict__ qbuf,
                            double* __restrict__ beta, int32_t* __restrict__ status) {
-  __shared__ double means[4096];
+  __shared__ long long keys[4096];
+  __shared__ double staged[kMomStaged];
   __shared__ double mid[2];
   const int64_t q = blockIdx.x;
   const QPlan& P = plans[q];
@@ -649,17 +720,33 @@ __global__ void mom_kernel(const QPlan* __restrict__ plans, const double* __rest
     }
     return;
   }
-  const uint32_t G = P.G;
-  for (uint32_t g = threadIdx.x; g < G; g += blockDim.x)
-    means[g] = block_mean(qbuf + P.q_begin + (uint64_t)g * P.B, P.B);
+  const uint32_t G = P.G, B = P.B;
+  const double* x = qbuf + P.q_begin;
+  const uint64_t K = (uint64_t)G * B;
+  if (K <= kMomStaged) {
+    for (uint32_t k = threadIdx.x; k < (uint32_t)K; k += blockDim.x) staged[k] = x[k];
+    __syncthreads();
+  }
+  auto mean = [&](uint32_t g) {
+    return K <= kMomStaged ? block_mean(staged + g * B, B) : block_mean(x + (uint64_t)g * B, B);
+  };
+  double own = 0.0;  // this thread's first mean; others are few and computed again
+  for (uint32_t g = threadIdx.x; g < G; g += blockDim.x) {
+    const double v = mean(g);
+    if (g == threadIdx.x) own = v;
+    keys[g] = order_key(v);
+  }
   __syncthreads();
   const uint32_t hi = G / 2, lo = (G & 1u) ? hi : hi - 1;
   for (uint32_t g = threadIdx.x; g < G; g += blockDim.x) {
-    const double v = means[g];
+    const long long v = keys[g];
     uint32_t rank = 0;
-    for (uint32_t j = 0; j < G; ++j) rank += (means[j] < v || (means[j] == v && j < g)) ? 1u : 0u;
-    if (rank == lo) mid[0] = v;
-    if (rank == hi) mid[1] = v;
+    for (uint32_t j = 0; j < G; ++j) rank += (keys[j] < v || (keys[j] == v && j < g)) ? 1u : 0u;
+    if (rank == lo || rank == hi) {
+      const double m = g == threadIdx.x ? own : mean(g);
+      if (rank == lo) mid[0] = m;
+      if (rank == hi) mid[1] = m;
+    }
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -755,6 +842,23 @@ static int grid_of(pw_graph* g, WalkFn fn, int threads, size_t smem) {
   const int grid = g->sm_count * (nb > 0 ? nb : 1);
   g->grids[key] = grid;
   return grid;
+}
+
+static WalkFn spread_fn(WalkAccess access) {
+  return access == WalkAccess::kFused   ? pilot_spread_kernel<WalkAccess::kFused>
+         : access == WalkAccess::kSplit ? pilot_spread_kernel<WalkAccess::kSplit>
+                                        : pilot_spread_kernel<WalkAccess::kRanked>;
+}
+
+// The pilot's walks: a block per probe while all probes' blocks fit the GPU twice over.
+static pw_status launch_walk(pw_graph* g, cudaStream_t stream, const WalkArgs& a, bool debug, bool pilot);
+static pw_status launch_pilot(pw_graph* g, cudaStream_t stream, const WalkArgs& a, int64_t probes) {
+  if (probes > 2ll * g->sm_count) return launch_walk(g, stream, a, false, true);
+  const cudaError_t e =
+      launch_with_window(g, spread_fn(g->access), (int)probes, kWalkThreads, 0, stream, a);
+  count_launch();
+  PW_CUDA_TRY(e);
+  return PW_OK;
 }
 
 static pw_status launch_walk(pw_graph* g, cudaStream_t stream, const WalkArgs& a, bool debug, bool pilot) {
@@ -880,7 +984,8 @@ static pw_status enqueue_walks(pw_graph* g, int64_t count, const QueryArrays& Q,
     count_launch();
   }
   PW_CUDA_TRY(cudaGetLastError());
-  const int warp_blocks = (int)((count + kPilotThreads / 32 - 1) / (kPilotThreads / 32));
+  const int wthreads = pilot_threads(count);
+  const int warp_blocks = (int)((count + wthreads / 32 - 1) / (wthreads / 32));
   if (pilot) {
     wa.plans = B.pplans;
     wa.tile_prefix = pprefix;
@@ -893,12 +998,12 @@ static pw_status enqueue_walks(pw_graph* g, int64_t count, const QueryArrays& Q,
     prof_begin(g, stream, &ev);
     wa.pilot = 1;
     wa.table_prefix = pprefix + (nq + 1);
-    if ((st = team_pilot ? launch_table(g, stream, wa, false) : launch_walk(g, stream, wa, false, true)) != PW_OK)
+    if ((st = team_pilot ? launch_table(g, stream, wa, false) : launch_pilot(g, stream, wa, count * ba.K0)) != PW_OK)
       return st;
     wa.pilot = 0;
     prof_end(g, stream, ev, 1);
     if (g->prof.enabled) g->prof.pilot_transitions += 2ull * nq * (uint64_t)ba.K0 * (uint64_t)ba.R0;
-    pilot_budget_scan_kernel<<<warp_blocks, kPilotThreads, 0, stream>>>(count, B.plans, B.pplans, B.pilot_s, ba,
+    pilot_budget_scan_kernel<<<warp_blocks, wthreads, 0, stream>>>(count, B.plans, B.pplans, B.pilot_s, ba,
                                                                         g->d_node, main_scan, B.counters + 3);
     count_launch();
     PW_CUDA_TRY(cudaGetLastError());
@@ -952,7 +1057,7 @@ static pw_status enqueue_walks(pw_graph* g, int64_t count, const QueryArrays& Q,
     ScanArgs second = main_scan;
     second.totals = B.totals + 2;
     second.keep_q = 1;
-    adapt_scan_kernel<<<warp_blocks, kPilotThreads, 0, stream>>>(count, B.plans, B.q, ba, g->d_node, second,
+    adapt_scan_kernel<<<warp_blocks, wthreads, 0, stream>>>(count, B.plans, B.q, ba, g->d_node, second,
                                                                  B.counters + 5);
     count_launch();
     const cudaError_t e = cudaGetLastError();

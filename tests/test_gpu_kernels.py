@@ -176,3 +176,21 @@ def test_ranked_records(pw):
             np.testing.assert_array_equal([pw.pw_server_poll(srv, x)[1] for x in tickets], want)
         finally:
             pw.pw_server_destroy(srv)
+
+
+@pytest.mark.parametrize("K0,R0", [(1, 2), (5, 7), (64, 8), (64, 9), (63, 31), (64, 32), (400, 32)])
+def test_pilot_forms(pw, oracle_lib, K0, R0):
+    """The pilot by a block per probe (few probes) and by a warp per probe, with
+    replica counts that leave some of the block's warps without any: the budget
+    and the estimate of one query and of several against the oracle."""
+    host = barabasi_albert(3000, 3, 5)
+    params, cfg = pw.make_params(pilot_K0=K0, pilot_R0=R0), oracle.budget_cfg(K0=K0, R0=R0)
+    with pw.Graph(host.row_ptr, host.col_idx) as g:
+        for L in (0, 5):
+            b = oracle.budget(host, 3, 2999, 0.4, L, 11, cfg)
+            assert pw.pw_budget(g.handle, 3, 2999, 0.4, L, 11, params) == {k: b[k] for k in "BGKR"}
+            want = oracle.query(host, 3, 2999, 0.4, L, 11, cfg)["beta"]
+            assert pw.pw_query(g.handle, 3, 2999, 0.4, L, 11, params) == want
+            many, _ = pw.pw_query_batch(g.handle, np.full(9, 3), np.full(9, 2999), 0.4, L,
+                                        np.full(9, 11, np.uint64), params)
+            np.testing.assert_array_equal(many, want)
