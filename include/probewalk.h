@@ -405,8 +405,9 @@ pw_status pw_profile(pw_graph* g, int32_t enable, int32_t reset, pw_profile_stat
  * the policy and window checks below run at the caller's own budget, where a
  * sample of 32 queries or more stands for the batch far better than 8),
  * params' G, and R = 1024 replicas, each run after one untimed
- * warm-up: the per-visit kernel; the per-probe shared-memory table with
- * blocks of 256, 512 and 1024 threads, keeping the fastest; and that table
+ * warm-up: the per-visit kernel; the per-probe shared-memory table (with
+ * blocks of 512 and of 1024 threads, keeping the faster, on graphs of more than
+ * 278,528 nodes; smaller ones have one form, of 256); and that table
  * kernel again at R = 256 (the same probes, a quarter of the visits).  The
  * kept block size is stored in the graph and used by every later batch.  From the main walk kernels'
  * CUDA-event time of the kept runs it fits

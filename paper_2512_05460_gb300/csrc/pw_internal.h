@@ -44,7 +44,7 @@ struct Totals {
   unsigned long long probes;        // all probes (Q slots)
   unsigned long long steps;         // sum of K * R * L (walk pairs times length)
   unsigned long long visits;        // sum of 2 K R (L + 1)
-  unsigned long long team;          // warps per probe of the team table kernel (1, 2, 4 or 8)
+  unsigned long long team;          // warps per probe of the team table kernel (4 or 8)
   unsigned long long pad[1];
 };
 
@@ -129,8 +129,8 @@ struct pw_graph {
   pw::WalkAccess access = pw::WalkAccess::kFused;  // the layout's form that walks read
   cudaStream_t stream = nullptr;
   std::map<std::pair<const void*, size_t>, int> grids;  // persistent grid per walk kernel and shared memory
-  // Table-kernel block size (pw_autotune; 0: by shared memory, else 256, 512
-  // or 1024 threads).
+  // Table-kernel block size (pw_autotune; 0: by shared memory, else 256 (the
+  // team kernel), 512 or 1024 threads).
   int table_threads = 0;
   int walk_policy = 0;  // walk_mode 0 means: 0 the cost model per query, 1 all per-visit, 2 all table
   // L2 access-policy window of the walk and server launches

@@ -88,8 +88,10 @@ struct ModeArgs {
   double visit_gain;  // saving per visit when entries come from the table
 };
 
-// Graphs of up to this many nodes run their table probes in the team kernel.
-constexpr int64_t kTeamNodes = 4096;
+// Graphs of up to this many nodes (tables of 34 KB) run their table probes in the
+// team kernel.
+constexpr int64_t kTeamNodes = 278528;
+constexpr size_t kTeamTableBytes = 33 * 1024;  // tables of one block: two up to 131,072 nodes, then one of up to 34 KB
 
 struct ScanArgs {
   QPlan* plans;
@@ -99,6 +101,7 @@ struct ScanArgs {
   int32_t keep_q;      // the second stage of ADAPTIVE queries: the Q slots stay where the first stage put them
   int32_t g0, g1;      // g1 > 0: a sharded query keeps only median-of-means blocks [g0, g1)
   int32_t warps;       // resident warps of the team table kernel
+  int32_t team_min;    // fewest warps per team: the tables of a block's teams fit its shared memory
 };
 
 // Walk mode and offsets of every query, by one block of at most 1024 threads.
@@ -178,9 +181,9 @@ __device__ void scan_plans(const ScanArgs& S, int64_t nq) {
         if (j == 6) T->probes = x;
         if (j == 2) table_probes = x;
         if (j == 7) {
-          // warps per table probe: the fewest that make four waves of probes over
-          // the resident warps, and no more than a probe has tiles
-          unsigned long long team = 1;
+          // warps per table probe: at least team_min, and as many as make four waves
+          // of probes over the resident warps, but no more than a probe has tiles
+          unsigned long long team = (unsigned long long)S.team_min;
           while (team < 8 && table_probes * team < 4ull * S.warps && table_probes * team < x) team *= 2;
           T->team = team;
         }
@@ -510,10 +513,10 @@ __global__ void __launch_bounds__(kWalkThreads, 2) pilot_spread_kernel(WalkArgs 
 // digits, and the block writes the probe's Q_R.  Same values as the per-visit
 // kernel; cheaper whenever a probe's walks visit more nodes than the Feistel
 // domain has (2 R (L+1) > 2^b).
-// THREADS: 256 (five blocks per SM for small tables), 512 or 1024 (one or two
-// blocks per SM with up to 200 KB of table, still 32 warps).
+// THREADS: 512 or 1024 (two or one blocks per SM with up to 200 KB of table).
+// For graphs beyond the team kernel's.
 template <bool DEBUG, WalkAccess ACCESS, int THREADS>
-__global__ void __launch_bounds__(THREADS, THREADS == 256 ? 5 : (THREADS == 512 ? 2 : 1)) walk_table_kernel(WalkArgs A) {
+__global__ void __launch_bounds__(THREADS, THREADS == 512 ? 2 : 1) walk_table_kernel(WalkArgs A) {
   const auto gr = GraphOf<ACCESS>::get(A);
   extern __shared__ uint32_t tab[];
   __shared__ unsigned long long sh_probe;
@@ -536,7 +539,9 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 5 : (THREADS == 512 
     const QPlan& P = A.plans[q];
     const uint32_t kl = (uint32_t)(j - P.table_begin);
     const uint32_t k = P.k_begin + kl;
-    build_probe_table(make_probe(n, P.seed, k, A.probe_tag), tab, n);
+    if (threadIdx.x < 2) tab[(n + 31u) / 32u + threadIdx.x] = 0xFFFFFFFFu;
+    __syncthreads();
+    build_probe_table(make_probe(n, P.seed, k, A.probe_tag), tab, n, threadIdx.x, THREADS);
     __syncthreads();
     const ZTable zp = table_reader(tab, n);
     const uint32_t R = P.R, chunks = P.chunks;
@@ -574,23 +579,25 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 5 : (THREADS == 512 
   }
 }
 
-// Table kernel of graphs of few nodes (kTeamNodes): a team of 1, 2, 4 or 8 of a
-// block's warps (Totals::team) claims a probe, builds its table through the
-// warps' pools and runs its tiles.  With a block per probe, seven of 256 threads
-// built a 200-node table one after another, warps without a tile waited at three
-// barriers a probe (66 % of the stalls), and tiles of few steps paid for 110
-// shuffles each: 64 queries on a 200-node graph took 1.28 ms, 0.84 with teams (a
-// probe's table 18 ns of the GPU, 2.6 with teams).  Up to 4,096 nodes the eight
-// tables of a block take 4 KB.  Also the pilot walks of graphs of up to
-// kTeamPilotNodes, (S1, S2) per probe: one query 113 us, 93 so; building 1,024
-// entries takes a warp as long as 20 steps of per-visit walks.
+// Table kernel of graphs whose tables are up to 34 KB (kTeamNodes): a team of
+// four or eight of a block's warps (Totals::team) claims a probe, builds its
+// table and runs its tiles.  With a block per probe, seven of 256 threads built a
+// 200-node table one after another, warps without a tile waited at three barriers
+// a probe (66 % of the stalls), and tiles of few steps paid for 110 shuffles
+// each.  Four blocks per SM (64 registers): five (48, spilling) are 8 to 30 %
+// slower.  Walk stage, a block of 256 per probe -> teams: 64 queries on 200 nodes
+// 1.19 -> 0.7 ms; 33 at L = 60 on 20,001 nodes 5.97 -> 5.27 ms; 16 at L = 200 on
+// 10^5 nodes 59.3 -> 57.5 ms; 262,000 nodes 65.5 -> 64.0 ms.  Teams of two are 5 %
+// better than four at 12 tiles a probe and 14 % worse at 5; of one, worse.
+// Also the pilot walks of graphs of up to kTeamPilotNodes, (S1, S2) per probe:
+// building 1,024 entries takes less than 20 steps of per-visit walks.
 constexpr int64_t kTeamPilotNodes = 1024;
 constexpr uint32_t kTeamWarps = 8;
 template <bool DEBUG, WalkAccess ACCESS>
 __global__ void __launch_bounds__(kTeamWarps * 32, DEBUG ? 1 : 4) walk_team_kernel(WalkArgs A) {
   const auto gr = GraphOf<ACCESS>::get(A);
   __shared__ VisitPool pools[kTeamWarps];
-  __shared__ uint32_t tabs[kTeamWarps][kTeamNodes / 32 + 2];
+  extern __shared__ uint32_t tabs[];  // one table per team
   __shared__ unsigned long long sums[kTeamWarps][kSumDigits];
   __shared__ unsigned long long claims[kTeamWarps];
   const unsigned long long total = A.totals->table_probes;
@@ -598,9 +605,9 @@ __global__ void __launch_bounds__(kTeamWarps * 32, DEBUG ? 1 : 4) walk_team_kern
   const uint32_t lane = threadIdx.x & 31u, size = (uint32_t)A.totals->team;
   const uint32_t team = (threadIdx.x >> 5) / size, warp = (threadIdx.x >> 5) % size;
   VisitPool& pool = pools[threadIdx.x >> 5];
-  uint32_t* tab = tabs[team];
-  unsigned long long* sum_of = sums[team];
   const uint32_t n = A.n;
+  uint32_t* tab = tabs + team * table_words(n);
+  unsigned long long* sum_of = sums[team];
   auto sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(team + 1u), "r"(size * 32u) : "memory"); };
   for (;;) {
     if (warp == 0) {
@@ -618,7 +625,10 @@ __global__ void __launch_bounds__(kTeamWarps * 32, DEBUG ? 1 : 4) walk_team_kern
     const Probe pr = make_probe_warp(n, P.seed, k, A.probe_tag);
     if (lane == 0) pool.probe = pr;
     __syncwarp();
-    build_probe_table_team(pool, tab, n, warp, size, lane);
+    if (n >= 2048u * size)  // two words and more per lane: no pool needed to keep the lanes busy
+      build_probe_table(pr, tab, n, warp * 32u + lane, size * 32u);
+    else
+      build_probe_table_team(pool, tab, n, warp, size, lane);
     sync();
     const ZTable zp = table_reader(tab, n);
     const uint32_t R = P.R, chunks = P.chunks;
@@ -794,13 +804,12 @@ void prof_end(pw_graph* g, cudaStream_t stream, cudaEvent_t a, int kind) {
 static size_t table_bytes(const pw_graph* g) { return sizeof(uint32_t) * (size_t)table_words((uint32_t)g->n); }
 static constexpr size_t kMaxTableBytes = 200 * 1024;
 
-// Table-kernel block size by shared memory: 256 threads up to 32 KB a table (five
-// blocks per SM; at 41 KB and R = 1024 five tables left the gathers 20 KB of L1
-// and took 64 ms where two blocks of 512 took 30, at 24 KB 7.8 against 8.0), 512
-// while two tables fit, else 1024.
+// Table-kernel block size beyond the team kernel: 512 threads while two tables
+// fit per SM, else 1024.  (Five 41 KB tables per SM left the gathers 20 KB of L1
+// and took 64 ms where two blocks of 512 took 30.)
 static int default_table_threads(const pw_graph* g) {
-  const size_t per_block = table_bytes(g) + 2048;
-  return per_block <= ((size_t)34 << 10) ? 256 : (2 * per_block <= ((size_t)228 << 10) ? 512 : 1024);
+  if (g->n <= kTeamNodes) return (int)kTeamWarps * 32;
+  return 2 * (table_bytes(g) + 2048) <= ((size_t)228 << 10) ? 512 : 1024;
 }
 
 using WalkFn = void (*)(WalkArgs);
@@ -816,13 +825,11 @@ static WalkFn walk_fn(bool debug, bool pilot, WalkAccess access) {
                                         : walk_fn_of<WalkAccess::kRanked>(debug, pilot);
 }
 
-// The table kernel of a launch (DEBUG builds exist only at 256 threads).
+// The table kernel of a launch (DEBUG builds exist only at 512 threads).
 template <WalkAccess ACCESS>
 static WalkFn table_fn_of(bool debug, int threads) {
-  if (debug) return walk_table_kernel<true, ACCESS, 256>;
-  return threads == 1024  ? walk_table_kernel<false, ACCESS, 1024>
-         : threads == 512 ? walk_table_kernel<false, ACCESS, 512>
-                          : walk_table_kernel<false, ACCESS, 256>;
+  if (debug) return walk_table_kernel<true, ACCESS, 512>;
+  return threads == 1024 ? walk_table_kernel<false, ACCESS, 1024> : walk_table_kernel<false, ACCESS, 512>;
 }
 static WalkFn table_fn(bool debug, WalkAccess access, int threads) {
   return access == WalkAccess::kFused   ? table_fn_of<WalkAccess::kFused>(debug, threads)
@@ -874,26 +881,36 @@ static int table_threads(const pw_graph* g) {
 }
 
 // The team table kernel of a graph, its grid, and whether the graph uses it.
-static WalkFn team_fn(bool debug, WalkAccess access) {  // ranked arrays belong to larger graphs
-  if (debug)
-    return access == WalkAccess::kFused ? walk_team_kernel<true, WalkAccess::kFused>
-                                        : walk_team_kernel<true, WalkAccess::kSplit>;
-  return access == WalkAccess::kFused ? walk_team_kernel<false, WalkAccess::kFused>
-                                      : walk_team_kernel<false, WalkAccess::kSplit>;
+template <bool DEBUG>
+static WalkFn team_fn_of(WalkAccess access) {
+  return access == WalkAccess::kFused   ? walk_team_kernel<DEBUG, WalkAccess::kFused>
+         : access == WalkAccess::kSplit ? walk_team_kernel<DEBUG, WalkAccess::kSplit>
+                                        : walk_team_kernel<DEBUG, WalkAccess::kRanked>;
 }
-static int team_grid(pw_graph* g) { return grid_of(g, team_fn(false, g->access), kTeamWarps * 32, 0); }
+static WalkFn team_fn(bool debug, WalkAccess access) {
+  return debug ? team_fn_of<true>(access) : team_fn_of<false>(access);
+}
+// Fewest warps per team, four or so many that a block's tables fit
+// kTeamTableBytes, and the shared memory they take.
+static int team_min(const pw_graph* g) {
+  int team = 4;
+  while (team < (int)kTeamWarps && table_bytes(g) * (kTeamWarps / team) > kTeamTableBytes) team *= 2;
+  return team;
+}
+static size_t team_bytes(const pw_graph* g) { return table_bytes(g) * (kTeamWarps / team_min(g)); }
+static int team_grid(pw_graph* g) { return grid_of(g, team_fn(false, g->access), kTeamWarps * 32, team_bytes(g)); }
 
 static pw_status launch_table(pw_graph* g, cudaStream_t stream, const WalkArgs& a, bool debug) {
   if (g->n <= kTeamNodes) {
     const WalkFn fn = team_fn(debug, g->access);
     const cudaError_t e =
-        launch_with_window(g, fn, grid_of(g, fn, kTeamWarps * 32, 0), kTeamWarps * 32, 0, stream, a);
+        launch_with_window(g, fn, grid_of(g, fn, kTeamWarps * 32, team_bytes(g)), kTeamWarps * 32, team_bytes(g), stream, a);
     count_launch();
     PW_CUDA_TRY(e);
     return PW_OK;
   }
   const size_t smem = table_bytes(g);
-  const int threads = debug ? 256 : table_threads(g);
+  const int threads = debug ? 512 : table_threads(g);
   const WalkFn fn = table_fn(debug, g->access, threads);
   const cudaError_t e = launch_with_window(g, fn, grid_of(g, fn, threads, smem), threads, smem, stream, a);
   count_launch();
@@ -963,10 +980,11 @@ static pw_status enqueue_walks(pw_graph* g, int64_t count, const QueryArrays& Q,
   const ModeArgs M{forced, table_ok ? 1 : 0, g->table_probe_cost, g->table_visit_gain};
   const bool team_pilot = g->n <= kTeamPilotNodes;
   const int warps = g->n <= kTeamNodes ? team_grid(g) * (int)kTeamWarps : 0;
+  const int tmin = g->n <= kTeamNodes ? team_min(g) : 1;
   ScanArgs main_scan{B.plans, prefix, B.totals, M, 0, sharded ? (int32_t)dbg->g_begin : 0,
-                     sharded ? (int32_t)dbg->g_end : 0, warps};
+                     sharded ? (int32_t)dbg->g_end : 0, warps, tmin};
   const ScanArgs pilot_scan{B.pplans, pprefix, B.totals + 1, ModeArgs{team_pilot ? 2 : 1, team_pilot ? 1 : 0, 0.0, 0.0},
-                            0, 0, 0, warps};
+                            0, 0, 0, warps, tmin};
   // plans and the first offsets: the pilot's, or the main walks' where there is no pilot
   const ScanArgs& first_scan = pilot ? pilot_scan : main_scan;
   QPlan* pplans = pilot ? B.pplans : nullptr;
@@ -1742,13 +1760,14 @@ pw_status pw_autotune(pw_graph* g, int64_t count, const int64_t* s, const int64_
     return tune_window();
   }
   out->table_available = 1;
-  // table kernel: block size
-  int best_threads = 256;
-  for (int threads : {256, 512, 1024}) {
+  // table kernel: block size (beyond the team kernel, whose is 256)
+  const std::vector<int> sizes = g->n <= kTeamNodes ? std::vector<int>{(int)kTeamWarps * 32} : std::vector<int>{512, 1024};
+  int best_threads = sizes[0];
+  for (int threads : sizes) {
     g->table_threads = threads;
     Run r;
     if ((st = timed(2, R_hi, &r)) != PW_OK) return st;
-    if (threads == 256 || r.d.walk_ms < dt.d.walk_ms) {
+    if (threads == sizes[0] || r.d.walk_ms < dt.d.walk_ms) {
       dt = r;
       best_threads = threads;
     }

@@ -228,7 +228,11 @@ __global__ void __launch_bounds__(kServerThreads, MINB) server_kernel(ServerArgs
     const uint32_t probe_tag = pilot ? kTagProbePilot : kTagProbe;
     const bool table = TABLE && !pilot && __ldcg(&S->use_table) != 0u;  // then nprobe == 1
     const uint32_t chunks = (R + 31u) / 32u;
-    if (TABLE && table) build_probe_table(make_probe(A.n, P.seed, k0, probe_tag), tab, A.n);
+    if (TABLE && table) {
+      if (threadIdx.x < 2) tab[(A.n + 31u) / 32u + threadIdx.x] = 0xFFFFFFFFu;
+      __syncthreads();
+      build_probe_table(make_probe(A.n, P.seed, k0, probe_tag), tab, A.n, threadIdx.x, kServerThreads);
+    }
     __syncthreads();
     // tiles of 32 replicas over the job's probes; each tile's exact sums go
     // into the digits of its probe j (any order gives the same digits)

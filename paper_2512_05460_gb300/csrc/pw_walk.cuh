@@ -265,16 +265,17 @@ __device__ __forceinline__ float walk_pair_table(const GR& gr, uint32_t* visits,
 }
 
 // z^(k) of every node into the shared-memory table: one Feistel cycle-walk
-// per node.  Each thread owns whole 32-node words and runs a flat queue (one
+// per node, by `threads` threads, of which this is number `tid`.  Each thread
+// owns whole 32-node words and runs a flat queue (one
 // Feistel pass per iteration; it moves to its next node when a pass lands in
 // [n]), so lanes stay busy even though cycle-walk lengths vary.  Nodes of the
 // zero set (pi >= n - r) are listed in the two words after the bits.
-__device__ __forceinline__ void build_probe_table(const Probe& pr, uint32_t* tab, uint32_t n) {
+// The caller sets the two zero-set words to 0xFFFFFFFF beforehand.
+__device__ __forceinline__ void build_probe_table(const Probe& pr, uint32_t* tab, uint32_t n, uint32_t tid,
+                                                  uint32_t threads) {
   const uint32_t nwords = (n + 31u) / 32u;
   uint32_t* zero = tab + nwords;
-  if (threadIdx.x < 2) zero[threadIdx.x] = 0xFFFFFFFFu;
-  __syncthreads();
-  uint32_t w = threadIdx.x, v = w * 32u, x = v, acc = 0;
+  uint32_t w = tid, v = w * 32u, x = v, acc = 0;
   uint32_t stop = n - v < 32u ? n : v + 32u;  // end of the word's nodes
   while (w < nwords) {
     x = feistel_once(pr, x);
@@ -283,7 +284,7 @@ __device__ __forceinline__ void build_probe_table(const Probe& pr, uint32_t* tab
       acc = __funnelshift_l(probe_sign(pr, x), acc, 1);
       if (++v == stop) {
         tab[w] = acc << ((w + 1u) * 32u - stop);  // a last word may hold fewer nodes
-        w += blockDim.x;
+        w += threads;
         v = w * 32u;
         stop = n - v < 32u ? n : v + 32u;
       }
@@ -293,13 +294,15 @@ __device__ __forceinline__ void build_probe_table(const Probe& pr, uint32_t* tab
 }
 
 // The same for a graph of few nodes by `warps` warps, of which this is number
-// `warp`, each taking up to 256 nodes at a time through its pool.
+// `warp`, each taking its share, up to 256 nodes at a time, through its pool.
 __device__ __forceinline__ void build_probe_table_team(VisitPool& pool, uint32_t* tab, uint32_t n, uint32_t warp,
                                                        uint32_t warps, uint32_t lane) {
-  constexpr uint32_t kBatch = 2u * kPoolSteps * 32u;
+  constexpr uint32_t kMost = 2u * kPoolSteps * 32u;
   const uint32_t n_active = pool.probe.n_active;
-  for (uint32_t base = warp * kBatch; base < n; base += warps * kBatch) {
-    const uint32_t count = n - base < kBatch ? n - base : kBatch;
+  const uint32_t share = (n / warps + 32u) & ~31u;  // whole words
+  const uint32_t batch = share < kMost ? share : kMost;
+  for (uint32_t base = warp * batch; base < n; base += warps * batch) {
+    const uint32_t count = n - base < batch ? n - base : batch;
     for (uint32_t i = lane; i < count; i += 32u) pool.node[i] = base + i;
     __syncwarp();
     if (pool.probe.rounds == 8u)
