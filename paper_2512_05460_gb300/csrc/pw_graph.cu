@@ -279,7 +279,7 @@ static void destroy(pw_graph* g) {
   if (g->stream) cudaStreamSynchronize(g->stream);
   if (g->l2_window || g->l2_limit_set) set_l2_window(g, 0);
   free_workspace(g->ws);
-  for (pw::DeviceBuffer* b : {&g->series.segs, &g->series.heavy, &g->series.arrived, &g->series.scratch}) free_buffer(*b);
+  for (pw::DeviceBuffer* b : {&g->series.rows, &g->series.segs, &g->series.heavy, &g->series.arrived, &g->series.scratch}) free_buffer(*b);
   for (auto& sp : g->prof.spans) {
     cudaEventDestroy(sp.a);
     cudaEventDestroy(sp.b);

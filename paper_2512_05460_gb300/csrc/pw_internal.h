@@ -90,10 +90,10 @@ struct GraphCache {
   uint64_t launches = 0;  // kernel launches in one replay
 };
 
-// Layout of the series steps on a graph: its heavy rows' segments, built by the
-// first pw_series_batch, and scratch kept between calls.
+// Layout of the series steps on a graph: its rows and heavy rows' segments, built
+// by the first pw_series_batch, and scratch kept between calls.
 struct SeriesPlan {
-  DeviceBuffer segs, heavy, arrived, scratch;
+  DeviceBuffer rows, segs, heavy, arrived, scratch;
   int32_t nseg = 0, nheavy = 0;
   bool ready = false;
 };

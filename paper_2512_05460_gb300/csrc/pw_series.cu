@@ -105,6 +105,7 @@ struct SeriesArgs {
   const int32_t* col;
   const int4* node;
   const float2* inv;
+  const int2* rows;       // {e_begin, entries} of each row, entries -1 for heavy rows; [n] = {0, -1}
   const int4* segs;       // {heavy row, e_begin, e_end, partial slot}
   const int4* heavy;      // {row, first partial slot, partial count, -}
   float2* partial;        // nseg x C
@@ -140,46 +141,50 @@ struct PairSum {
   }
 };
 
-// The first C neighbour ids of a row of len entries, one per lane of its part.
+// The first C neighbour ids of a row of len entries, one per lane of its part;
+// past the row's end the index of the zero row after x's last, n.
 template <int C>
-__device__ __forceinline__ int32_t series_ids(const int32_t* __restrict__ col, int32_t e0, int32_t len, uint32_t sub) {
-  return (int32_t)sub < len ? __ldg(col + e0 + (int32_t)sub) : 0;
+__device__ __forceinline__ uint32_t series_ids(const int32_t* __restrict__ col, int32_t e0, int32_t len, uint32_t sub,
+                                               uint32_t n) {
+  return (int32_t)sub < len ? (uint32_t)__ldg(col + e0 + (int32_t)sub) : n;
 }
 
 // Sum of x_u (column = lane mod C) over the entries [e0, e0 + len) of one row,
 // in CSR order; every lane of the warp calls, 32 / C rows at once.  `mine`: the
 // row's first ids (series_ids), the next C come with one coalesced load; up to 8
-// row loads are in flight.  Rows shorter than the warp's longest add zeros,
-// which leaves a sum unchanged.
+// row loads are in flight.  Rows shorter than the warp's longest add the zero
+// row, which leaves a sum unchanged.  An entry costs a shuffle, an address, a
+// load and 8 additions; a predicate and a zero for each had cost as much again.
 template <int C>
 __device__ __forceinline__ float2 series_row_sum(const float2* __restrict__ x, const int32_t* __restrict__ col,
-                                                 int32_t mine, int32_t e0, int32_t len, uint32_t sub) {
+                                                 uint32_t mine, int32_t e0, int32_t len, uint32_t sub, uint32_t n) {
   PairSum acc;
   const int32_t longest = C == 32 ? len : __reduce_max_sync(0xffffffffu, len);
+  const float2* mycol = x + sub;
   for (int32_t b = 0; b < longest; b += C) {
-    const int32_t cnt = len - b;
     const int32_t lim = longest - b < C ? longest - b : C;  // the same in the whole warp
-    const int32_t next = b + C < longest ? series_ids<C>(col, e0 + b + C, cnt - C, sub) : 0;
+    const uint32_t next = b + C < longest ? series_ids<C>(col, e0 + b + C, len - b - C, sub, n) : n;
     for (int32_t j = 0; j < lim; j += 8) {
+      const int32_t rem = lim - j;
       float2 v[8];
       auto load = [&](int q) {
-        const int32_t u = __shfl_sync(0xffffffffu, mine, j + q, C);
-        v[q] = j + q < cnt ? __ldg(x + (size_t)(uint32_t)u * C + sub) : make_float2(0.f, 0.f);
+        const uint32_t u = __shfl_sync(0xffffffffu, mine, j + q, C);
+        v[q] = __ldg(mycol + (size_t)u * C);
       };
-#pragma unroll
-      for (int q = 0; q < 4; ++q) load(q);
-      const bool more = C > 4 && j + 4 < lim;
-      if (more) {
-#pragma unroll
-        for (int q = 4; q < 8; ++q) load(q);
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc.add(v[q]);
-      if (more) {
-#pragma unroll
-        for (int q = 4; q < 8; ++q) acc.add(v[q]);
-      }
-      if (j + 8 < lim) acc.fold();
+      auto two = [&](int q) {
+        acc.add(v[q]);
+        acc.add(v[q + 1]);
+      };
+      load(0);
+      load(1);
+      if (rem > 2) load(2), load(3);
+      if (C > 4 && rem > 4) load(4), load(5);
+      if (C > 4 && rem > 6) load(6), load(7);
+      two(0);
+      if (rem > 2) two(2);
+      if (C > 4 && rem > 4) two(4);
+      if (C > 4 && rem > 6) two(6);
+      if (rem > 8) acc.fold();
     }
     if (b + C < longest) acc.fold();
     mine = next;
@@ -189,12 +194,13 @@ __device__ __forceinline__ float2 series_row_sum(const float2* __restrict__ x, c
 
 // One iteration over all rows.  ACC: 0 leaves h, 1 adds x_i and then x_{i+1},
 // 2 starts h as their sum.  The segments of heavy rows come first.
-// Bound by the latency of a row's loads on graphs in L2 and by L2 and HBM
-// bandwidth beyond; 5 blocks per SM (48 registers) against 4 (58) or 6 (40): 268,
-// 388 and 307 us a step on a 1000^2 grid.  Microseconds a step, before -> now:
-// 10^5-node power-law graph, 32 / 16 / 4 columns 168 -> 47 / 175 -> 29 / 168 ->
-// 19; R-MAT 2^20, 32 / 8 columns 1,498 -> 1,244 / 1,499 -> 377; 2000^2 grid, 32
-// columns 1,540 -> 1,142.
+// Bound by issue (two thirds of the slots) and the latency of a row's loads on
+// graphs in L2, by L2 and HBM bandwidth beyond; 5 blocks per SM (48 registers)
+// against 6 (40): 258 and 277 us a step on a 1000^2 grid.  Microseconds a step,
+// with a warp per row of up to 1,024 entries and always 32 columns -> now:
+// 10^5-node power-law graph, 32 / 16 / 4 columns 168 -> 44 / 175 -> 28 / 168 ->
+// 18; R-MAT 2^20, 32 / 8 columns 1,498 -> 1,110 / 1,499 -> 318; 2000^2 grid, 32
+// columns 1,540 -> 1,037.
 template <int C, int ACC>
 __global__ void __launch_bounds__(kSeriesThreads, 5) series_step_kernel(SeriesArgs A) {
   constexpr uint32_t kRows = 32 / C;
@@ -206,7 +212,12 @@ __global__ void __launch_bounds__(kSeriesThreads, 5) series_step_kernel(SeriesAr
   auto finish = [&](size_t at, float2 sum, float2 inv, float2 x, float2 h) {
     const float2 y = df_mul(sum, inv);
     A.y[at] = y;
-    if (ACC == 1) A.h[at] = df_add(df_add(h, x), y);
+    if (ACC == 1) {
+      PairSum sum_h{h.x, 0.f, h.y};
+      sum_h.add(x);
+      sum_h.add(y);
+      A.h[at] = sum_h.value();
+    }
     if (ACC == 2) A.h[at] = df_add(x, y);
   };
   uint32_t g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -215,7 +226,7 @@ __global__ void __launch_bounds__(kSeriesThreads, 5) series_step_kernel(SeriesAr
     const bool valid = i < (uint32_t)A.nseg;
     const int4 sg = valid ? __ldg(A.segs + i) : make_int4(0, 0, 0, 0);
     const int32_t len = sg.z - sg.y;
-    const float2 sum = series_row_sum<C>(A.x, A.col, series_ids<C>(A.col, sg.y, len, sub), sg.y, len, sub);
+    const float2 sum = series_row_sum<C>(A.x, A.col, series_ids<C>(A.col, sg.y, len, sub, A.n), sg.y, len, sub, A.n);
     if (valid) __stcg(A.partial + (size_t)sg.w * C + sub, sum);
     __threadfence();
     __syncwarp();
@@ -248,25 +259,23 @@ __global__ void __launch_bounds__(kSeriesThreads, 5) series_step_kernel(SeriesAr
   g -= seg_groups;
   uint32_t v = g * kRows + part;
   const uint32_t step = warps * kRows;
-  auto record = [&](uint32_t u) {  // {row start, entries}; rows of other warps and heavy ones have none
-    const int4 r = u < A.n ? __ldg(A.node + u) : make_int4(0, 0, 0, 0);
-    return make_int2(r.y, u < A.n ? (r.z <= kSeriesRow ? r.z : -1) : -1);
-  };
+  auto record = [&](uint32_t u) { return __ldg(A.rows + (u < A.n ? u : A.n)); };
   int2 r0 = record(v), r1 = record(v + step);
-  int32_t ids = series_ids<C>(A.col, r0.x, r0.y, sub);
+  uint32_t ids = series_ids<C>(A.col, r0.x, r0.y, sub, A.n);
+  size_t at = (size_t)v * C + sub;
   for (; g < row_groups; g += warps) {
     const bool light = r0.y >= 0;
-    const size_t at = (size_t)v * C + sub;
     const float2 inv = light ? __ldg(A.inv + v) : zero;
     const float2 x = ACC && light ? A.x[at] : zero, h = ACC == 1 && light ? A.h[at] : zero;
-    const int32_t ids_next = series_ids<C>(A.col, r1.x, r1.y, sub);
+    const uint32_t ids_next = series_ids<C>(A.col, r1.x, r1.y, sub, A.n);
     const int2 r2 = record(v + 2 * step);
-    const float2 sum = series_row_sum<C>(A.x, A.col, ids, r0.x, light ? r0.y : 0, sub);
+    const float2 sum = series_row_sum<C>(A.x, A.col, ids, r0.x, light ? r0.y : 0, sub, A.n);
     if (light) finish(at, sum, inv, x, h);
     r0 = r1;
     r1 = r2;
     ids = ids_next;
     v += step;
+    at += (size_t)step * C;
   }
 }
 
@@ -337,7 +346,9 @@ template <int C>
 static int series_pass(SeriesArgs A, float2* x_buf, float2* y_buf, const int2* st, int ncols, int32_t L, int grid,
                        int reduce_grid, double* block_sums, unsigned int* reduce_arrived, double* out,
                        cudaStream_t stream) {
-  cudaMemsetAsync(x_buf, 0, sizeof(float2) * (size_t)A.n * C, stream);
+  // x_0 and the zero rows after the last
+  cudaMemsetAsync(x_buf, 0, sizeof(float2) * ((size_t)A.n + 1) * C, stream);
+  cudaMemsetAsync(y_buf + (size_t)A.n * C, 0, sizeof(float2) * C, stream);
   series_seed_kernel<<<1, kSeriesCols, 0, stream>>>(x_buf, st, ncols, C, A.node);
   float2 *x = x_buf, *y = y_buf;
   for (int32_t i = 0; i < L; ++i) {
@@ -351,11 +362,12 @@ static int series_pass(SeriesArgs A, float2* x_buf, float2* y_buf, const int2* s
   return L + 2;
 }
 
-// Heavy rows' segments, laid out once per graph (they depend on its degrees only).
+// Rows and heavy rows' segments, laid out once per graph (they depend on its degrees only).
 static pw_status series_plan(pw_graph* g) {
   SeriesPlan& P = g->series;
   if (P.ready) return PW_OK;
   std::vector<int4> segs, heavy;
+  std::vector<int2> rows((size_t)g->n + 1, make_int2(0, -1));
   int64_t start = 0;
   int32_t slot = 0;
   for (int64_t v = 0; v < g->n; ++v) {
@@ -367,13 +379,17 @@ static pw_status series_plan(pw_graph* g) {
       for (int64_t e = start; e < start + d; e += size)
         segs.push_back(make_int4((int)heavy.size(), (int)e, (int)std::min<int64_t>(e + size, start + d), slot++));
       heavy.push_back(make_int4((int)v, first, slot - first, 0));
+    } else {
+      rows[(size_t)v] = make_int2((int)start, d);
     }
     start += d;
   }
   pw_status st;
+  if ((st = ensure_buffer(P.rows, sizeof(int2) * rows.size())) != PW_OK) return st;
   if ((st = ensure_buffer(P.segs, sizeof(int4) * segs.size())) != PW_OK) return st;
   if ((st = ensure_buffer(P.heavy, sizeof(int4) * heavy.size())) != PW_OK) return st;
   if ((st = ensure_buffer(P.arrived, sizeof(unsigned int) * (heavy.size() + 1))) != PW_OK) return st;
+  PW_CUDA_TRY(cudaMemcpyAsync(P.rows.ptr, rows.data(), sizeof(int2) * rows.size(), cudaMemcpyHostToDevice, g->stream));
   PW_CUDA_TRY(cudaMemcpyAsync(P.segs.ptr, segs.data(), sizeof(int4) * segs.size(), cudaMemcpyHostToDevice, g->stream));
   PW_CUDA_TRY(cudaMemcpyAsync(P.heavy.ptr, heavy.data(), sizeof(int4) * heavy.size(), cudaMemcpyHostToDevice,
                               g->stream));
@@ -431,7 +447,7 @@ extern "C" pw_status pw_series_batch(pw_graph* g, int64_t count, const int64_t* 
   const int reduce_grid = g->sm_count * 4;
   // x, y, h, 1/d, partial sums, the reduction's block sums, (s, t) and results
   auto align = [](size_t b) { return (b + 255) & ~(size_t)255; };
-  const size_t b_vec = align(sizeof(float2) * n * (size_t)most), b_inv = align(sizeof(float2) * n);
+  const size_t b_vec = align(sizeof(float2) * (n + 1) * (size_t)most), b_inv = align(sizeof(float2) * n);
   const size_t b_part = align(sizeof(float2) * (size_t)most * (size_t)P.nseg);
   const size_t b_sums = align(sizeof(double) * 2 * (size_t)most * (size_t)reduce_grid);
   const size_t b_st = align(sizeof(int2) * (size_t)count), b_out = align(sizeof(double) * (size_t)count);
@@ -458,6 +474,7 @@ extern "C" pw_status pw_series_batch(pw_graph* g, int64_t count, const int64_t* 
   A.inv = inv;
   A.col = g->d_col;
   A.node = g->d_node;
+  A.rows = (const int2*)P.rows.ptr;
   A.segs = (const int4*)P.segs.ptr;
   A.heavy = (const int4*)P.heavy.ptr;
   A.arrived = (unsigned int*)P.arrived.ptr;
