@@ -102,6 +102,7 @@ struct ScanArgs {
   int32_t g0, g1;      // g1 > 0: a sharded query keeps only median-of-means blocks [g0, g1)
   int32_t warps;       // resident warps of the team table kernel
   int32_t team_min;    // fewest warps per team: the tables of a block's teams fit its shared memory
+  Totals* host;        // pinned copy of the totals, or null
 };
 
 // Walk mode and offsets of every query, by one block of at most 1024 threads.
@@ -172,13 +173,18 @@ __device__ void scan_plans(const ScanArgs& S, int64_t nq) {
       sh[j][lane] = x - own;  // before this warp
       if (lane == 31) {
         Totals* T = S.totals;
-        if (j == 0) T->tiles = prefix[nq] = x;
-        if (j == 1) T->visit_probes = x;
-        if (j == 2) T->table_probes = prefix[(nq + 1) + nq] = x;
+        if (j == 0) prefix[nq] = x;
+        if (j == 2) prefix[(nq + 1) + nq] = x;
         if (j == 3 && !S.keep_q) prefix[2 * (nq + 1) + nq] = x;
-        if (j == 4) T->steps = x;
-        if (j == 5) T->visits = x;
-        if (j == 6) T->probes = x;
+        for (Totals* to : {T, S.host}) {
+          if (!to) continue;
+          if (j == 0) to->tiles = x;
+          if (j == 1) to->visit_probes = x;
+          if (j == 2) to->table_probes = x;
+          if (j == 4) to->steps = x;
+          if (j == 5) to->visits = x;
+          if (j == 6) to->probes = x;
+        }
         if (j == 2) table_probes = x;
         if (j == 7) {
           // warps per table probe: at least team_min, and as many as make four waves
@@ -216,11 +222,15 @@ __device__ void scan_plans(const ScanArgs& S, int64_t nq) {
 
 __global__ void __launch_bounds__(1024) scan_kernel(ScanArgs S, int64_t nq) { scan_plans(S, nq); }
 
-// A small batch's plans and their offsets in one launch of one block.  Up to
-// kFusedPlans queries: the FP64 divisions of more would queue up on one SM.
+// A small batch's plans, their offsets and the cleared counters in one launch of
+// one block.  Up to kFusedPlans queries: the FP64 divisions of more would queue up
+// on one SM.  A host-array batch of this size reads its queries from and writes
+// its results to pinned host memory: the copies of a few bytes each way, of the
+// totals and of the counters' zeros were four of a call's eleven operations.
 constexpr int64_t kFusedPlans = 256;
 __global__ void __launch_bounds__(kFusedPlans) plan_scan_kernel(int64_t nq, QueryArrays Q, BudgetArgs A, int64_t n, const int4* __restrict__ node,
-                                 QPlan* plans, QPlan* pilot, ScanArgs S) {
+                                 QPlan* plans, QPlan* pilot, ScanArgs S, unsigned long long* counters) {
+  if (threadIdx.x < 8) counters[threadIdx.x] = 0ull;
   for (int64_t q = threadIdx.x; q < nq; q += blockDim.x) plan_one(q, Q, A, n, node, plans, pilot);
   __syncthreads();
   scan_plans(S, nq);
@@ -608,7 +618,10 @@ __global__ void __launch_bounds__(kTeamWarps * 32, DEBUG ? 1 : 4) walk_team_kern
   const uint32_t n = A.n;
   uint32_t* tab = tabs + team * table_words(n);
   unsigned long long* sum_of = sums[team];
-  auto sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(team + 1u), "r"(size * 32u) : "memory"); };
+  auto sync = [&]() {  // the team's own barrier; its warps arrive whole
+    __syncwarp();
+    asm volatile("bar.sync %0, %1;" ::"r"(team + 1u), "r"(size * 32u) : "memory");
+  };
   for (;;) {
     if (warp == 0) {
       if (lane == 0) claims[team] = atomicAdd(A.counter, 1ull);
@@ -982,18 +995,19 @@ static pw_status enqueue_walks(pw_graph* g, int64_t count, const QueryArrays& Q,
   const int warps = g->n <= kTeamNodes ? team_grid(g) * (int)kTeamWarps : 0;
   const int tmin = g->n <= kTeamNodes ? team_min(g) : 1;
   ScanArgs main_scan{B.plans, prefix, B.totals, M, 0, sharded ? (int32_t)dbg->g_begin : 0,
-                     sharded ? (int32_t)dbg->g_end : 0, warps, tmin};
+                     sharded ? (int32_t)dbg->g_end : 0, warps, tmin, g->ws.host_totals};
   const ScanArgs pilot_scan{B.pplans, pprefix, B.totals + 1, ModeArgs{team_pilot ? 2 : 1, team_pilot ? 1 : 0, 0.0, 0.0},
-                            0, 0, 0, warps, tmin};
+                            0, 0, 0, warps, tmin, nullptr};
   // plans and the first offsets: the pilot's, or the main walks' where there is no pilot
   const ScanArgs& first_scan = pilot ? pilot_scan : main_scan;
   QPlan* pplans = pilot ? B.pplans : nullptr;
-  PW_CUDA_TRY(cudaMemsetAsync(B.counters, 0, 64, stream));
   if (count <= kFusedPlans) {
     const int threads = (int)((count + 31) / 32 * 32);
-    plan_scan_kernel<<<1, threads, 0, stream>>>(count, Q, ba, g->n, g->d_node, B.plans, pplans, first_scan);
+    plan_scan_kernel<<<1, threads, 0, stream>>>(count, Q, ba, g->n, g->d_node, B.plans, pplans, first_scan,
+                                                B.counters);
     count_launch();
   } else {
+    PW_CUDA_TRY(cudaMemsetAsync(B.counters, 0, 64, stream));
     const int qthreads = 128;
     budget_init_kernel<<<(int)((count + qthreads - 1) / qthreads), qthreads, 0, stream>>>(count, Q, ba, g->n, g->d_node,
                                                                                           B.plans, pplans);
@@ -1074,6 +1088,7 @@ static pw_status enqueue_walks(pw_graph* g, int64_t count, const QueryArrays& Q,
     // probes with their own offsets and totals (Q slots stay in place)
     ScanArgs second = main_scan;
     second.totals = B.totals + 2;
+    second.host = nullptr;
     second.keep_q = 1;
     adapt_scan_kernel<<<warp_blocks, wthreads, 0, stream>>>(count, B.plans, B.q, ba, g->d_node, second,
                                                                  B.counters + 5);
@@ -1169,7 +1184,7 @@ static pw_status device_total_K(pw_graph* g, int64_t count, const int64_t* d_s, 
   return PW_OK;
 }
 
-// Every stage of a batch whose scratch is sized, then a copy of its totals.
+// Every stage of a batch whose scratch is sized.
 static pw_status enqueue_batch(pw_graph* g, int64_t count, const int64_t* d_s, const int64_t* d_t,
                                const double* d_eps, const int32_t* d_L, const uint64_t* d_seeds,
                                const pw_params* params, const BudgetArgs& ba, const BatchBuffers& B, double* d_beta,
@@ -1177,7 +1192,6 @@ static pw_status enqueue_batch(pw_graph* g, int64_t count, const int64_t* d_s, c
   pw_status st;
   const QueryArrays Q{d_s, d_t, d_eps, d_L, d_seeds};
   if ((st = enqueue_walks(g, count, Q, params, ba, B, d_beta, d_status, stream, dbg)) != PW_OK) return st;
-  PW_CUDA_TRY(cudaMemcpyAsync(g->ws.host_totals, B.totals, sizeof(Totals), cudaMemcpyDeviceToHost, stream));
   st = prof_totals(g, B.totals, stream);
   if (st == PW_OK && ba.mode == PW_BUDGET_ADAPTIVE && !(dbg && dbg->budget_only)) st = prof_totals(g, B.totals + 2, stream);
   return st;
@@ -1271,15 +1285,18 @@ static pw_status graph_batch(pw_graph* g, int64_t count, const char* h, char* ho
     }
     const uint64_t before = pw_launch_count(0);
     PW_CUDA_TRY(cudaStreamBeginCapture(g->stream, cudaStreamCaptureModeThreadLocal));
-    char* d = (char*)ws.queries.ptr;
+    const bool direct = count <= kFusedPlans;  // reads and writes the pinned staging memory itself
+    const char* d = direct ? h : (const char*)ws.queries.ptr;
+    char* r = direct ? ho : (char*)ws.results.ptr;
     const size_t nq = (size_t)count;
-    cudaError_t e = cudaMemcpyAsync(d, h, in_bytes, cudaMemcpyHostToDevice, g->stream);
+    cudaError_t e = cudaSuccess;
+    if (!direct) e = cudaMemcpyAsync(ws.queries.ptr, h, in_bytes, cudaMemcpyHostToDevice, g->stream);
     st = e == cudaSuccess ? PW_OK : cuda_error(e, "graph input copy");
     if (st == PW_OK)
       st = enqueue_batch(g, count, (const int64_t*)d, (const int64_t*)(d + nq * 8), (const double*)(d + nq * 16),
                          (const int32_t*)(d + nq * 32), (const uint64_t*)(d + nq * 24), params, ba, B,
-                         (double*)ws.results.ptr, (int32_t*)((char*)ws.results.ptr + nq * 8), g->stream, nullptr);
-    if (st == PW_OK) {
+                         (double*)r, (int32_t*)(r + nq * 8), g->stream, nullptr);
+    if (st == PW_OK && !direct) {
       e = cudaMemcpyAsync(ho, ws.results.ptr, out_bytes, cudaMemcpyDeviceToHost, g->stream);
       if (e != cudaSuccess) st = cuda_error(e, "graph result copy");
     }
@@ -1325,10 +1342,11 @@ static pw_status host_batch(pw_graph* g, int64_t count, const int64_t* s, const 
   Workspace& ws = g->ws;
   const size_t nq = (size_t)count;
   const size_t in_bytes = nq * (8 + 8 + 8 + 8 + 4), out_bytes = nq * (8 + 4);
+  const size_t out_at = (in_bytes + 63) & ~(size_t)63;  // results in the staging memory
   BudgetArgs ba;
   pw_status st = resolve_budget(params, g, &ba, nullptr);
   if (st != PW_OK) return st;
-  if ((st = ensure_host_staging(ws, in_bytes + out_bytes + 64)) != PW_OK) return st;
+  if ((st = ensure_host_staging(ws, out_at + out_bytes + 64)) != PW_OK) return st;
   if ((st = ensure_buffer(ws.queries, in_bytes + 64)) != PW_OK) return st;
   if ((st = ensure_buffer(ws.results, out_bytes + 64)) != PW_OK) return st;
   PW_CUDA_TRY(cudaStreamWaitEvent(g->stream, ws.last_use, 0));
@@ -1345,10 +1363,12 @@ static pw_status host_batch(pw_graph* g, int64_t count, const int64_t* s, const 
   }
   memcpy(h + nq * 32, L, nq * 4);
   const size_t K = host_total_K(g, count, s, t, eps, L, ba);
-  char* d = (char*)ws.queries.ptr;
-  double* d_beta = (double*)ws.results.ptr;
-  int32_t* d_status = (int32_t*)((char*)ws.results.ptr + nq * 8);
-  char* ho = h + in_bytes;
+  char* ho = h + out_at;
+  const bool direct = count <= kFusedPlans;  // reads and writes the pinned staging memory itself
+  char* d = direct ? h : (char*)ws.queries.ptr;
+  char* r = direct ? ho : (char*)ws.results.ptr;
+  double* d_beta = (double*)r;
+  int32_t* d_status = (int32_t*)(r + nq * 8);
   if (!dbg && !g->prof.enabled) {
     st = graph_batch(g, count, h, ho, in_bytes, out_bytes, params, ba, K);
     if (st == PW_OK) {
@@ -1357,7 +1377,7 @@ static pw_status host_batch(pw_graph* g, int64_t count, const int64_t* s, const 
     }
     if (st != PW_PENDING) return st;  // PENDING: shape not seen twice yet, run it eagerly
   }
-  PW_CUDA_TRY(cudaMemcpyAsync(d, h, in_bytes, cudaMemcpyHostToDevice, g->stream));
+  if (!direct) PW_CUDA_TRY(cudaMemcpyAsync(d, h, in_bytes, cudaMemcpyHostToDevice, g->stream));
   st = run_batch(g, count, (const int64_t*)d, (const int64_t*)(d + nq * 8), (const double*)(d + nq * 16),
                  (const int32_t*)(d + nq * 32), (const uint64_t*)(d + nq * 24), params, d_beta, d_status, g->stream,
                  dbg, (int64_t)K);
@@ -1366,7 +1386,7 @@ static pw_status host_batch(pw_graph* g, int64_t count, const int64_t* s, const 
     PW_CUDA_TRY(cudaStreamSynchronize(g->stream));
     return PW_OK;
   }
-  PW_CUDA_TRY(cudaMemcpyAsync(ho, ws.results.ptr, out_bytes, cudaMemcpyDeviceToHost, g->stream));
+  if (!direct) PW_CUDA_TRY(cudaMemcpyAsync(ho, r, out_bytes, cudaMemcpyDeviceToHost, g->stream));
   PW_CUDA_TRY(cudaStreamSynchronize(g->stream));
   memcpy(beta, ho, nq * 8);
   memcpy(status, ho + nq * 8, nq * 4);
@@ -1997,7 +2017,6 @@ extern "C" pw_status pw_query_batch_noalloc(pw_graph* g, int64_t count, const in
   B.q = (double*)(base + o_q);
   B.acc = (ProbeAcc*)(base + o_acc);
   if ((st = enqueue_walks(g, count, Q, params, ba, B, d_beta_hat, d_status, stream, nullptr)) != PW_OK) return st;
-  PW_CUDA_TRY(cudaMemcpyAsync(g->ws.host_totals, B.totals, sizeof(Totals), cudaMemcpyDeviceToHost, stream));
   PW_CUDA_TRY(cudaEventRecord(g->ws.last_use, stream));
   return PW_OK;
 }
