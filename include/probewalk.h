@@ -405,10 +405,11 @@ pw_status pw_profile(pw_graph* g, int32_t enable, int32_t reset, pw_profile_stat
  * the policy and window checks below run at the caller's own budget, where a
  * sample of 32 queries or more stands for the batch far better than 8),
  * params' G, and R = 1024 replicas, each run after one untimed
- * warm-up: the per-visit kernel; the per-probe shared-memory table (with
- * blocks of 512 and of 1024 threads, keeping the faster, on graphs of more than
- * 278,528 nodes; smaller ones have one form, of 256); and that table
- * kernel again at R = 256 (the same probes, a quarter of the visits).  The
+ * warm-up: the per-visit kernel; the per-probe shared-memory table, and that
+ * table kernel again at R = 256 (the same probes, a quarter of the visits), on
+ * graphs of more than 278,528 nodes with blocks of 512 and of 1024 threads,
+ * keeping the faster at R = 2048 by extrapolation (smaller ones have one form, of
+ * 256).  The
  * kept block size is stored in the graph and used by every later batch.  From the main walk kernels'
  * CUDA-event time of the kept runs it fits
  *   per-visit:  t = visits * visit_ns
@@ -441,7 +442,7 @@ typedef struct pw_tune_result {
   double sample_ms[3];     /* walk-kernel time of the kept runs (per-visit; table at R = 1024; table at R = 256) */
   int32_t table_available; /* 1 when the probe table fits in shared memory */
   int32_t sample_mode;     /* walk kernel the fitted model picks for the sample: 1 per-visit, 2 table */
-  int32_t visit_occupancy; /* resident blocks of 256 per SM of the per-visit kernel: 3 */
+  int32_t visit_occupancy; /* resident blocks of 256 per SM of the per-visit kernel: 3, or 4 on large split graphs */
   int32_t table_threads;   /* table-kernel block size kept: 256, 512 or 1024 (0 when unavailable) */
   double policy_ms[3];     /* walk time of the sample at the caller's budget: per-query model, all per-visit, all table */
   int32_t policy;          /* the policy walk_mode 0 now follows: 0 per-query model, 1 all per-visit, 2 all table */

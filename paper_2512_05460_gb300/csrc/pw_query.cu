@@ -403,11 +403,13 @@ struct GraphOf<WalkAccess::kRanked> {
 };
 
 // 3 blocks per SM (80 registers, 9 KB of pools each, the rest of the SM's
-// memory caching the graph): 4 blocks (64 registers, some spilled) took 5.9 ps
-// a visit on a 2000^2 grid against 5.3, 6.2 against 5.8 on a 10^5-node graph,
-// and 9.8 against 10.2 on R-MAT 2^20.
+// memory caching the graph), 4 (64 registers, some spilled) on ranked graphs,
+// where the gathers' latency is most of a visit: 8.8 ps against 9.4 on R-MAT 2^20,
+// but 6.0 against 5.4 on a 2000^2 grid, 6.0 against 5.9 on a 10^5-node graph and
+// 19.8 against 19.5 on R-MAT 2^22.
 template <bool DEBUG, bool PILOT, WalkAccess ACCESS>
-__global__ void __launch_bounds__(kWalkThreads, DEBUG ? 1 : 3) walk_kernel(WalkArgs A) {
+__global__ void __launch_bounds__(kWalkThreads, DEBUG ? 1 : (ACCESS == WalkAccess::kRanked ? 4 : 3))
+walk_kernel(WalkArgs A) {
   const auto gr = GraphOf<ACCESS>::get(A);
   const uint32_t lane = threadIdx.x & 31u;
   const unsigned long long total = A.totals->tiles;
@@ -819,10 +821,17 @@ static constexpr size_t kMaxTableBytes = 200 * 1024;
 
 // Table-kernel block size beyond the team kernel: 512 threads while two tables
 // fit per SM, else 1024.  (Five 41 KB tables per SM left the gathers 20 KB of L1
-// and took 64 ms where two blocks of 512 took 30.)
+// and took 64 ms where two blocks of 512 took 30.)  One block of 1024 also on
+// ranked graphs with tables of over 60 KB, whose hub records a second table would
+// push out of L1: R-MAT 2^20 (79 KB) 4.5 ps a visit against 7.3, 115 ms against
+// 155 at R = 4096 and 48.6 against 49.1 at 1024 (at 256 it loses, 32 against 23,
+// but there visits without a table are cheaper still); at 41 KB two blocks stay
+// ahead, 30 against 35 ms.
 static int default_table_threads(const pw_graph* g) {
   if (g->n <= kTeamNodes) return (int)kTeamWarps * 32;
-  return 2 * (table_bytes(g) + 2048) <= ((size_t)228 << 10) ? 512 : 1024;
+  const size_t table = table_bytes(g);
+  if (2 * (table + 2048) > ((size_t)228 << 10)) return 1024;
+  return g->access == WalkAccess::kRanked && table > ((size_t)60 << 10) ? 1024 : 512;
 }
 
 using WalkFn = void (*)(WalkArgs);
@@ -1744,7 +1753,7 @@ pw_status pw_autotune(pw_graph* g, int64_t count, const int64_t* s, const int64_
   };
   Run dv, dt, dq;
   if ((st = timed(1, R_hi, &dv)) != PW_OK) return st;
-  out->visit_occupancy = 3;
+  out->visit_occupancy = g->access == WalkAccess::kRanked ? 4 : 3;
   out->sample_ms[0] = dv.d.walk_ms;
   out->visit_ns = dv.n_visits > 0 ? 1e6 * dv.d.walk_ms / dv.n_visits : 0.0;
   out->sample_mode = 1;
@@ -1782,19 +1791,24 @@ pw_status pw_autotune(pw_graph* g, int64_t count, const int64_t* s, const int64_
   out->table_available = 1;
   // table kernel: block size (beyond the team kernel, whose is 256)
   const std::vector<int> sizes = g->n <= kTeamNodes ? std::vector<int>{(int)kTeamWarps * 32} : std::vector<int>{512, 1024};
+  // the faster at R = 2048, extrapolated from 1024 and 256: the table serves the queries with many replicas
   int best_threads = sizes[0];
+  double best_2048 = 0.0;
   for (int threads : sizes) {
     g->table_threads = threads;
-    Run r;
-    if ((st = timed(2, R_hi, &r)) != PW_OK) return st;
-    if (threads == sizes[0] || r.d.walk_ms < dt.d.walk_ms) {
-      dt = r;
+    Run hi, lo;
+    if ((st = timed(2, R_hi, &hi)) != PW_OK) return st;
+    if ((st = timed(2, R_lo, &lo)) != PW_OK) return st;
+    const double at_2048 = hi.d.walk_ms + (hi.d.walk_ms - lo.d.walk_ms) / 0.75;
+    if (threads == sizes[0] || at_2048 < best_2048) {
+      dt = hi;
+      dq = lo;
+      best_2048 = at_2048;
       best_threads = threads;
     }
   }
   g->table_threads = best_threads;
   out->table_threads = best_threads;
-  if ((st = timed(2, R_lo, &dq)) != PW_OK) return st;
   out->sample_ms[1] = dt.d.walk_ms;
   out->sample_ms[2] = dq.d.walk_ms;
   // solve  T = P c + V w  for the two table runs (times in ns)
