@@ -57,16 +57,17 @@ def workload_eps(wl: dict, count: int, rank: int = 0) -> np.ndarray:
 
 SECTOR_BYTES = 32  # one 16-byte neighbour record per transition lives in one 32-byte sector
 L2_BYTES = 129 << 20
-WALK_KERNEL_NAME = {1: "walk_kernel (per-visit probe evaluation)", 2: "walk_table_kernel (per-probe table)",
-                    3: "walk_table_kernel and walk_kernel (walk kernel chosen per query)"}
-# DRAM and L2 traffic of a walk kernel from one ncu capture on a small case of
-# the same workload (null when no capture of the current kernel exists, or
-# when the batch ran both walk kernels).  BA, table kernel, one launch of 8
-# queries (5.2096e9 transitions): dram read+write 16.04 MB + 2.6 KB, the record
-# array read once into L2 whatever the transitions, so the DRAM bytes are not
-# scaled; lts__t_sectors 5.653e9, 1.085 sectors per transition, scaled.
+WALK_KERNEL_NAME = {1: "walk_kernel (per-visit probe evaluation)", 2: "walk_team_kernel or, beyond 278,528 nodes, walk_table_kernel (per-probe table)",
+                    3: "the table kernel and walk_kernel (walk kernel chosen per query)"}
+# DRAM and L2 traffic of a walk kernel from one ncu capture on a small case (null
+# when no capture of the current kernel exists, or when the batch ran both walk
+# kernels).  BA, table kernel, one launch of 8 queries on another 10^5-node
+# preferential-attachment graph of the same size (8.785e9 transitions): dram
+# read+write 16.05 MB, the record array read once into L2 whatever the
+# transitions, so the DRAM bytes are not scaled; lts__t_sectors 8.862e9, 1.009
+# sectors per transition, scaled.
 WALK_TRAFFIC = {
-    ("ba-1e5", 2): {"dram_per_launch": 16.041472e6 + 2560.0, "l2_per_transition": 5652706685 * 32 / 5.2096e9,
+    ("ba-1e5", 2): {"dram_per_launch": 16.046848e6, "l2_per_transition": 8862413619 * 32 / 8.78528e9,
                     "note": "ncu capture of one 8-query launch: DRAM reads are the 16 MB record array, loaded once "
                             "into L2 (not scaled); L2 sectors scaled by transitions"},
 }
