@@ -40,6 +40,10 @@ constexpr int kServerThreads = 256;
 constexpr uint32_t kServerGmax = 2048;  // block means of the final job live in shared memory
 constexpr size_t kServerMeansBytes = sizeof(double) * kServerGmax;
 constexpr uint32_t kJobProbes = 8;      // at most 8 probes per job
+// Graphs of up to this many nodes may have a job's tables side by side, each
+// built by one warp (a warp's whole build of 2048 nodes is 8 pools).
+constexpr uint32_t kJobTableNodes = 2048;
+constexpr uint32_t kJobTableWords = kJobTableNodes / 32 + 2;
 
 struct SlotDev {
   QPlan plan;          // main plan; R written by the pilot transition in PILOT mode
@@ -112,10 +116,21 @@ __device__ __forceinline__ QPlan load_plan(const QPlan* p) {
 // Device-ring (main stage) work is taken first.
 // Probes per job: one when the main stage reads a per-probe table (a block
 // builds one table at a time), else enough probes for about 8 tiles of 32
-// replicas, so every warp of the block has work when R is small.
-__device__ __forceinline__ uint32_t probes_per_job(const SlotDev* S, uint32_t stage) {
+// replicas, so every warp of the block has work when R is small.  On a small
+// graph a table job is short beside its claim, its build by the few threads
+// that have a word, and its sums, so it takes up to 8 probes, a warp building
+// each table, as long as the queries that wait (`pending`, this one among
+// them) leave every block two jobs: the last query's jobs are single again.
+// Bursts, single probes -> up to 8: 7 queries on 1,241 nodes at L = 13 716 ->
+// 533 us; 31 on 39 nodes at L = 43 1,378 -> 1,200 us.
+__device__ __forceinline__ uint32_t probes_per_job(const ServerArgs& A, const SlotDev* S, uint32_t stage, uint32_t K,
+                                                   unsigned long long pending) {
   const uint32_t R = stage == kStagePilot ? __ldcg(&S->R0) : __ldcg(&S->plan.R);
-  if (stage == kStageMain && __ldcg(&S->use_table)) return 1u;
+  if (stage == kStageMain && __ldcg(&S->use_table)) {
+    if (A.n > kJobTableNodes) return 1u;
+    const unsigned long long jobs = pending * K / (2u * gridDim.x);
+    return jobs < 2u ? 1u : jobs < kJobProbes ? (uint32_t)jobs : kJobProbes;
+  }
   const uint32_t chunks = (R + 31u) / 32u;
   return chunks >= 8u ? 1u : 8u / chunks;
 }
@@ -132,7 +147,7 @@ __device__ bool find_job(const ServerArgs& A, uint32_t& slot, uint32_t& stage, u
       const uint32_t sg = ld_volatile(A.ring_stage + idx);
       SlotDev* S = A.slots + sl;
       const uint32_t K = __ldcg(&S->K[sg]);
-      const uint32_t want = probes_per_job(S, sg);
+      const uint32_t want = probes_per_job(A, S, sg, K, r == 1 ? ld_volatile(A.dtail) - h : 1u);
       const uint32_t kk = atomicAdd(&S->next[sg], want);
       if (kk < K) {
         slot = sl;
@@ -170,6 +185,23 @@ __device__ __noinline__ float server_walk_visit(const GR gr, uint32_t n, uint32_
   const Probe pr = make_probe_warp(n, seed, k, probe_tag);
   if ((threadIdx.x & 31u) == 0u) pool.probe = pr;
   return walk_pair_visit<false>(gr, nullptr, walk_tag, pool, s, t, L, seed, pair, m, threadIdx.x & 31u);
+}
+
+// Where the tables of a job of several probes stand: after the warps' pools.
+constexpr uint32_t kJobTableAt = (kServerThreads / 32) * sizeof(VisitPool) / 4;
+static_assert(4 * (kJobTableAt + kJobProbes * kJobTableWords) <= kServerMeansBytes, "a job's tables fit");
+static_assert(kJobProbes <= kServerThreads / 32, "a warp per table");
+
+// The table of one probe of such a job, by one warp through its pool.
+__device__ __noinline__ void server_table(uint32_t n, uint64_t seed, uint32_t k, uint32_t probe_tag, uint32_t* tab) {
+  extern __shared__ uint32_t smem[];
+  const uint32_t lane = threadIdx.x & 31u;
+  VisitPool& pool = ((VisitPool*)smem)[threadIdx.x >> 5];
+  const Probe pr = make_probe_warp(n, seed, k, probe_tag);
+  if (lane == 0u) pool.probe = pr;
+  if (lane < 2u) tab[(n + 31u) / 32u + lane] = 0xFFFFFFFFu;
+  __syncwarp();
+  build_probe_table_team(pool, tab, n, 0u, 1u, lane);
 }
 
 // TABLE: the graph's probe table fits in shared memory, so main-stage jobs may
@@ -226,9 +258,12 @@ __global__ void __launch_bounds__(kServerThreads, MINB) server_kernel(ServerArgs
     const uint32_t R = pilot ? __ldcg(&S->R0) : P.R;
     const uint32_t walk_tag = pilot ? kTagWalkPilot : kTagWalk;
     const uint32_t probe_tag = pilot ? kTagProbePilot : kTagProbe;
-    const bool table = TABLE && !pilot && __ldcg(&S->use_table) != 0u;  // then nprobe == 1
+    const bool table = TABLE && !pilot && __ldcg(&S->use_table) != 0u;
     const uint32_t chunks = (R + 31u) / 32u;
-    if (TABLE && table) {
+    if (TABLE && table && nprobe > 1u) {
+      const uint32_t warp = threadIdx.x >> 5;
+      if (warp < nprobe) server_table(A.n, P.seed, k0 + warp, probe_tag, smem + kJobTableAt + warp * kJobTableWords);
+    } else if (TABLE && table) {
       if (threadIdx.x < 2) tab[(A.n + 31u) / 32u + threadIdx.x] = 0xFFFFFFFFu;
       __syncthreads();
       build_probe_table(make_probe(A.n, P.seed, k0, probe_tag), tab, A.n, threadIdx.x, kServerThreads);
@@ -248,7 +283,7 @@ __global__ void __launch_bounds__(kServerThreads, MINB) server_kernel(ServerArgs
       const uint64_t pair = (uint64_t)k * R + p;
       float U = 0.0f;
       if (TABLE && table) {
-        const ZTable zp = table_reader(tab, A.n);
+        const ZTable zp = table_reader(nprobe > 1u ? smem + kJobTableAt + j * kJobTableWords : tab, A.n);
         if (p < R) U = walk_pair_table<false>(gr, nullptr, walk_tag, zp, P.s, P.t, P.L, P.seed, pair);
       } else {
         const uint32_t rest = R - (p - lane), m = rest < 32u ? rest : 32u;

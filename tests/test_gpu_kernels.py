@@ -194,3 +194,26 @@ def test_pilot_forms(pw, oracle_lib, K0, R0):
             many, _ = pw.pw_query_batch(g.handle, np.full(9, 3), np.full(9, 2999), 0.4, L,
                                         np.full(9, 11, np.uint64), params)
             np.testing.assert_array_equal(many, want)
+
+
+@pytest.mark.parametrize("n", [5, 32, 33, 257, 2047, 2048, 2049])
+def test_server_small_graph_jobs(pw, n):
+    """A burst on a small graph: jobs of several tables side by side (up to 2048
+    nodes), tapering to one as the queue drains, give the batch's estimates; so
+    does a lone query, whose jobs are single."""
+    host = barabasi_albert(n, 3, 8)
+    s, t = uniform_pairs(n, 40, 91)
+    seeds = query_seeds(40, 92)
+    with pw.Graph(host.row_ptr, host.col_idx) as g:
+        want, st = pw.pw_query_batch(g.handle, s, t, 0.2, 40, seeds)
+        assert np.all(st == 0)
+        srv = pw.pw_server_create(g.handle, None, 1 << 26)
+        try:
+            tickets = [pw.pw_server_submit(srv, int(s[i]), int(t[i]), 0.2, 40, int(seeds[i])) for i in range(40)]
+            pw.pw_server_drain(srv, 60000)
+            np.testing.assert_array_equal([pw.pw_server_poll(srv, x)[1] for x in tickets], want)
+            one = pw.pw_server_submit(srv, int(s[7]), int(t[7]), 0.2, 40, int(seeds[7]))
+            pw.pw_server_drain(srv, 60000)
+            assert pw.pw_server_poll(srv, one)[1] == want[7]
+        finally:
+            pw.pw_server_destroy(srv)
