@@ -187,10 +187,15 @@ __device__ void scan_plans(const ScanArgs& S, int64_t nq) {
         }
         if (j == 2) table_probes = x;
         if (j == 7) {
-          // warps per table probe: at least team_min, and as many as make four waves
-          // of probes over the resident warps, but no more than a probe has tiles
+          // warps per table probe: at least team_min, and as many as make sixteen waves
+          // of probes over the resident warps, but no more than a probe has tiles.  A hub
+          // pair's probe has 128 tiles, and in fewer waves the last ones are waited for:
+          // 6 queries at L = 217 on 3,833 nodes 8.24 ms with four waves, 7.42 with eight or
+          // more; 15 at L = 216 on 20,587 nodes 27.5 and 27.5, 25.3 with sixteen.  Sixty-four
+          // give teams of eight to batches of short probes: 64 queries on 200 nodes
+          // 0.79 -> 0.92 ms.
           unsigned long long team = (unsigned long long)S.team_min;
-          while (team < 8 && table_probes * team < 4ull * S.warps && table_probes * team < x) team *= 2;
+          while (team < 8 && table_probes * team < 16ull * S.warps && table_probes * team < x) team *= 2;
           T->team = team;
         }
       }
