@@ -610,20 +610,29 @@ __global__ void __launch_bounds__(THREADS, THREADS == 512 ? 2 : 1) walk_table_ke
 // building 1,024 entries takes less than 20 steps of per-visit walks.
 constexpr int64_t kTeamPilotNodes = 1024;
 constexpr uint32_t kTeamWarps = 8;
+// From this many nodes per warp of a team on, two words of the table and more for
+// each lane, no pool is needed to keep the lanes busy.  A graph that no team builds
+// through pools has none, and its gathers the 36 KB more of L1 per SM: 15 queries at
+// L = 216 on 20,587 nodes 113.5 -> 112.4 ms (five seeds), 75 at L = 200 on 10^5 nodes
+// 218.1 -> 217.2 ms.
+constexpr uint32_t kTeamPoolNodes = 2048;
+__host__ __device__ constexpr uint32_t team_pool_words(uint32_t n) {
+  return n < kTeamPoolNodes * kTeamWarps ? kTeamWarps * (uint32_t)sizeof(VisitPool) / 4u : 0u;
+}
 template <bool DEBUG, WalkAccess ACCESS>
 __global__ void __launch_bounds__(kTeamWarps * 32, DEBUG ? 1 : 4) walk_team_kernel(WalkArgs A) {
   const auto gr = GraphOf<ACCESS>::get(A);
-  __shared__ VisitPool pools[kTeamWarps];
-  extern __shared__ uint32_t tabs[];  // one table per team
+  extern __shared__ uint32_t team_smem[];  // the warps' pools, where tables are built through them; a table per team
   __shared__ unsigned long long sums[kTeamWarps][kSumDigits];
   __shared__ unsigned long long claims[kTeamWarps];
   const unsigned long long total = A.totals->table_probes;
   if (total == 0ull) return;
   const uint32_t lane = threadIdx.x & 31u, size = (uint32_t)A.totals->team;
   const uint32_t team = (threadIdx.x >> 5) / size, warp = (threadIdx.x >> 5) % size;
-  VisitPool& pool = pools[threadIdx.x >> 5];
   const uint32_t n = A.n;
-  uint32_t* tab = tabs + team * table_words(n);
+  const bool pooled = n < kTeamPoolNodes * size;
+  VisitPool& pool = ((VisitPool*)team_smem)[threadIdx.x >> 5];
+  uint32_t* tab = team_smem + team_pool_words(n) + team * table_words(n);
   unsigned long long* sum_of = sums[team];
   auto sync = [&]() {  // the team's own barrier; its warps arrive whole
     __syncwarp();
@@ -643,12 +652,13 @@ __global__ void __launch_bounds__(kTeamWarps * 32, DEBUG ? 1 : 4) walk_team_kern
     const uint32_t kl = (uint32_t)(j - P.table_begin);
     const uint32_t k = P.k_begin + kl;
     const Probe pr = make_probe_warp(n, P.seed, k, A.probe_tag);
-    if (lane == 0) pool.probe = pr;
-    __syncwarp();
-    if (n >= 2048u * size)  // two words and more per lane: no pool needed to keep the lanes busy
-      build_probe_table(pr, tab, n, warp * 32u + lane, size * 32u);
-    else
+    if (pooled) {
+      if (lane == 0) pool.probe = pr;
+      __syncwarp();
       build_probe_table_team(pool, tab, n, warp, size, lane);
+    } else {
+      build_probe_table(pr, tab, n, warp * 32u + lane, size * 32u);
+    }
     sync();
     const ZTable zp = table_reader(tab, n);
     const uint32_t R = P.R, chunks = P.chunks;
@@ -924,7 +934,9 @@ static int team_min(const pw_graph* g) {
   while (team < (int)kTeamWarps && table_bytes(g) * (kTeamWarps / team) > kTeamTableBytes) team *= 2;
   return team;
 }
-static size_t team_bytes(const pw_graph* g) { return table_bytes(g) * (kTeamWarps / team_min(g)); }
+static size_t team_bytes(const pw_graph* g) {
+  return 4 * (size_t)team_pool_words((uint32_t)g->n) + table_bytes(g) * (kTeamWarps / team_min(g));
+}
 static int team_grid(pw_graph* g) { return grid_of(g, team_fn(false, g->access), kTeamWarps * 32, team_bytes(g)); }
 
 static pw_status launch_table(pw_graph* g, cudaStream_t stream, const WalkArgs& a, bool debug) {

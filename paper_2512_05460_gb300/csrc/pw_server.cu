@@ -189,7 +189,7 @@ __device__ __noinline__ float server_walk_visit(const GR gr, uint32_t n, uint32_
 
 // Where the tables of a job of several probes stand: after the warps' pools.
 constexpr uint32_t kJobTableAt = (kServerThreads / 32) * sizeof(VisitPool) / 4;
-static_assert(4 * (kJobTableAt + kJobProbes * kJobTableWords) <= kServerMeansBytes, "a job's tables fit");
+constexpr size_t kJobTableBytes = 4 * (size_t)kJobProbes * kJobTableWords;
 static_assert(kJobProbes <= kServerThreads / 32, "a warp per table");
 
 // The table of one probe of such a job, by one warp through its pool.
@@ -711,12 +711,17 @@ pw_status pw_server_create(pw_graph* g, const pw_params* params, size_t accum_by
   sv->slot_submit_ms.assign(sv->S, 0.0);
   for (uint32_t s = 0; s < sv->S; ++s) sv->free_slots.push_back(sv->S - 1 - s);
   // shared memory: the probe table (if it fits), the warps' pools and the block
-  // means of a finished query, all at the same place
+  // means of a finished query (G of them), all at the same place and no more than
+  // they need: what the blocks leave free is L1 (with room for
+  // 2,048 means, 20 queries at L = 89 on 2,535 nodes 53.8 ms over five seeds, now
+  // 52.7; 64 at L = 100 on 20,001 nodes 136.9, now 135.9)
   const size_t tbytes = sizeof(uint32_t) * (size_t)table_words((uint32_t)g->n);
   const size_t pbytes = sizeof(VisitPool) * (kServerThreads / 32);
   const bool with_table = tbytes + kServerMeansBytes <= 200 * 1024;
   sv->has_table = with_table;
-  sv->smem = kServerMeansBytes > pbytes ? kServerMeansBytes : pbytes;
+  sv->smem = pbytes + (g->n <= kJobTableNodes ? kJobTableBytes : 0);
+  const size_t mbytes = sizeof(double) * (sv->ba.G < kServerGmax ? (size_t)sv->ba.G : kServerGmax);
+  if (mbytes > sv->smem) sv->smem = mbytes;
   if (with_table && tbytes > sv->smem) sv->smem = tbytes;
   for (int v = 0; v < (with_table ? 1 : 2); ++v) {
     const ServerFn fn = server_fn(with_table, g->access, 2 + v);
