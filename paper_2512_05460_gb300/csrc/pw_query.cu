@@ -753,7 +753,9 @@ __global__ void mom_kernel(const QPlan* __restrict__ plans, const double* __rest
   __shared__ double mid[2];
   const int64_t q = blockIdx.x;
   const QPlan& P = plans[q];
-  if (P.status != PW_OK || P.K == 0) {
+  // B is 0 when s == t.  (K is 0, too, after an ADAPTIVE query's second stage
+  // without probes: its first stage's G B values stand.)
+  if (P.status != PW_OK || P.B == 0) {
     if (threadIdx.x == 0) {
       beta[q] = P.status == PW_OK ? 0.0 : __longlong_as_double(0x7ff8000000000000ll);
       status[q] = P.status;

@@ -217,3 +217,37 @@ def test_server_small_graph_jobs(pw, n):
             assert pw.pw_server_poll(srv, one)[1] == want[7]
         finally:
             pw.pw_server_destroy(srv)
+
+
+@pytest.mark.parametrize("graph_fn,eps", [(lambda: barabasi_albert(400, 5, 5), 0.3), (lambda: er_cycle(200, 8 / 199, 0), 0.8)])
+def test_adaptive_stops_after_the_first_stage(pw, oracle_lib, graph_fn, eps):
+    """ADAPTIVE queries whose stopping rule keeps the first stage's probes, and so
+    run none in the second, return the first stage's estimate: alone, in a batch
+    with queries that go on, as a replayed launch, and level by level."""
+    host = graph_fn()
+    params = pw.make_params(budget_mode=pw.PW_BUDGET_ADAPTIVE)
+    cfg = oracle.budget_cfg(mode=oracle.MODE_ADAPTIVE)
+    first = (int(np.ceil(0.5 / eps**2)) + 3) // 4
+    count = 40
+    s, t = uniform_pairs(host.n, count, 7)
+    seeds = query_seeds(count, 8)
+    t[3], s[4] = s[3], -1  # no work and an invalid query beside them
+    ok = np.arange(count) != 4
+    with pw.Graph(host.row_ptr, host.col_idx) as g:
+        for L in (0, 1, 2):
+            want, budgets, _ = oracle.query_many(host, s[ok], t[ok], eps, L, seeds[ok], cfg)
+            stops = np.flatnonzero(ok)[(budgets[:, 0] == first) & (s != t)[ok]]
+            assert 0 < stops.size < count - 2
+            for _ in range(3):  # eager, captured, replayed
+                beta, st = pw.pw_query_batch(g.handle, s, t, eps, L, seeds, params)
+                np.testing.assert_array_equal(beta[ok], want)
+                assert st[4] == pw.PW_ERR_ARG and np.all(st[ok] == 0) and np.isnan(beta[4])
+            assert beta[3] == 0.0
+            i = int(stops[0])
+            one = oracle.query(host, int(s[i]), int(t[i]), eps, L, int(seeds[i]), cfg)["beta"]
+            assert pw.pw_query(g.handle, int(s[i]), int(t[i]), eps, L, int(seeds[i]), params) == one
+        beta, stop, st = pw.pw_query_stabilized(g.handle, s[ok], t[ok], eps, 8, seeds[ok], params)
+        assert np.all(st == 0)
+        for j, i in enumerate(np.flatnonzero(ok)):
+            want, want_stop, _ = oracle.stabilized(host, int(s[i]), int(t[i]), eps, 8, int(seeds[i]), cfg)
+            assert (beta[j], stop[j]) == (want, want_stop)
