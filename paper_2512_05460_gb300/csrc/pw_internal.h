@@ -173,6 +173,18 @@ inline cudaError_t launch_with_window(const pw_graph* g, void (*fn)(K...), int g
   return cudaLaunchKernelEx(&cfg, fn, static_cast<A&&>(args)...);
 }
 
+constexpr size_t kMaxTableBytes = 200 * 1024;  // largest probe table
+
+// Lets fn be launched with smem bytes of dynamic shared memory (48 KB less its
+// static part need no leave).  The limit belongs to the function on its device,
+// not to a graph or server, so it is only ever raised, to one constant: set to
+// what one graph needs, it refused the launches of a larger one.
+inline cudaError_t allow_shared(const void* fn, size_t smem) {
+  return smem > 32 * 1024
+             ? cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxTableBytes)
+             : cudaSuccess;
+}
+
 // The walk-mode cost model of an untuned graph or server, in Feistel passes: a
 // table takes one per element of the permutation's domain 2^b, and a visit
 // that reads the table saves 1.15 (n = 10^5: 333 ns against 2.9 ps; R-MAT 2^20:

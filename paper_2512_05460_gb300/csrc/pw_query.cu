@@ -834,7 +834,6 @@ void prof_end(pw_graph* g, cudaStream_t stream, cudaEvent_t a, int kind) {
 
 // Largest graph whose probe table (1 bit per node) fits in shared memory next to the kernel's own state.
 static size_t table_bytes(const pw_graph* g) { return sizeof(uint32_t) * (size_t)table_words((uint32_t)g->n); }
-static constexpr size_t kMaxTableBytes = 200 * 1024;
 
 // Table-kernel block size beyond the team kernel: 512 threads while two tables
 // fit per SM, else 1024.  (Five 41 KB tables per SM left the gathers 20 KB of L1
@@ -877,15 +876,17 @@ static WalkFn table_fn(bool debug, WalkAccess access, int threads) {
 }
 
 // Persistent grid: SMs x resident blocks, measured once per kernel and
-// shared-memory size on this graph.
+// shared-memory size on this graph (not kept when CUDA gives no answer: the
+// launch then reports the error).
 static int grid_of(pw_graph* g, WalkFn fn, int threads, size_t smem) {
   const auto key = std::make_pair((const void*)fn, smem);
   auto it = g->grids.find(key);
   if (it != g->grids.end()) return it->second;
   int nb = 0;
-  if (smem > 48 * 1024) cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void*)fn, threads, smem);
+  cudaError_t e = allow_shared((const void*)fn, smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void*)fn, threads, smem);
   const int grid = g->sm_count * (nb > 0 ? nb : 1);
+  if (e != cudaSuccess) return grid;
   g->grids[key] = grid;
   return grid;
 }

@@ -251,3 +251,23 @@ def test_adaptive_stops_after_the_first_stage(pw, oracle_lib, graph_fn, eps):
         for j, i in enumerate(np.flatnonzero(ok)):
             want, want_stop, _ = oracle.stabilized(host, int(s[i]), int(t[i]), eps, 8, int(seeds[i]), cfg)
             assert (beta[j], stop[j]) == (want, want_stop)
+
+
+def test_tables_of_several_graphs(pw):
+    """Graphs with probe tables of over 48 KB (the last with the kernel's own shared
+    memory) and the same table kernel: using a smaller one leaves the larger one's
+    launches as they were."""
+    graphs = [cycle_graph(n) for n in (500_000, 420_000, 393_000)]  # 62.5, 52.5 and 48 KB
+    seeds = query_seeds(3, 5)
+    with pw.Graph(graphs[0].row_ptr, graphs[0].col_idx) as a, \
+            pw.Graph(graphs[1].row_ptr, graphs[1].col_idx) as b, pw.Graph(graphs[2].row_ptr, graphs[2].col_idx) as c:
+        for count in (1, 2, 3):  # a new count: launched, not replayed
+            s, t = np.array([0, 7, 250_000])[:count], np.array([9, 30, 250_003])[:count]
+            for g in (c, a, b, a, c):
+                got = []
+                for mode in (1, 2):
+                    params = pw.make_params(budget_mode=pw.PW_BUDGET_FIXED, B=2, G=3, R=40, walk_mode=mode)
+                    beta, st = pw.pw_query_batch(g.handle, s, t, 0.3, 5, seeds[:count], params)
+                    assert np.all(st == 0)
+                    got.append(beta)
+                np.testing.assert_array_equal(got[0], got[1])
