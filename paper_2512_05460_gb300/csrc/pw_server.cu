@@ -725,8 +725,7 @@ pw_status pw_server_create(pw_graph* g, const pw_params* params, size_t accum_by
   if (with_table && tbytes > sv->smem) sv->smem = tbytes;
   for (int v = 0; v < (with_table ? 1 : 2); ++v) {
     const ServerFn fn = server_fn(with_table, g->access, 2 + v);
-    if ((e = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sv->smem)) !=
-        cudaSuccess)
+    if ((e = allow_shared((const void*)fn, sv->smem)) != cudaSuccess)
       return fail(cuda_error(e, "server smem attribute"));
     int nb = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void*)fn, kServerThreads, sv->smem)) !=

@@ -271,3 +271,29 @@ def test_tables_of_several_graphs(pw):
                     assert np.all(st == 0)
                     got.append(beta)
                 np.testing.assert_array_equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("large,small", [(200_000, 20_001), (500_000, 420_000)])
+def test_servers_of_two_graphs(pw, large, small):
+    """Two live servers whose kernels are one function with different shared
+    memory (25 and 9 KB, 62.5 and 52.5 KB): the first goes on after the second's
+    creation, and after the idle time that ends its kernel."""
+    import time
+
+    graphs = [cycle_graph(large), cycle_graph(small)]
+    params = pw.make_params(budget_mode=pw.PW_BUDGET_FIXED, B=2, G=3, R=40)
+    with pw.Graph(graphs[0].row_ptr, graphs[0].col_idx) as a, pw.Graph(graphs[1].row_ptr, graphs[1].col_idx) as b:
+        servers = []
+        try:
+            for g in (a, b):
+                servers.append(pw.pw_server_create(g.handle, params, 1 << 20))
+                for g2, srv in zip((a, b), servers):
+                    for i in range(2):
+                        ticket = pw.pw_server_submit(srv, i, 1000 + i, 0.3, 9, 5 + i)
+                        pw.pw_server_drain(srv, 60000)
+                        want = pw.pw_query(g2.handle, i, 1000 + i, 0.3, 9, 5 + i, params)
+                        assert pw.pw_server_poll(srv, ticket)[1] == want
+                        time.sleep(0.05)
+        finally:
+            for srv in servers:
+                pw.pw_server_destroy(srv)
