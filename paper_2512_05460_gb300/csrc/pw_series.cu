@@ -150,7 +150,9 @@ __device__ __forceinline__ uint32_t series_ids(const int32_t* __restrict__ col, 
 }
 
 // Sum of x_u (column = lane mod C) over the entries [e0, e0 + len) of one row,
-// in CSR order; every lane of the warp calls, 32 / C rows at once.  `mine`: the
+// in CSR order, folded after every 8 entries whatever C, so that a query's bits do
+// not depend on the pass's width (a fold past a row's end changes nothing); every
+// lane of the warp calls, 32 / C rows at once.  `mine`: the
 // row's first ids (series_ids), the next C come with one coalesced load; up to 8
 // row loads are in flight.  Rows shorter than the warp's longest add the zero
 // row, which leaves a sum unchanged.  An entry costs a shuffle, an address, a
@@ -161,7 +163,8 @@ __device__ __forceinline__ float2 series_row_sum(const float2* __restrict__ x, c
   PairSum acc;
   const int32_t longest = C == 32 ? len : __reduce_max_sync(0xffffffffu, len);
   const float2* mycol = x + sub;
-  for (int32_t b = 0; b < longest; b += C) {
+  if (longest == 0) return make_float2(0.f, 0.f);
+  for (int32_t b = 0;; b += C) {
     const int32_t lim = longest - b < C ? longest - b : C;  // the same in the whole warp
     const uint32_t next = b + C < longest ? series_ids<C>(col, e0 + b + C, len - b - C, sub, n) : n;
     for (int32_t j = 0; j < lim; j += 8) {
@@ -186,7 +189,8 @@ __device__ __forceinline__ float2 series_row_sum(const float2* __restrict__ x, c
       if (C > 4 && rem > 6) two(6);
       if (rem > 8) acc.fold();
     }
-    if (b + C < longest) acc.fold();
+    if (b + C >= longest) break;
+    if (C > 4 || (b & 4)) acc.fold();
     mine = next;
   }
   return acc.value();
@@ -199,7 +203,7 @@ __device__ __forceinline__ float2 series_row_sum(const float2* __restrict__ x, c
 // against 6 (40): 258 and 277 us a step on a 1000^2 grid.  Microseconds a step,
 // with a warp per row of up to 1,024 entries and always 32 columns -> now:
 // 10^5-node power-law graph, 32 / 16 / 4 columns 168 -> 44 / 175 -> 28 / 168 ->
-// 18; R-MAT 2^20, 32 / 8 columns 1,498 -> 1,110 / 1,499 -> 318; 2000^2 grid, 32
+// 17; R-MAT 2^20, 32 / 8 columns 1,498 -> 1,110 / 1,499 -> 318; 2000^2 grid, 32
 // columns 1,540 -> 1,037.
 template <int C, int ACC>
 __global__ void __launch_bounds__(kSeriesThreads, 5) series_step_kernel(SeriesArgs A) {

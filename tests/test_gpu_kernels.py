@@ -297,3 +297,19 @@ def test_servers_of_two_graphs(pw, large, small):
         finally:
             for srv in servers:
                 pw.pw_server_destroy(srv)
+
+
+@pytest.mark.parametrize("graph_fn", [lambda: er_cycle(2000, 12 / 1999, 0), lambda: barabasi_albert(2000, 5, 3)])
+def test_series_alone_and_in_a_pass(pw, graph_fn):
+    """Ordinary rows of more than 4 entries: a query's bits are the same in passes
+    of 4, 8, 16 and 32 columns."""
+    host = graph_fn()
+    with pw.Graph(host.row_ptr, host.col_idx) as g:
+        for seed in range(4):
+            s, t = uniform_pairs(host.n, 32, 60 + seed)
+            for L in (7, 50, 200):
+                want = pw.pw_series_batch(g.handle, s, t, L)
+                for size in (1, 3, 8, 13):
+                    got = np.concatenate([pw.pw_series_batch(g.handle, s[i : i + size], t[i : i + size], L)
+                                          for i in range(0, 32, size)])
+                    np.testing.assert_array_equal(got, want)
