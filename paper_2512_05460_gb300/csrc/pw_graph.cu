@@ -173,6 +173,46 @@ static pw_status validate_csr(int64_t n, const int64_t* rp, const int32_t* col, 
   return PW_OK;
 }
 
+// RankedRecords' arrays from col_idx and the node records on the device.  They
+// stand beside those two, so a graph may fit without them: then it is walked in
+// the split layout.
+static cudaError_t upload_ranked(pw_graph* g, int blocks, int threads) {
+  int32_t* d_rank = nullptr;
+  cudaError_t e = cudaMalloc(&g->d_packed, sizeof(uint64_t) * (size_t)((g->nnz + 2) / 3));
+  if (e == cudaSuccess) e = cudaMalloc(&g->d_ranked, sizeof(int4) * (size_t)g->n);
+  if (e == cudaSuccess) e = cudaMalloc(&d_rank, sizeof(int32_t) * (size_t)g->n);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    if (g->d_packed) cudaFree(g->d_packed);
+    if (g->d_ranked) cudaFree(g->d_ranked);
+    g->d_packed = nullptr;
+    g->d_ranked = nullptr;
+    g->access = WalkAccess::kSplit;
+    return cudaSuccess;
+  }
+  // by degree, the largest first, in node order among equals
+  std::vector<int32_t> first((size_t)g->d_max + 2, 0), rank((size_t)g->n);
+  for (int32_t d : g->deg) ++first[(size_t)d];
+  int32_t at = 0;
+  for (int32_t d = g->d_max; d >= 0; --d) {
+    const int32_t c = first[(size_t)d];
+    first[(size_t)d] = at;
+    at += c;
+  }
+  for (int64_t v = 0; v < g->n; ++v) rank[(size_t)v] = first[(size_t)g->deg[(size_t)v]]++;
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(d_rank, rank.data(), sizeof(int32_t) * (size_t)g->n, cudaMemcpyHostToDevice, g->stream);
+  if (e == cudaSuccess) {
+    build_ranked_kernel<<<blocks, threads, 0, g->stream>>>(g->d_col, g->d_node, d_rank, g->n, g->nnz, g->d_packed,
+                                                           g->d_ranked);
+    count_launch();
+    e = cudaGetLastError();
+  }
+  const cudaError_t e_sync = cudaStreamSynchronize(g->stream);  // before `rank` and d_rank go
+  if (d_rank) cudaFree(d_rank);
+  return e == cudaSuccess ? e_sync : e;
+}
+
 static pw_status upload(pw_graph* g, const int64_t* rp64, const int32_t* col) {
   PW_CUDA_TRY(cudaSetDevice(g->device));
   PW_CUDA_TRY(cudaDeviceGetAttribute(&g->sm_count, cudaDevAttrMultiProcessorCount, g->device));
@@ -195,31 +235,10 @@ static pw_status upload(pw_graph* g, const int64_t* rp64, const int32_t* col) {
   const int blocks = (int)std::min<int64_t>((work + threads - 1) / threads, (int64_t)g->sm_count * 32);
   build_records_kernel<<<blocks, threads, 0, g->stream>>>(d_rp, d_col, g->n, g->nnz, g->d_rec, g->d_node);
   count_launch();
-  int32_t* d_rank = nullptr;
-  std::vector<int32_t> rank;  // by degree, the largest first, in node order among equals
-  if (g->access == WalkAccess::kRanked) {
-    std::vector<int32_t> first((size_t)g->d_max + 2, 0);
-    for (int32_t d : g->deg) ++first[(size_t)d];
-    int32_t at = 0;
-    for (int32_t d = g->d_max; d >= 0; --d) {
-      const int32_t c = first[(size_t)d];
-      first[(size_t)d] = at;
-      at += c;
-    }
-    rank.resize((size_t)g->n);
-    for (int64_t v = 0; v < g->n; ++v) rank[(size_t)v] = first[(size_t)g->deg[(size_t)v]]++;
-    PW_CUDA_TRY(cudaMalloc(&g->d_packed, sizeof(uint64_t) * (size_t)((g->nnz + 2) / 3)));
-    PW_CUDA_TRY(cudaMalloc(&g->d_ranked, sizeof(int4) * (size_t)g->n));
-    PW_CUDA_TRY(cudaMalloc(&d_rank, sizeof(int32_t) * (size_t)g->n));
-    PW_CUDA_TRY(cudaMemcpyAsync(d_rank, rank.data(), sizeof(int32_t) * (size_t)g->n, cudaMemcpyHostToDevice, g->stream));
-    build_ranked_kernel<<<blocks, threads, 0, g->stream>>>(d_col, g->d_node, d_rank, g->n, g->nnz, g->d_packed,
-                                                           g->d_ranked);
-    count_launch();
-  }
+  if (g->access == WalkAccess::kRanked) PW_CUDA_TRY(upload_ranked(g, blocks, threads));
   PW_CUDA_TRY(cudaGetLastError());
   PW_CUDA_TRY(cudaStreamSynchronize(g->stream));
   cudaFree(d_rp);
-  if (d_rank) cudaFree(d_rank);
   PW_CUDA_TRY(cudaMallocHost(&g->ws.host_totals, sizeof(Totals)));
   PW_CUDA_TRY(cudaEventCreateWithFlags(&g->ws.last_use, cudaEventDisableTiming));
   return PW_OK;

@@ -313,3 +313,40 @@ def test_series_alone_and_in_a_pass(pw, graph_fn):
                     got = np.concatenate([pw.pw_series_batch(g.handle, s[i : i + size], t[i : i + size], L)
                                           for i in range(0, 32, size)])
                     np.testing.assert_array_equal(got, want)
+
+
+def test_ranked_records_need_not_fit(pw):
+    """A graph that fits device memory, but not its ranked form beside it, loads
+    and gives the same estimates."""
+    import torch
+
+    from pw_inputs import rmat_native
+
+    host = rmat_native(18, 80, (0.57, 0.19, 0.19, 0.05), 6)
+    assert 4 * host.nnz + 16 * host.n > 64 << 20 and host.n <= 1 << 21
+    s, t = uniform_pairs(host.n, 3, 71)
+    seeds = query_seeds(3, 72)
+
+    def estimates(g):
+        beta, st = pw.pw_query_batch(g.handle, s, t, 0.3, 21, seeds)
+        assert np.all(st == 0)
+        return beta
+
+    def free():
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    for _ in range(2):  # the second load finds the kernels loaded
+        before = free()
+        with pw.Graph(host.row_ptr, host.col_idx, flags=pw.LOAD_NO_CONNECTIVITY) as g:
+            used = before - free()
+            want = estimates(g)
+    extra = 8 * host.nnz // 3 + 16 * host.n
+    fill = torch.empty(free() - (used - extra // 3), dtype=torch.uint8, device="cuda")
+    try:
+        assert free() < used
+        with pw.Graph(host.row_ptr, host.col_idx, flags=pw.LOAD_NO_CONNECTIVITY) as g:
+            np.testing.assert_array_equal(estimates(g), want)
+    finally:
+        del fill
+        torch.cuda.empty_cache()
