@@ -425,37 +425,56 @@ extern "C" pw_status pw_series_batch(pw_graph* g, int64_t count, const int64_t* 
   pw_status st = series_plan(g);
   if (st != PW_OK) return st;
   SeriesPlan& P = g->series;
-  // queries with the same L share a pass: group by L in input order
-  std::vector<int64_t> order((size_t)count);
-  for (int64_t i = 0; i < count; ++i) order[(size_t)i] = i;
-  std::stable_sort(order.begin(), order.end(), [&](int64_t a, int64_t b) { return L[a] < L[b]; });
-  struct Pass {
-    size_t begin;
-    int ncols, cols;
-  };
-  std::vector<Pass> passes;
-  int most = 0;  // columns of the widest pass
-  for (size_t pos = 0; pos < order.size();) {
-    size_t end = pos;
-    while (end < order.size() && end - pos < (size_t)kSeriesCols && L[order[end]] == L[order[pos]]) ++end;
-    const int ncols = (int)(end - pos);
-    const int cols = ncols <= 4 ? 4 : (ncols <= 8 ? 8 : (ncols <= 16 ? 16 : 32));
-    passes.push_back({pos, ncols, cols});
-    most = std::max(most, cols);
-    pos = end;
-  }
   int occ = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, series_step_kernel<32, 1>, kSeriesThreads, 0) != cudaSuccess ||
       occ < 1)
     occ = 1;
+  // blocks of a step: as many warps as the pass has rows and segments to hand out
+  auto step_blocks = [&](int cols) {
+    const int64_t groups = (int64_t)(n * (size_t)cols + 31) / 32 + ((int64_t)P.nseg * cols + 31) / 32;
+    return (groups * 32 + kSeriesThreads - 1) / kSeriesThreads;
+  };
+  const int64_t resident = (int64_t)g->sm_count * occ;
+  // queries with the same L share a pass: group by L in input order
+  std::vector<int64_t> order((size_t)count);
+  for (int64_t i = 0; i < count; ++i) order[(size_t)i] = i;
+  std::stable_sort(order.begin(), order.end(), [&](int64_t a, int64_t b) { return L[a] < L[b]; });
+  // Where the resident warps have a row each at most, a step is short beside its launch,
+  // and a group of several passes is captured once as a CUDA graph of 32 columns and
+  // replayed, its last pass, which may hold fewer, too.  Launched each -> replayed: 1,000
+  // queries at L = 200 on 200 nodes 32.5 -> 20.1 ms, 33 at L = 2000 20.5 -> 15.4, 64 at L =
+  // 200 on 2,000 nodes 3.96 -> 3.44.  The capture costs what some 32 replayed steps save
+  // (two passes on 200 nodes: 0.40 ms either way at L = 32, 0.17 -> 0.21 at L = 8); from
+  // 64 on it pays (three passes at L = 32 0.55 -> 0.53).
+  struct Pass {
+    size_t begin;
+    int ncols, cols;
+    bool replay;
+  };
+  std::vector<Pass> passes;
+  int most = 0;  // columns of the widest pass
+  for (size_t pos = 0, group_end = 0; pos < order.size();) {
+    bool replay = pos < group_end && passes.back().replay;
+    if (pos == group_end) {
+      while (group_end < order.size() && L[order[group_end]] == L[order[pos]]) ++group_end;
+      const int64_t again = (int64_t)((group_end - pos - 1) / (size_t)kSeriesCols);  // passes after the first
+      replay = again * L[order[pos]] >= 64 && step_blocks(kSeriesCols) <= resident;
+    }
+    const int ncols = (int)std::min(group_end - pos, (size_t)kSeriesCols);
+    const int cols = replay || ncols > 16 ? 32 : (ncols <= 4 ? 4 : (ncols <= 8 ? 8 : 16));
+    passes.push_back({pos, ncols, cols, replay});
+    most = std::max(most, cols);
+    pos += (size_t)ncols;
+  }
   const int reduce_grid = g->sm_count * 4;
-  // x, y, h, 1/d, partial sums, the reduction's block sums, (s, t) and results
+  // x, y, h, 1/d, partial sums, the reduction's block sums, (s, t) and results, and those of a replayed pass
   auto align = [](size_t b) { return (b + 255) & ~(size_t)255; };
   const size_t b_vec = align(sizeof(float2) * (n + 1) * (size_t)most), b_inv = align(sizeof(float2) * n);
   const size_t b_part = align(sizeof(float2) * (size_t)most * (size_t)P.nseg);
   const size_t b_sums = align(sizeof(double) * 2 * (size_t)most * (size_t)reduce_grid);
   const size_t b_st = align(sizeof(int2) * (size_t)count), b_out = align(sizeof(double) * (size_t)count);
-  const size_t bytes = 3 * b_vec + b_inv + b_part + b_sums + b_st + b_out;
+  const size_t b_pass_st = align(sizeof(int2) * kSeriesCols), b_pass_out = align(sizeof(double) * kSeriesCols);
+  const size_t bytes = 3 * b_vec + b_inv + b_part + b_sums + b_st + b_out + b_pass_st + b_pass_out;
   DeviceBuffer own;
   DeviceBuffer& buf = bytes <= kSeriesKeptBytes ? P.scratch : own;
   if ((st = ensure_buffer(buf, bytes)) != PW_OK) return st;
@@ -475,6 +494,8 @@ extern "C" pw_status pw_series_batch(pw_graph* g, int64_t count, const int64_t* 
   double* sums = (double*)take(b_sums);
   int2* d_st = (int2*)take(b_st);
   double* d_out = (double*)take(b_out);
+  int2* pass_st = (int2*)take(b_pass_st);
+  double* pass_out = (double*)take(b_pass_out);
   A.inv = inv;
   A.col = g->d_col;
   A.node = g->d_node;
@@ -490,28 +511,55 @@ extern "C" pw_status pw_series_batch(pw_graph* g, int64_t count, const int64_t* 
   cudaError_t e = cudaMemcpyAsync(d_st, h_st.data(), sizeof(int2) * (size_t)count, cudaMemcpyHostToDevice, stream);
   series_inv_degree_kernel<<<g->sm_count * occ, kSeriesThreads, 0, stream>>>(g->d_node, inv, (uint32_t)n);
   count_launch();
+  cudaGraphExec_t exec = nullptr;
+  int32_t exec_L = -1;
+  int exec_kernels = 0;
   for (const Pass& p : passes) {
     if (e != cudaSuccess) break;
     const int32_t Lc = L[order[p.begin]];
-    // as many warps as the pass has rows and segments to hand out, at most the resident ones
-    const int64_t groups = (int64_t)(n * (size_t)p.cols + 31) / 32 + ((int64_t)P.nseg * p.cols + 31) / 32;
-    const int grid = (int)std::min<int64_t>((int64_t)g->sm_count * occ,
-                                            (groups * 32 + kSeriesThreads - 1) / kSeriesThreads);
+    const int grid = (int)std::min(resident, step_blocks(p.cols));
+    const auto pass = p.cols == 4 ? series_pass<4> : (p.cols == 8 ? series_pass<8> : (p.cols == 16 ? series_pass<16> : series_pass<32>));
+    if (p.replay && exec_L != Lc) {
+      if (exec) {
+        e = cudaStreamSynchronize(stream);
+        cudaGraphExecDestroy(exec);
+        exec = nullptr;
+      }
+      cudaGraph_t graph = nullptr;
+      if (e == cudaSuccess) e = cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal);
+      if (e != cudaSuccess) break;
+      exec_kernels = pass(A, xb, yb, pass_st, kSeriesCols, Lc, grid, reduce_grid, sums, reduce_arrived, pass_out, stream);
+      const cudaError_t e_launch = cudaGetLastError();
+      e = cudaStreamEndCapture(stream, &graph);  // always ends the capture
+      if (e == cudaSuccess) e = e_launch;
+      if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
+      if (graph) cudaGraphDestroy(graph);
+      if (e != cudaSuccess) break;
+      exec_L = Lc;
+    }
     cudaEvent_t ev = nullptr;
     prof_begin(g, stream, &ev);
-    const auto pass = p.cols == 4 ? series_pass<4> : (p.cols == 8 ? series_pass<8> : (p.cols == 16 ? series_pass<16> : series_pass<32>));
-    const int kernels = pass(A, xb, yb, d_st + p.begin, p.ncols, Lc, grid, reduce_grid, sums, reduce_arrived,
-                             d_out + p.begin, stream);
-    count_launches(kernels);
+    if (p.replay) {  // the group's first pass is full, so every column has a query
+      e = cudaMemcpyAsync(pass_st, d_st + p.begin, sizeof(int2) * (size_t)p.ncols, cudaMemcpyDeviceToDevice, stream);
+      if (e == cudaSuccess) e = cudaGraphLaunch(exec, stream);
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(d_out + p.begin, pass_out, sizeof(double) * (size_t)p.ncols, cudaMemcpyDeviceToDevice, stream);
+      count_launches(exec_kernels);
+    } else {
+      count_launches(pass(A, xb, yb, d_st + p.begin, p.ncols, Lc, grid, reduce_grid, sums, reduce_arrived,
+                          d_out + p.begin, stream));
+    }
     prof_end(g, stream, ev, 3);
     if (g->prof.enabled) g->prof.series_steps += (uint64_t)Lc + 1;
-    e = cudaGetLastError();
+    const cudaError_t e_last = cudaGetLastError();
+    if (e == cudaSuccess) e = e_last;
   }
   std::vector<double> res((size_t)count);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(res.data(), d_out, sizeof(double) * (size_t)count, cudaMemcpyDeviceToHost, stream);
   const cudaError_t e_sync = cudaStreamSynchronize(stream);  // also before `own` and the host arrays go
   if (e == cudaSuccess) e = e_sync;
+  if (exec) cudaGraphExecDestroy(exec);
   free_buffer(own);
   if (e != cudaSuccess) return cuda_error(e, "series");
   for (size_t j = 0; j < order.size(); ++j) {

@@ -350,3 +350,28 @@ def test_ranked_records_need_not_fit(pw):
     finally:
         del fill
         torch.cuda.empty_cache()
+
+
+def test_series_replayed_passes(pw, oracle_lib):
+    """Groups of several passes on a small graph run as one captured pass that is
+    replayed, also for a last pass of fewer queries and for a second group: each
+    query's bits are those of a call of its own."""
+    from oracle import exact
+
+    host = er_cycle(200, 8 / 199, 0)
+    count = 150
+    s, t = uniform_pairs(host.n, count, 17)
+    t[5] = s[5]
+    L = np.tile(np.array([70, 64, 3], np.int32), count // 3)  # replayed (33 and more of each), replayed, not
+    L[3:21] = 70
+    with pw.Graph(host.row_ptr, host.col_idx) as g:
+        for _ in range(2):
+            got = pw.pw_series_batch(g.handle, s, t, L)
+            alone = [pw.pw_series_batch(g.handle, s[i : i + 1], t[i : i + 1], L[i : i + 1])[0] for i in range(count)]
+            np.testing.assert_array_equal(got, alone)
+        assert got[5] == 0.0
+        for length in (64, 70):
+            at = np.flatnonzero(L == length)
+            assert at.size > 32
+            want = exact.series_beta_many(host.row_ptr, host.col_idx, host.n, s[at], t[at], length)
+            np.testing.assert_allclose(got[at], want, rtol=1e-9, atol=0)
