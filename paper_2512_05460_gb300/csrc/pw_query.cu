@@ -91,7 +91,7 @@ struct ModeArgs {
 // Graphs of up to this many nodes (tables of 34 KB) run their table probes in the
 // team kernel.
 constexpr int64_t kTeamNodes = 278528;
-constexpr size_t kTeamTableBytes = 33 * 1024;  // tables of one block: two up to 131,072 nodes, then one of up to 34 KB
+constexpr size_t kTeamTableBytes = 33 * 1024;  // tables of one block: two up to 135,104 nodes, then one of up to 34 KB
 
 struct ScanArgs {
   QPlan* plans;

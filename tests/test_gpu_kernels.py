@@ -375,3 +375,23 @@ def test_series_replayed_passes(pw, oracle_lib):
             assert at.size > 32
             want = exact.series_beta_many(host.row_ptr, host.col_idx, host.n, s[at], t[at], length)
             np.testing.assert_allclose(got[at], want, rtol=1e-9, atol=0)
+
+
+@pytest.mark.parametrize("n", [8191, 8192, 8193, 16383, 16384, 16385, 135_104, 135_105, 278_528, 278_529])
+def test_team_limits(pw, n):
+    """Node counts on both sides of the team kernel's limits: builds through pools
+    (teams of four below 8,192 nodes, of eight below 16,384, where the pools leave
+    shared memory), two tables a block up to 135,104, and a block per probe beyond
+    278,528; probes of 3 tiles (teams of four where they fit) and of 10 (eight)."""
+    host = cycle_graph(n)
+    s, t = np.array([0, 1, n - 1]), np.array([5, n // 2, n - 4])
+    seeds = query_seeds(3, n)
+    with pw.Graph(host.row_ptr, host.col_idx) as g:
+        for R in (96, 300):
+            got = []
+            for mode in (1, 2):
+                params = pw.make_params(budget_mode=pw.PW_BUDGET_FIXED, B=2, G=11, R=R, walk_mode=mode)
+                beta, st = pw.pw_query_batch(g.handle, s, t, 0.3, 9, seeds, params)
+                assert np.all(st == 0)
+                got.append(beta)
+            np.testing.assert_array_equal(got[0], got[1])
