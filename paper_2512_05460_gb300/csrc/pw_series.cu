@@ -163,8 +163,7 @@ __device__ __forceinline__ float2 series_row_sum(const float2* __restrict__ x, c
   PairSum acc;
   const int32_t longest = C == 32 ? len : __reduce_max_sync(0xffffffffu, len);
   const float2* mycol = x + sub;
-  if (longest == 0) return make_float2(0.f, 0.f);
-  for (int32_t b = 0;; b += C) {
+  for (int32_t b = 0; b < longest; b += C) {
     const int32_t lim = longest - b < C ? longest - b : C;  // the same in the whole warp
     const uint32_t next = b + C < longest ? series_ids<C>(col, e0 + b + C, len - b - C, sub, n) : n;
     for (int32_t j = 0; j < lim; j += 8) {
@@ -189,8 +188,9 @@ __device__ __forceinline__ float2 series_row_sum(const float2* __restrict__ x, c
       if (C > 4 && rem > 6) two(6);
       if (rem > 8) acc.fold();
     }
-    if (b + C >= longest) break;
-    if (C > 4 || (b & 4)) acc.fold();
+    // leaving here is up to 2 % faster than not, but 0.6 % slower with a row per warp
+    if (C < 32 && b + C >= longest) break;
+    if (C == 32 ? b + C < longest : C > 4 || (b & 4)) acc.fold();
     mine = next;
   }
   return acc.value();
