@@ -57,8 +57,15 @@ def workload_eps(wl: dict, count: int, rank: int = 0) -> np.ndarray:
 
 SECTOR_BYTES = 32  # one 16-byte neighbour record per transition lives in one 32-byte sector
 L2_BYTES = 129 << 20
-WALK_KERNEL_NAME = {1: "walk_kernel (per-visit probe evaluation)", 2: "walk_team_kernel or, beyond 278,528 nodes, walk_table_kernel (per-probe table)",
-                    3: "the table kernel and walk_kernel (walk kernel chosen per query)"}
+TEAM_NODES = 278_528  # largest graph whose table probes run in the team kernel
+
+
+def walk_kernel_name(mode: int, n: int) -> str:
+    table = "walk_team_kernel" if n <= TEAM_NODES else "walk_table_kernel"
+    return {1: "walk_kernel (per-visit probe evaluation)", 2: f"{table} (per-probe table)",
+            3: f"{table} and walk_kernel (walk kernel chosen per query)"}[mode]
+
+
 # DRAM and L2 traffic of a walk kernel from one ncu capture on a small case (null
 # when no capture of the current kernel exists, or when the batch ran both walk
 # kernels).  BA, table kernel, one launch of 8 queries on another 10^5-node
@@ -574,6 +581,18 @@ def run_accuracy(args, wl, world, rank, local):
     g.close()
 
 
+def series_pass_bytes(n: int, nnz: int, L: int, queries: int) -> int:
+    """Bytes that one series pass requests, in rows of 8 bytes a column (4, 8, 16
+    or 32): every step writes y and reads a row record and 1/d (8 bytes each) per
+    node, and a neighbour's x row and 4-byte id per entry; every second step also
+    reads its own x row and h and writes h (the first starts h unread); the final
+    sums read h, and the last x when no step added it."""
+    row = 8 * next(c for c in (4, 8, 16, 32) if queries <= c)
+    h_steps = (L + 1) // 2
+    return (L * (n * (row + 16) + nnz * (row + 4)) + n * row * (3 * h_steps - (L > 0))
+            + n * row * ((L > 0) + (L % 2 == 0)))
+
+
 def run_series(args, wl, world, rank, local):
     """The deterministic truncated series beta^(L) (Lemma 2.3) on the GPU
     (pw_series_batch, double-float steps, 32 queries per pass): queries/s and
@@ -609,11 +628,8 @@ def run_series(args, wl, world, rank, local):
     assert np.all(np.isfinite(beta))
     dev_s = prof["series_ms"] / 1000.0
     steps = prof["series_steps"]
-    # requested bytes per sparse step: per node its x row (h += x), h read and
-    # written, y written (4 x 256 B) and its 16-B record; per neighbour entry
-    # the neighbour's x row (256 B) and its 16-B record
-    step_bytes = host.n * (4 * 256 + 16) + host.nnz * (256 + 16)
-    achieved = steps * step_bytes / dev_s / 1e9
+    pass_bytes = sum(series_pass_bytes(host.n, host.nnz, L, min(32, nq - at)) for at in range(0, nq, 32))
+    achieved = args.steps * pass_bytes / dev_s / 1e9
     hbm_peak, peak_kind = load_peaks()
     # the steps run in double-float (FP32 pairs, about 20 FP32 operations per
     # addition), so they are bound by memory, not by GB300's FP64 rate
@@ -639,8 +655,8 @@ def run_series(args, wl, world, rank, local):
             "series_steps_per_s": steps / dev_s, "wall_s": wall,
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                          "frac": achieved / hbm_peak, "peak_kind": peak_kind,
-                         "bytes_model": "per step n (4 x 256 B + 16 B) + nnz (256 B + 16 B) requested; neighbour "
-                                        "rows that hit L2 count as requested bytes",
+                         "bytes_model": "per step n (256 B + 16 B) + nnz (256 B + 4 B) requested, and 3 x 256 B per node every "
+                                        "second step; neighbour rows that hit L2 count as requested bytes",
                          "arithmetic": "double-float (hi + lo FP32 pairs, TwoSum / fused-multiply-add TwoProd); "
                                        "beta reduced in FP64"},
             "cpu_baseline": {"value": cpu_qps, "unit": "queries/s", "cores": 1, "kind": "oracle",
@@ -841,7 +857,7 @@ def run_ours(args, wl, world, rank, local):
     roofline.update({"traffic": tr and tr["dram_per_launch"],
                      "l2_traffic": tr and tr["l2_per_transition"] * transitions_per_step,
                      "traffic_note": tr and tr["note"],
-                     "kernel": WALK_KERNEL_NAME[walk_mode],
+                     "kernel": walk_kernel_name(walk_mode, host.n),
                      "algorithmic_bytes_per_launch": walk_bytes,
                      "layout": {1: "fused 16-B neighbour records", 2: "col_idx + 16-B node records"}[layout],
                      "bytes_model": ("32 B (one sector holding the 16 B neighbour record) per walk transition"
