@@ -612,9 +612,9 @@ constexpr int64_t kTeamPilotNodes = 1024;
 constexpr uint32_t kTeamWarps = 8;
 // From this many nodes per warp of a team on, two words of the table and more for
 // each lane, no pool is needed to keep the lanes busy.  A graph that no team builds
-// through pools has none, and its gathers the 36 KB more of L1 per SM: 15 queries at
-// L = 216 on 20,587 nodes 113.5 -> 112.4 ms (five seeds), 75 at L = 200 on 10^5 nodes
-// 218.1 -> 217.2 ms.
+// through pools has none, and its gathers the 36 KB more of L1 per SM: five batches of
+// 15 queries at L = 216 on 20,587 nodes 113.5 -> 112.4 ms together, of 75 at L = 200 on
+// 10^5 nodes 1,124.7 -> 1,119.7 ms.
 constexpr uint32_t kTeamPoolNodes = 2048;
 __host__ __device__ constexpr uint32_t team_pool_words(uint32_t n) {
   return n < kTeamPoolNodes * kTeamWarps ? kTeamWarps * (uint32_t)sizeof(VisitPool) / 4u : 0u;

@@ -121,6 +121,8 @@ __device__ __forceinline__ QPlan load_plan(const QPlan* p) {
 // that have a word, and its sums, so it takes up to 8 probes, a warp building
 // each table, as long as the queries that wait (`pending`, this one among
 // them) leave every block two jobs: the last query's jobs are single again.
+// The device ring tells how many wait, so this is for PILOT budgets; queries of
+// others come to their main stage through the host ring and count alone.
 // Bursts, single probes -> up to 8: 7 queries on 1,241 nodes at L = 13 716 ->
 // 533 us; 31 on 39 nodes at L = 43 1,378 -> 1,200 us.
 __device__ __forceinline__ uint32_t probes_per_job(const ServerArgs& A, const SlotDev* S, uint32_t stage, uint32_t K,
